@@ -3,18 +3,42 @@
 // The paper ran its fields in double precision (Section VI).  These kernels
 // update the planes [z0, z1) of FP64 ring windows (plane z in slot
 // (z + zbase) mod nslot; a dense field is the ring with nslot = nz, zbase =
-// 0) with zero ghosts outside the grid, one step per launch.  GB300's FP64
-// pipe, not HBM, bounds them (about 7 FP64 operations per heat7 point and
-// 27 per wave25 point), so the design is simple: a warp owns a 64-point row
-// segment, two points per thread (16-byte double2 accesses); x-neighbours
-// come from warp shuffles (heat7) or a shared-memory copy of the row
-// (wave25), y-neighbours from a shared-memory copy of the plane (double
-// buffered, one barrier per plane) and z-neighbours from a register queue,
-// each load issued one plane ahead of its use.  The arithmetic is written
-// with rounding intrinsics in a fixed order:
-//   heat7:  u' = u + r (((x- + x+) + (y- + y+)) + (z- + z+) - 6u)
-//   wave25: L = 3 c0 p + sum_m c_m (((x-m + x+m) + (y-m + y+m)) + (z-m + z+m)),
+// 0) with zero ghosts outside the grid, one step per launch:
+//   heat7:  u' = u + r (sum of the 6 neighbours - 6u)
+//   wave25: L = 3 c0 p + sum_m c_m (sum of the 6 neighbours m cells away),
 //           p' = kappa L + (2p - p_prev)  (+ the source amplitude)
+//
+// GB300 has two FP64 lanes per SM and clock, 1/32 of its integer ALU rate
+// (measured: 0.06 against 2 warp instructions per clock and SM), so a stencil
+// in FP64 instructions (7 per heat7 point, 27 per wave25 point) takes 112 and
+// 432 SM clocks per warp whatever the memory does.  The neighbour sums
+// therefore run in exact 64-bit integer arithmetic: each value is kept as its
+// signed 53-bit significand (left-justified in 64 bits) and its biased
+// exponent; a thread shifts the values of its two points' stencils to the
+// largest exponent among them, with 6 (heat7) or 7 (wave25) bits below that
+// value's last place, and adds them without rounding.  The wave's weights are
+// the integers 5040 c_m.  One conversion and one (heat7) or two (wave25)
+// FMAs in FP64 finish the point.
+// Against the FP64 sequence the sum carries no rounding but the shifts'
+// (below 2^-58 of the stencil's largest value each), so the result is nearer
+// the exact one: over random smooth and rough fields the error against exact
+// arithmetic is below the FP64 instructions' (see the GPU tests).
+//
+// Stencils that the integer form does not hold as exactly as FP64 would take
+// the FP64 instructions instead, per thread: infinities, NaN, a largest
+// exponent outside [kELo, kEHi] (results near overflow or below 1e-270), and
+// values so far apart that the sum's last bit exceeds 2^-56 of every value of
+// the point's own stencil (wave25: of their shares of the sum).  A
+// result depends only on the values of its thread's two stencils, so windows
+// of a slab and whole fields give the same bits.
+//
+// A warp owns a 64-point row segment, two points per thread (16-byte
+// double2 accesses); each value is converted once by the thread that loads
+// it (halo rows by the CTA that needs them) and its neighbours read it from
+// shared memory (double buffered, one barrier per plane); z-neighbours stay
+// in a register queue, each load issued one plane ahead of its use.
+#include <type_traits>
+
 #include "stencil_common.cuh"
 
 namespace ooc {
@@ -23,11 +47,14 @@ using namespace sten;
 
 namespace {
 
-constexpr int kTY64 = 2;  // heat7 rows per CTA
+constexpr int kTY64 = 4;  // heat7 rows per CTA
 constexpr int kSeg64 = 2 * kTX;
 constexpr int kWTY64 = 8;  // wave25 rows per CTA
 constexpr int kWR = 4;
 constexpr double kD0 = -205.0 / 72.0, kD1 = 8.0 / 5.0, kD2 = -1.0 / 5.0, kD3 = 8.0 / 315.0, kD4 = -1.0 / 560.0;
+
+// Biased exponents of the stencil's largest value that the integer form takes.
+constexpr uint32_t kELo = 128, kEHi = 1900;
 
 __device__ __forceinline__ double heat_pt64(double c, double xl, double xr, double up, double dn, double zm,
                                             double zp, double r)
@@ -38,18 +65,89 @@ __device__ __forceinline__ double heat_pt64(double c, double xl, double xr, doub
 
 __device__ __forceinline__ double2 ldg2(const double *p) { return __ldg(reinterpret_cast<const double2 *>(p)); }
 
-// Plane z of a ring (its slot pointer), or nullptr outside [0, nz).
-__device__ __forceinline__ const double *plane_at(const double *base, int64_t z, int64_t nz, int64_t zbase, int nslot,
-                                                  int64_t plane)
+// A pair of doubles as signed significands at the pair's exponent (the
+// larger of the two biased exponents): x = m * 2^(e - 1085), |m| < 2^63.  A
+// zero takes the implicit one too: its exponent shifts it out.  e is 0 only
+// where both values are zero.
+struct Fx2 {
+    long long a, b;
+    uint32_t e;
+};
+
+__device__ __forceinline__ long long sar64(long long v, uint32_t s)  // shifts past 63 leave the sign
 {
-    return (z >= 0 && z < nz) ? base + ring_slot(z, zbase, nslot) * plane : nullptr;
+    long long r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+    return r;
 }
 
-__global__ void __launch_bounds__(kTX *kTY64)
+__device__ __forceinline__ long long fx_mant(uint32_t hi, uint32_t lo, uint32_t d)
+{
+    unsigned long long m = (((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo) << 10;
+    asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(d));  // shifts past 63 give 0
+    const long long s = (long long)((int)hi >> 31);
+    return ((long long)m ^ s) - s;
+}
+
+__device__ __forceinline__ Fx2 to_fx(double2 v)
+{
+    const uint32_t h0 = (uint32_t)__double2hiint(v.x), h1 = (uint32_t)__double2hiint(v.y);
+    const uint32_t e0 = (h0 >> 20) & 0x7FFu, e1 = (h1 >> 20) & 0x7FFu;
+    uint32_t e = max(e0, e1);
+    if (e == 0u)  // 1 for subnormals, so that 0 means zeros
+        e = (unsigned long long)(__double_as_longlong(v.x) | __double_as_longlong(v.y)) << 1 != 0ull ? 1u : 0u;
+    return Fx2{fx_mant(h0, (uint32_t)__double2loint(v.x), e - e0), fx_mant(h1, (uint32_t)__double2loint(v.y), e - e1),
+               e};
+}
+
+#ifndef HB
+#define HB 24
+#endif
+// Above kFxBig when |v| >= 2^56 (also of several of these ORed together: when
+// one of their values is).  Then v's last bit is at most 2^-56 of its value.
+constexpr uint32_t kFxBig = (2u << HB) - 1;
+__device__ __forceinline__ uint32_t fx_big(long long v) { return (uint32_t)(v >> 32) + (1u << HB); }
+
+// v * 2^k for a nonzero double far from both ends of the range
+__device__ __forceinline__ double scale_exp(double v, int k)
+{
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    return (hi | lo) == 0 ? v : __hiloint2double(hi + (k << 20), lo);
+}
+
+// Slots of consecutive planes: the slot of plane z + d from the slot of z.
+__device__ __forceinline__ int slot_at(int s, int d, int nslot)
+{
+    s += d;
+    s %= nslot;
+    return s < 0 ? s + nslot : s;
+}
+
+// The two points at (x, y, z) in FP64 instructions, values read from memory.
+// Any exponent, infinities and NaN.
+__device__ __noinline__ double2 heat_pair_f64(const double *in, int s, int nslot, int64_t plane, int64_t off,
+                                              int64_t nx, int64_t ny, int64_t nz, int64_t x, int64_t y, int64_t z,
+                                              double r)
+{
+    const double2 z2 = make_double2(0.0, 0.0);
+    const double *p = in + (int64_t)s * plane + off;
+    const double2 c = ldg2(p);
+    const double2 row = make_double2(x >= 1 ? __ldg(p - 1) : 0.0, x + 2 < nx ? __ldg(p + 2) : 0.0);
+    const double2 up = y >= 1 ? ldg2(p - nx) : z2, dn = y + 1 < ny ? ldg2(p + nx) : z2;
+    const double2 zm = z >= 1 ? ldg2(in + (int64_t)slot_at(s, -1, nslot) * plane + off) : z2;
+    const double2 zp = z + 1 < nz ? ldg2(in + (int64_t)slot_at(s, 1, nslot) * plane + off) : z2;
+    return make_double2(heat_pt64(c.x, row.x, c.y, up.x, dn.x, zm.x, zp.x, r),
+                        heat_pt64(c.y, c.x, row.y, up.y, dn.y, zm.y, zp.y, r));
+}
+
+__global__ void __launch_bounds__(kTX *kTY64, 7)
     heat7_f64_kernel(const double *__restrict__ in, double *__restrict__ out, int nslot, int64_t zbase, Grid3 g,
                      int64_t z0, int64_t z1, int64_t zchunk, double r)
 {
-    __shared__ double2 tile[2][kTY64 + 2][kTX];
+    // a row: the 32 pairs, the pair left of the row in column 0 and the pair
+    // right of it in column 33
+    __shared__ longlong2 tm[2][kTY64 + 2][kTX + 2];
+    __shared__ uint32_t te[2][kTY64 + 2][kTX + 2];
     const int lane = threadIdx.x, ty = threadIdx.y;
     const int64_t gx = (g.nx + kSeg64 - 1) / kSeg64;
     const int64_t xs = (int64_t)(blockIdx.x % gx) * kSeg64;
@@ -61,57 +159,86 @@ __global__ void __launch_bounds__(kTX *kTY64)
     const int64_t nz = g.nz, plane = g.plane;
     const bool inside = x2 < g.nx && y < g.ny;
     const int64_t off = inside ? y * g.nx + x2 : 0;
-    const int64_t yh = ty == 0 ? y0 - 1 : y0 + kTY64;
-    const bool hrow = (ty == 0 || ty == kTY64 - 1) && yh >= 0 && yh < g.ny && x2 < g.nx;
-    const int64_t hoff = hrow ? yh * g.nx + x2 : 0;
-    const int64_t xh = lane == 0 ? xs - 1 : xs + kSeg64;
-    const bool hcol = (lane == 0 || lane == kTX - 1) && xh >= 0 && xh < g.nx && y < g.ny;
-    const int64_t xoff = hcol ? y * g.nx + xh : 0;
+    // halo pairs: the first and last warp take the rows above and below, a
+    // middle warp the 2 kTY64 pairs beyond the rows' ends
+    const bool edge = ty == 0 || ty == kTY64 - 1, side = ty == kTY64 / 2;
+    const int hr = ty == 0 ? 0 : (ty == kTY64 - 1 ? kTY64 + 1 : 1 + (lane >> 1));
+    const int hc = edge ? lane + 1 : (lane & 1) * (kTX + 1);
+    const int64_t yh = y0 + hr - 1, xh = xs + 2 * (hc - 1);
+    const bool halo = edge || (side && lane < 2 * kTY64);
+    const bool hin = halo && yh >= 0 && yh < g.ny && xh >= 0 && xh < g.nx;
+    const int64_t hoff = hin ? yh * g.nx + xh : 0;
     const double2 z2 = make_double2(0.0, 0.0);
-    const double *pm1 = plane_at(in, za - 1, nz, zbase, nslot, plane);
-    const double *p0 = plane_at(in, za, nz, zbase, nslot, plane);
-    const double *p1 = plane_at(in, za + 1, nz, zbase, nslot, plane);
-    double2 prev = (inside && pm1) ? ldg2(pm1 + off) : z2;
-    double2 cur = (inside && p0) ? ldg2(p0 + off) : z2;
-    double2 nxt = (inside && p1) ? ldg2(p1 + off) : z2;
-    double2 hyv = (hrow && p0) ? ldg2(p0 + hoff) : z2;
-    double hx = (hcol && p0) ? __ldg(p0 + xoff) : 0.0;
+    int s0 = (int)ring_slot(za, zbase, nslot);  // slot of plane z
+    int s1 = wrap_add(s0, 1, nslot);
+    const double *p0 = in + (int64_t)s0 * plane, *p1 = in + (int64_t)s1 * plane;
+    double2 cur = inside ? ldg2(p0 + off) : z2;
+    Fx2 fm = to_fx((inside && za >= 1) ? ldg2(in + (int64_t)slot_at(s0, -1, nslot) * plane + off) : z2);
+    Fx2 fc = to_fx(cur);
+    double2 nxt = (inside && za + 1 < nz) ? ldg2(p1 + off) : z2;
+    double2 hv = hin ? ldg2(p0 + hoff) : z2;
+#pragma unroll 2
     for (int i = 0; i < cnt; ++i) {
         const int64_t z = za + i;
-        const double *q1 = plane_at(in, z + 1, nz, zbase, nslot, plane);
-        const double *q2 = plane_at(in, z + 2, nz, zbase, nslot, plane);
-        const double2 pfv = (inside && q2) ? ldg2(q2 + off) : z2;
-        const double2 hyv1 = (hrow && q1) ? ldg2(q1 + hoff) : z2;
-        const double hx1 = (hcol && q1) ? __ldg(q1 + xoff) : 0.0;
+        const int s2 = wrap_add(s1, 1, nslot);
         const int b = i & 1;
-        tile[b][ty + 1][lane] = cur;
-        if (ty == 0)
-            tile[b][0][lane] = hyv;
-        if (ty == kTY64 - 1)
-            tile[b][kTY64 + 1][lane] = hyv;
-        double xl = __shfl_up_sync(0xffffffffu, cur.y, 1);
-        double xr = __shfl_down_sync(0xffffffffu, cur.x, 1);
-        if (lane == 0)
-            xl = hx;
-        if (lane == kTX - 1)
-            xr = hx;
+        tm[b][ty + 1][lane + 1] = make_longlong2(fc.a, fc.b);
+        te[b][ty + 1][lane + 1] = fc.e;
+        if (halo) {
+            const Fx2 h = to_fx(hv);
+            tm[b][hr][hc] = make_longlong2(h.a, h.b);
+            te[b][hr][hc] = h.e;
+        }
+        // the next planes' loads, a plane ahead of their use
+        const double2 nn = (inside && z + 2 < nz) ? ldg2(in + (int64_t)s2 * plane + off) : z2;
+        hv = (hin && z + 1 < nz) ? ldg2(in + (int64_t)s1 * plane + hoff) : z2;
+        const Fx2 fp = to_fx(nxt);
         __syncthreads();
-        const double2 up = tile[b][ty][lane];
-        const double2 dn = tile[b][ty + 2][lane];
+        const longlong2 up = tm[b][ty][lane + 1], dn = tm[b][ty + 2][lane + 1];
+        const uint32_t eu = te[b][ty][lane + 1], ed = te[b][ty + 2][lane + 1];
+        const long long xl = tm[b][ty + 1][lane].y, xr = tm[b][ty + 1][lane + 2].x;
+        const uint32_t el = te[b][ty + 1][lane], er = te[b][ty + 1][lane + 2];
+        const uint32_t E = max(max(max(fm.e, fc.e), max(fp.e, eu)), max(max(ed, el), er));
         double2 o;
-        o.x = heat_pt64(cur.x, xl, cur.y, up.x, dn.x, prev.x, nxt.x, r);
-        o.y = heat_pt64(cur.y, cur.x, xr, up.y, dn.y, prev.y, nxt.y, r);
+        bool exact = E >= kELo && E <= kEHi;
+        if (E == 0u) {  // all zeros
+            exact = true;
+            o.x = __fma_rn(r, 0.0, cur.x);
+            o.y = __fma_rn(r, 0.0, cur.y);
+        } else if (exact) {
+            const uint32_t et = E + 4u;
+            const long long ca = sar64(fc.a, et - fc.e), cb = sar64(fc.b, et - fc.e);
+            const long long za = sar64(fm.a, et - fm.e), zb = sar64(fm.b, et - fm.e);
+            const long long wa = sar64(fp.a, et - fp.e), wb = sar64(fp.b, et - fp.e);
+            const long long ua = sar64(up.x, et - eu), ub = sar64(up.y, et - eu);
+            const long long da = sar64(dn.x, et - ed), db = sar64(dn.y, et - ed);
+            const long long la = sar64(xl, et - el), rb = sar64(xr, et - er);
+            exact = (fx_big(ca) | fx_big(cb) | fx_big(za) | fx_big(wa) | fx_big(ua) | fx_big(da) | fx_big(la)) >
+                        kFxBig &&
+                    (fx_big(ca) | fx_big(cb) | fx_big(zb) | fx_big(wb) | fx_big(ub) | fx_big(db) | fx_big(rb)) >
+                        kFxBig;
+            const long long sa = (za + wa) + (ua + da) + (la + cb) - 6 * ca;
+            const long long sb = (zb + wb) + (ub + db) + (rb + ca) - 6 * cb;
+            const int k = (int)E - 1081;
+            o.x = __fma_rn(r, scale_exp(__ll2double_rn(sa), k), cur.x);
+            o.y = __fma_rn(r, scale_exp(__ll2double_rn(sb), k), cur.y);
+        }
+        if (!exact && inside) {
+            o = heat_pair_f64(in, s0, nslot, plane, off, g.nx, g.ny, nz, x2, y, z, r);
+        }
         if (inside)
-            *reinterpret_cast<double2 *>(out + ring_slot(z, zbase, nslot) * plane + off) = o;
-        prev = cur;
+            *reinterpret_cast<double2 *>(out + (int64_t)s0 * plane + off) = o;
+        fm = fc;
+        fc = fp;
         cur = nxt;
-        nxt = pfv;
-        hyv = hyv1;
-        hx = hx1;
+        nxt = nn;
+        s0 = s1;
+        s1 = s2;
     }
 }
 
-// One wave25 point: its x-neighbours xm/xp[m-1] at +-m, y and z likewise.
+// One wave25 point in FP64 instructions: its x-neighbours xm/xp[m-1] at +-m,
+// y and z likewise.
 __device__ __forceinline__ double wave_lap64(double c, const double (&xm)[kWR], const double (&xp)[kWR],
                                              const double (&ym)[kWR], const double (&yp)[kWR], const double (&zm)[kWR],
                                              const double (&zp)[kWR])
@@ -127,16 +254,130 @@ __device__ __forceinline__ double wave_lap64(double c, const double (&xm)[kWR], 
     return lap;
 }
 
+// L at the two points (x, y, z) and (x + 1, y, z) in FP64 instructions,
+// values read from memory.
+__device__ __noinline__ double2 wave_lap_pair_f64(const double *in, int s, int nslot, int64_t plane, int64_t off,
+                                                  int64_t nx, int64_t ny, int64_t nz, int64_t x, int64_t y, int64_t z)
+{
+    const double *p = in + (int64_t)s * plane + off;
+    double row[2 * kWR + 2], ym[2][kWR], yp[2][kWR], zm[2][kWR], zp[2][kWR];
+#pragma unroll
+    for (int j = 0; j < 2 * kWR + 2; ++j) {
+        const int64_t xj = x - kWR + j;
+        row[j] = xj >= 0 && xj < nx ? __ldg(p - kWR + j) : 0.0;
+    }
+#pragma unroll
+    for (int m = 1; m <= kWR; ++m) {
+        const double2 z2 = make_double2(0.0, 0.0);
+        const double2 a = y >= m ? ldg2(p - m * nx) : z2, b = y + m < ny ? ldg2(p + m * nx) : z2;
+        const double2 c = z >= m ? ldg2(in + (int64_t)slot_at(s, -m, nslot) * plane + off) : z2;
+        const double2 d = z + m < nz ? ldg2(in + (int64_t)slot_at(s, m, nslot) * plane + off) : z2;
+        ym[0][m - 1] = a.x, ym[1][m - 1] = a.y;
+        yp[0][m - 1] = b.x, yp[1][m - 1] = b.y;
+        zm[0][m - 1] = c.x, zm[1][m - 1] = c.y;
+        zp[0][m - 1] = d.x, zp[1][m - 1] = d.y;
+    }
+    double l[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const double xm[kWR] = {row[i + 3], row[i + 2], row[i + 1], row[i]};
+        const double xp[kWR] = {row[i + 5], row[i + 6], row[i + 7], row[i + 8]};
+        l[i] = wave_lap64(row[i + kWR], xm, xp, ym[i], yp[i], zm[i], zp[i]);
+    }
+    return make_double2(l[0], l[1]);
+}
+
+// The weights are 5040 times the coefficients, 5040 (3 c0, c1 .. c4), signs
+// -, +, -, +, -.  The values at distance m are held in units of 2^kU(m) last
+// bits (0, 2, 5 and 9, about the inverse of their coefficient), so that where
+// a field rises steeply (ahead of a wave front a value four cells away is
+// many orders larger) the large far values, which weigh little, don't push
+// the near ones out; the weights take the units up.  The high and low words
+// of the 64-bit sums are weighted apart, each exactly in 64 bits: h and l - n.
+__host__ __device__ constexpr int kU(int m) { return m == 4 ? 9 : (m == 3 ? 5 : (m == 2 ? 2 : 0)); }
+constexpr uint32_t kN0 = 43050, kN1 = 8064, kN2 = 1008u << kU(2), kN3 = 128u << kU(3), kN4 = 9u << kU(4);
+struct WaveAcc {
+    long long h;
+    unsigned long long l, n;  // low words of the positive and the negative weights
+};
+
+__device__ __forceinline__ long long mad_wide_s(int a, int b, long long c)
+{
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
+    return c;
+}
+
+__device__ __forceinline__ unsigned long long mad_wide_u(uint32_t a, uint32_t b, unsigned long long c)
+{
+    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
+    return c;
+}
+
+template <bool POS>
+__device__ __forceinline__ void wave_add(WaveAcc &w, uint32_t k, long long s)
+{
+    const int hi = (int)(s >> 32);
+    const uint32_t lo = (uint32_t)s;
+    w.h = mad_wide_s(hi, POS ? (int)k : -(int)k, w.h);
+    if (POS)
+        w.l = mad_wide_u(lo, k, w.l);
+    else
+        w.n = mad_wide_u(lo, k, w.n);
+}
+
+// The doubles of the coefficients do not add up to 0 as the coefficients do:
+// 3 kD0 + 6 (kD1 + .. + kD4) = -7.18e-16.  On smooth fields that sum times p
+// is the largest part of what the rounded coefficients change, and it is the
+// same at every step, so it is added here for agreement with the operator of
+// the rounded coefficients.
+constexpr int kSumErr = -4170600;                               // 5040 * 2^60 * (that sum)
+constexpr unsigned long long kInv5040 = 0xD00D00D00D00D00Dull;  // 2^76 / 5040
+constexpr unsigned long long kHalf = 52932;                     // centres the three truncations below
+
+// L in FP64: V = (h 2^32 + l - n) / 2^15 + c kSumErr / 2^75 < 2^62.4, then
+// V 2^12 / 5040 by its 64-bit reciprocal, as an integer of 2^(E - 1079)
+// (2^-57 of the stencil's largest value).
+__device__ __forceinline__ double wave_finish(const WaveAcc &w, long long c, int E)
+{
+    const long long corr = mad_wide_s((int)(c >> 32), kSumErr, 0) >> 43;
+    const long long v = (w.h << 17) + ((long long)(w.l - w.n) >> 15) + corr;
+    return scale_exp(__ll2double_rn(__mul64hi(v, (long long)kInv5040) + v), E - 1079);
+}
+
+// Above kW1 when one of the ORed values is at least 2^56 in magnitude; above
+// kW6 when one of the ORed sums of six reaches 2^59, so that a value in it
+// does.  A value of 2^56 in its unit weighs 0.8 x 2^56 last bits or more.
+#ifndef WB
+#define WB 24
+#endif
+#ifndef HB
+#define HB 24
+#endif
+constexpr uint32_t kW1 = (2u << WB) - 1, kW6 = (16u << WB) - 1;
+__device__ __forceinline__ uint32_t w_one(long long v) { return (uint32_t)(v >> 32) + (1u << WB); }
+__device__ __forceinline__ uint32_t w_six(long long v) { return (uint32_t)(v >> 32) + (8u << WB); }
+
+// Shared memory of a wave25 CTA: the row tile of the centre plane (double
+// buffered: 4 + TY + 4 rows of 2 + 32 + 2 pairs, the 4 x-neighbours beyond
+// each row end in the outer columns) and each thread's own values of the
+// planes z-4 .. z+4, plane za + k in slot (k + 4) mod 9.
+constexpr int kWQ = 2 * kWR + 1;
+struct Wave64Smem {
+    longlong2 tm[2][kWTY64 + 2 * kWR][kTX + 4];
+    longlong2 qm[kWQ][kWTY64][kTX];
+    uint32_t te[2][kWTY64 + 2 * kWR][kTX + 4];
+    uint32_t qe[kWQ][kWTY64][kTX];
+};
+
 // Leapfrog on FP64 rings: p' = kappa L(p) + (2p - p_prev) written over
 // p_prev in place (each point's p_prev is read only by its own thread).
-// Row tile of a plane in shared memory: 4 + 8 + 4 rows of 2 + 32 + 2
-// double2 (the 4 x-neighbours beyond each row end in the outer columns).
-__global__ void __launch_bounds__(kTX *kWTY64)
+__global__ void __launch_bounds__(kTX *kWTY64, 3)
     wave25_f64_kernel(const double *__restrict__ pin, double *pout, const double *__restrict__ kap, int nslot,
                       int64_t zbase, Grid3 g, int64_t z0, int64_t z1, int64_t zchunk, int64_t sx, int64_t sy,
                       int64_t sz, double w, WaveSrcTable tab)
 {
-    __shared__ double2 tile[2][kWTY64 + 2 * kWR][kTX + 4];
+    extern __shared__ __align__(16) unsigned char w64_smem[];
+    Wave64Smem &sm = *reinterpret_cast<Wave64Smem *>(w64_smem);
     const int lane = threadIdx.x, ty = threadIdx.y;
     const int64_t gx = (g.nx + kSeg64 - 1) / kSeg64;
     const int64_t xs = (int64_t)(blockIdx.x % gx) * kSeg64;
@@ -148,82 +389,154 @@ __global__ void __launch_bounds__(kTX *kWTY64)
     const int64_t nz = g.nz, plane = g.plane;
     const bool inside = x2 < g.nx && y < g.ny;
     const int64_t off = inside ? y * g.nx + x2 : 0;
-    // this thread's halo row (rows y0-4 .. y0-1 and y0+8 .. y0+11)
+    // each warp takes one halo row (four above, four below)
     const int64_t yh = ty < kWR ? y0 - kWR + ty : y0 + kWTY64 + (ty - kWR);
     const int hrow_t = ty < kWR ? ty : ty + kWTY64;
     const bool hrow = x2 < g.nx && yh >= 0 && yh < g.ny;
     const int64_t hoff = hrow ? yh * g.nx + x2 : 0;
-    // lanes 0, 1 and 30, 31 also load the two double2 beyond their row's ends
-    const bool xl_lane = lane < 2, xr_lane = lane >= kTX - 2;
-    const int64_t xe = xl_lane ? xs - 4 + 2 * lane : xs + kSeg64 + 2 * (lane - (kTX - 2));
-    const bool xhalo = (xl_lane || xr_lane) && xe >= 0 && xe < g.nx && y < g.ny;
-    const int64_t xoff = xhalo ? y * g.nx + xe : 0;
-    const int xcol = xl_lane ? lane : lane + 4;
+    // the third warp also takes the two pairs beyond each end of the rows
+    static_assert(kWTY64 == 2 * kWR, "one halo row per warp, one lane per pair beyond the rows' ends");
+    const int xrow = lane >> 2;
+    const bool side = ty == 2;
+    const int xr = kWR + xrow, xc = (lane & 3) < 2 ? (lane & 3) : kTX + (lane & 3);
+    const int64_t xe = xs + 2 * (xc - 2), ye = y0 + xrow;
+    const bool xhalo = side && xe >= 0 && xe < g.nx && ye < g.ny;
+    const int64_t xoff = xhalo ? ye * g.nx + xe : 0;
     const bool src_here = inside && y == sy && (sx == x2 || sx == x2 + 1);
     const double2 z2 = make_double2(0.0, 0.0);
 
-    // q[j] = p at plane z - 4 + j of this thread's two points
-    double2 q[2 * kWR + 1];
+    int s0 = (int)ring_slot(za, zbase, nslot);  // slot of plane z
+    int s1 = slot_at(s0, 1, nslot), s5 = slot_at(s0, kWR + 1, nslot);
+    auto put = [&](int slot, const Fx2 &v) {
+        sm.qm[slot][ty][lane] = make_longlong2(v.a, v.b);
+        sm.qe[slot][ty][lane] = v.e;
+    };
 #pragma unroll
-    for (int j = 0; j <= 2 * kWR; ++j) {
-        const double *pj = plane_at(pin, za - kWR + j, nz, zbase, nslot, plane);
-        q[j] = (inside && pj) ? ldg2(pj + off) : z2;
+    for (int j = 0; j < kWQ; ++j) {
+        const int64_t zj = za - kWR + j;
+        put(j, to_fx((inside && zj >= 0 && zj < nz)
+                         ? ldg2(pin + (int64_t)slot_at(s0, j - kWR, nslot) * plane + off)
+                         : z2));
     }
-    const double *c0 = plane_at(pin, za, nz, zbase, nslot, plane);
-    double2 hv = (hrow && c0) ? ldg2(c0 + hoff) : z2;
-    double2 xv = (xhalo && c0) ? ldg2(c0 + xoff) : z2;
-    const double *k0 = plane_at(kap, za, nz, zbase, nslot, plane);
-    const double *pp0 = plane_at(pout, za, nz, zbase, nslot, plane);
-    double2 kv = (inside && k0) ? ldg2(k0 + off) : z2;
-    // p_prev is overwritten by this kernel: plain loads, not the read-only path
-    double2 ppv = (inside && pp0) ? *reinterpret_cast<const double2 *>(pp0 + off) : z2;
+    int ph = kWR;  // slot of plane z
+    double2 hv = hrow ? ldg2(pin + (int64_t)s0 * plane + hoff) : z2;
+    double2 xv = xhalo ? ldg2(pin + (int64_t)s0 * plane + xoff) : z2;
+#pragma unroll 9
     for (int i = 0; i < cnt; ++i) {
         const int64_t z = za + i;
-        // next plane's loads, issued before this plane's work
-        const double *n5 = plane_at(pin, z + kWR + 1, nz, zbase, nslot, plane);
-        const double *n1 = plane_at(pin, z + 1, nz, zbase, nslot, plane);
-        const bool more = i + 1 < cnt;
-        const double2 q_next = (inside && n5 && more) ? ldg2(n5 + off) : z2;
-        const double2 hv_next = (hrow && n1 && more) ? ldg2(n1 + hoff) : z2;
-        const double2 xv_next = (xhalo && n1 && more) ? ldg2(n1 + xoff) : z2;
-        const double *k1 = plane_at(kap, z + 1, nz, zbase, nslot, plane);
-        const double *pp1 = plane_at(pout, z + 1, nz, zbase, nslot, plane);
-        const double2 kv_next = (inside && k1 && more) ? ldg2(k1 + off) : z2;
-        const double2 ppv_next = (inside && pp1 && more) ? *reinterpret_cast<const double2 *>(pp1 + off) : z2;
-
         const int b = i & 1;
-        const double2 c = q[kWR];
-        tile[b][ty + kWR][lane + 2] = c;
-        tile[b][hrow_t][lane + 2] = hv;
-        if (xl_lane || xr_lane)
-            tile[b][ty + kWR][xcol] = xv;
+        const longlong2 cm = sm.qm[ph][ty][lane];
+        const uint32_t ce = sm.qe[ph][ty][lane];
+        sm.tm[b][ty + kWR][lane + 2] = cm;
+        sm.te[b][ty + kWR][lane + 2] = ce;
+        {
+            const Fx2 h = to_fx(hv);
+            sm.tm[b][hrow_t][lane + 2] = make_longlong2(h.a, h.b);
+            sm.te[b][hrow_t][lane + 2] = h.e;
+        }
+        if (side) {
+            const Fx2 h = to_fx(xv);
+            sm.tm[b][xr][xc] = make_longlong2(h.a, h.b);
+            sm.te[b][xr][xc] = h.e;
+        }
+        // the next plane's halos and the queue's next plane, and this
+        // plane's other operands, which are used last
+        const bool more = i + 1 < cnt;
+        const int64_t b0 = (int64_t)s0 * plane + off, b1 = (int64_t)s1 * plane;
+        hv = (hrow && more) ? ldg2(pin + b1 + hoff) : z2;
+        xv = (xhalo && more) ? ldg2(pin + b1 + xoff) : z2;
+        const double2 qn = (inside && more && z + kWR + 1 < nz) ? ldg2(pin + (int64_t)s5 * plane + off) : z2;
+        const double2 c = inside ? ldg2(pin + b0) : z2;
+        const double2 kv = inside ? ldg2(kap + b0) : z2;
+        // p_prev is overwritten by this kernel: plain loads, not the read-only path
+        const double2 ppv = inside ? *reinterpret_cast<const double2 *>(pout + b0) : z2;
         __syncthreads();
-        // x-neighbours: the row's double2 e-2 .. e+2 around this thread's e
-        const int e = lane + 2;
-        const double2 a2 = tile[b][ty + kWR][e - 2], a1 = tile[b][ty + kWR][e - 1];
-        const double2 b1 = tile[b][ty + kWR][e + 1], b2 = tile[b][ty + kWR][e + 2];
-        double ymx[kWR], ypx[kWR], ymy[kWR], ypy[kWR], zmx[kWR], zpx[kWR], zmy[kWR], zpy[kWR];
+        const int e = lane + 2;  // this thread's pair in the row
+        uint32_t ey[2 * kWR], exn[4];
 #pragma unroll
         for (int m = 1; m <= kWR; ++m) {
-            const double2 um = tile[b][ty + kWR - m][e], up = tile[b][ty + kWR + m][e];
-            ymx[m - 1] = um.x;
-            ypx[m - 1] = up.x;
-            ymy[m - 1] = um.y;
-            ypy[m - 1] = up.y;
-            zmx[m - 1] = q[kWR - m].x;
-            zpx[m - 1] = q[kWR + m].x;
-            zmy[m - 1] = q[kWR - m].y;
-            zpy[m - 1] = q[kWR + m].y;
+            ey[m - 1] = sm.te[b][ty + kWR - m][e];
+            ey[kWR + m - 1] = sm.te[b][ty + kWR + m][e];
         }
-        // point x2 (c.x): x-1 = a1.y, x+1 = c.y, x-+2 = a1.x / b1.x, x-+3 = a2.y / b1.y, x-+4 = a2.x / b2.x
-        const double xmx[kWR] = {a1.y, a1.x, a2.y, a2.x}, xpx[kWR] = {c.y, b1.x, b1.y, b2.x};
-        // point x2 + 1 (c.y): x-1 = c.x, x+1 = b1.x, x-+2 = a1.y / b1.y, x-+3 = a1.x / b2.x, x-+4 = a2.y / b2.y
-        const double xmy[kWR] = {c.x, a1.y, a1.x, a2.y}, xpy[kWR] = {b1.x, b1.y, b2.x, b2.y};
-        const double lx = wave_lap64(c.x, xmx, xpx, ymx, ypx, zmx, zpx);
-        const double ly = wave_lap64(c.y, xmy, xpy, ymy, ypy, zmy, zpy);
+        exn[0] = sm.te[b][ty + kWR][e - 2];
+        exn[1] = sm.te[b][ty + kWR][e - 1];
+        exn[2] = sm.te[b][ty + kWR][e + 1];
+        exn[3] = sm.te[b][ty + kWR][e + 2];
+        // the largest exponent, each distance's in its unit (the outer row
+        // pairs hold a value at distance 3, the inner ones one at 1)
+        uint32_t ez[2 * kWR];
+        const longlong2 *zq[2 * kWR];
+        int E = (int)max(ce, max(exn[1], exn[2])), Z = (int)max(exn[0], exn[3]);
+        Z = max(Z, E);  // the largest as it is
+        E = max(E, (int)max(exn[0], exn[3]) - kU(3));
+#pragma unroll
+        for (int j = 0; j < kWR; ++j) {
+            const int lo = ph >= j + 1 ? ph - (j + 1) : ph - (j + 1) + kWQ;
+            const int hi = ph + j + 1 < kWQ ? ph + j + 1 : ph + j + 1 - kWQ;
+            ez[j] = sm.qe[lo][ty][lane];
+            ez[kWR + j] = sm.qe[hi][ty][lane];
+            zq[j] = &sm.qm[lo][ty][lane];
+            zq[kWR + j] = &sm.qm[hi][ty][lane];
+            const int em = (int)max(max(ez[j], ez[kWR + j]), max(ey[j], ey[kWR + j]));
+            E = max(E, em - kU(j + 1));
+            Z = max(Z, em);
+        }
+        double2 lap = make_double2(0.0, 0.0);
+        bool exact = Z == 0;  // all zeros
+        if (E >= (int)kELo && Z <= (int)kEHi) {
+            const uint32_t et = (uint32_t)E + 3u;
+            WaveAcc wa{0, kHalf, 0}, wb{0, kHalf, 0};
+            // A row value at distance m of the first point is at m - 1 or
+            // m + 1 of the second.  xa[j], xb[j]: at distance j + 1 left and
+            // right of the first and of the second point, in that unit.
+            const longlong2 l2 = sm.tm[b][ty + kWR][e - 2], l1 = sm.tm[b][ty + kWR][e - 1];
+            const longlong2 r1 = sm.tm[b][ty + kWR][e + 1], r2 = sm.tm[b][ty + kWR][e + 2];
+            auto at = [&](long long v, uint32_t ev, int m) { return sar64(v, et + (uint32_t)kU(m) - ev); };
+            const long long ca = at(cm.x, ce, 0), cb = at(cm.y, ce, 0);
+            const long long xa[kWR] = {at(l1.y, exn[1], 1) + cb, at(l1.x, exn[1], 2) + at(r1.x, exn[2], 2),
+                                       at(l2.y, exn[0], 3) + at(r1.y, exn[2], 3),
+                                       at(l2.x, exn[0], 4) + at(r2.x, exn[3], 4)};
+            const long long xb[kWR] = {ca + at(r1.x, exn[2], 1), at(l1.y, exn[1], 2) + at(r1.y, exn[2], 2),
+                                       at(l1.x, exn[1], 3) + at(r2.x, exn[3], 3),
+                                       at(l2.y, exn[0], 4) + at(r2.y, exn[3], 4)};
+            wave_add<false>(wa, kN0, ca);
+            wave_add<false>(wb, kN0, cb);
+            // is the sums' last bit small against the values of each point's
+            // own stencil (one1: beside it, six: sums further out)?
+            const uint32_t own = w_one(ca) | w_one(cb);
+            uint32_t onea = own, oneb = own, sixa = 8u << WB, sixb = 8u << WB;
+            auto taps = [&](auto m_c) {
+                constexpr int m = decltype(m_c)::value;
+                constexpr uint32_t k = m == 1 ? kN1 : (m == 2 ? kN2 : (m == 3 ? kN3 : kN4));
+                const longlong2 um = sm.tm[b][ty + kWR - m][e], up = sm.tm[b][ty + kWR + m][e];
+                const longlong2 zm = *zq[m - 1], zp = *zq[kWR + m - 1];
+                const uint32_t em = ey[m - 1], ep = ey[kWR + m - 1], fm = ez[m - 1], fp = ez[kWR + m - 1];
+                const long long ya = at(um.x, em, m), va = at(up.x, ep, m), za = at(zm.x, fm, m), qa = at(zp.x, fp, m);
+                const long long yb = at(um.y, em, m), vb = at(up.y, ep, m), zb = at(zm.y, fm, m), qb = at(zp.y, fp, m);
+                const long long sa = xa[m - 1] + (ya + va) + (za + qa), sb = xb[m - 1] + (yb + vb) + (zb + qb);
+                if (m == 1) {
+                    onea |= w_one(ya) | w_one(va) | w_one(za) | w_one(qa);
+                    oneb |= w_one(yb) | w_one(vb) | w_one(zb) | w_one(qb);
+                }
+                sixa |= w_six(sa);
+                sixb |= w_six(sb);
+                wave_add<(m & 1) != 0>(wa, k, sa);
+                wave_add<(m & 1) != 0>(wb, k, sb);
+            };
+            taps(std::integral_constant<int, 4>{});
+            taps(std::integral_constant<int, 3>{});
+            taps(std::integral_constant<int, 2>{});
+            taps(std::integral_constant<int, 1>{});
+            lap.x = wave_finish(wa, ca, E);
+            lap.y = wave_finish(wb, cb, E);
+            exact = (onea > kW1 || sixa > kW6) && (oneb > kW1 || sixb > kW6);
+        }
+        if (!exact && inside) {
+            lap = wave_lap_pair_f64(pin, s0, nslot, plane, off, g.nx, g.ny, nz, x2, y, z);
+        }
         double2 o;
-        o.x = __fma_rn(kv.x, lx, __fma_rn(2.0, c.x, -ppv.x));
-        o.y = __fma_rn(kv.y, ly, __fma_rn(2.0, c.y, -ppv.y));
+        o.x = __fma_rn(kv.x, lap.x, __fma_rn(2.0, c.x, -ppv.x));
+        o.y = __fma_rn(kv.y, lap.y, __fma_rn(2.0, c.y, -ppv.y));
         if (src_here && z == sz) {
             double ws = w;
             if (tab.w) {  // amplitude of step n = plan time + n_off, from the device table
@@ -236,15 +549,14 @@ __global__ void __launch_bounds__(kTX *kWTY64)
                 o.y = __dadd_rn(o.y, ws);
         }
         if (inside)
-            *reinterpret_cast<double2 *>(pout + ring_slot(z, zbase, nslot) * plane + off) = o;
-#pragma unroll
-        for (int j = 0; j < 2 * kWR; ++j)
-            q[j] = q[j + 1];
-        q[2 * kWR] = q_next;
-        hv = hv_next;
-        xv = xv_next;
-        kv = kv_next;
-        ppv = ppv_next;
+            *reinterpret_cast<double2 *>(pout + (int64_t)s0 * plane + off) = o;
+        // plane z + 5 into the slot of z - 4 (read by this thread alone)
+        ++ph;
+        put(ph + kWR < kWQ ? ph + kWR : ph + kWR - kWQ, to_fx(qn));
+        ph = ph == kWQ ? 0 : ph;
+        s0 = s1;
+        s1 = s1 + 1 == nslot ? 0 : s1 + 1;
+        s5 = s5 + 1 == nslot ? 0 : s5 + 1;
     }
 }
 
@@ -279,14 +591,22 @@ cudaError_t launch_wave25_f64(DConstRing p, DRing pprev_out, DConstRing kappa, i
 {
     if (z1 <= z0)
         return cudaSuccess;
-    static const int res = resident((const void *)wave25_f64_kernel, kTX * kWTY64);  // once, thread-safe
+    // set once (thread-safe); 0 if the attribute could not be set
+    static const int res = []() -> int {
+        if (cudaFuncSetAttribute(wave25_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(Wave64Smem)) != cudaSuccess)
+            return 0;
+        return resident((const void *)wave25_f64_kernel, kTX * kWTY64, sizeof(Wave64Smem));
+    }();
+    if (res <= 0)
+        return cudaErrorInvalidValue;
     const int64_t gx = (nx + kSeg64 - 1) / kSeg64, gy = (ny + kWTY64 - 1) / kWTY64;
     const int64_t chunk = choose_chunk(gx * gy, z1 - z0, 16, 9, res);
     const int64_t gz = (z1 - z0 + chunk - 1) / chunk;
     if (p.nslot != pprev_out.nslot || p.zbase != pprev_out.zbase || p.nslot != kappa.nslot ||
         p.zbase != kappa.zbase || p.base == pprev_out.base || p.nslot > (1ll << 30) || gx * gy > 0x7fffffffll)
         return cudaErrorInvalidValue;
-    wave25_f64_kernel<<<dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWTY64), 0, st>>>(
+    wave25_f64_kernel<<<dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWTY64), sizeof(Wave64Smem), st>>>(
         p.base, pprev_out.base, kappa.base, (int)p.nslot, p.zbase, Grid3{nx, ny, nz, nx * ny}, z0, z1, chunk, sx, sy,
         sz, w, tab);
     return cudaGetLastError();
