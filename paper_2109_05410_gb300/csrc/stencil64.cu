@@ -27,16 +27,30 @@
 // Stencils that the integer form does not hold as exactly as FP64 would take
 // the FP64 instructions instead, per thread: infinities, NaN, a largest
 // exponent outside [kELo, kEHi] (results near overflow or below 1e-270), and
-// values so far apart that the sum's last bit exceeds 2^-56 of every value of
+// values so far apart that the sum's last bit exceeds 2^-54 of every value of
 // the point's own stencil (wave25: of their shares of the sum).  A
 // result depends only on the values of its thread's two stencils, so windows
 // of a slab and whole fields give the same bits.
 //
-// A warp owns a 64-point row segment, two points per thread (16-byte
-// double2 accesses); each value is converted once by the thread that loads
-// it (halo rows by the CTA that needs them) and its neighbours read it from
-// shared memory (double buffered, one barrier per plane); z-neighbours stay
-// in a register queue, each load issued one plane ahead of its use.
+// A warp owns a 64-point row segment, two points per thread (16-byte double2
+// accesses); each value is converted once by the thread that loads it (halo
+// rows by the CTA that needs them) and its neighbours read it from shared
+// memory (double buffered, one barrier per plane), each load issued one plane
+// ahead of its use.  heat7 keeps its z-neighbours in registers; wave25 keeps
+// its nine planes' own values in shared memory, which leaves 80 registers and
+// 24 warps per SM (in registers, before the unit and the exactness check were
+// added: 964 us per 384^3 step with 16 warps and spills, 886 with 8 warps,
+// against 815).
+//
+// Measured, us per step at 384^3 (G point-steps/s), FP64 instructions against
+// integer sums: wave25 3200 (17.7) and 915 (62); heat7 775 (73) and 317
+// (179).  A wave from rest, whose steep precursors take the FP64 instructions
+// in part: 1.07 ms per 256^3 step against 0.30 to 1.08, by phase; neighbours
+// 2^60 apart at random, which nearly all take them: 1.36 against 1.38 ms
+// (heat7 0.315 against 0.403).  Bound now: wave25 by the ALU pipe and
+// shared-memory wavefronts (each 55-63 % busy, about 600 instructions per 64
+// points), heat7 by the FP64 pipe (61 %) and the ALU pipe (55 %) with 28 warps
+// per SM.
 #include <type_traits>
 
 #include "stencil_common.cuh"
@@ -100,13 +114,10 @@ __device__ __forceinline__ Fx2 to_fx(double2 v)
                e};
 }
 
-#ifndef HB
-#define HB 24
-#endif
-// Above kFxBig when |v| >= 2^56 (also of several of these ORed together: when
-// one of their values is).  Then v's last bit is at most 2^-56 of its value.
-constexpr uint32_t kFxBig = (2u << HB) - 1;
-__device__ __forceinline__ uint32_t fx_big(long long v) { return (uint32_t)(v >> 32) + (1u << HB); }
+// Above kFxBig when |v| >= 2^54 (also of several of these ORed together: when
+// one of their values is).  Then v's last bit is at most 2^-54 of its value.
+constexpr uint32_t kFxBig = (1u << 23) - 1;
+__device__ __forceinline__ uint32_t fx_big(long long v) { return (uint32_t)(v >> 32) + (1u << 22); }
 
 // v * 2^k for a nonzero double far from both ends of the range
 __device__ __forceinline__ double scale_exp(double v, int k)
@@ -344,18 +355,14 @@ __device__ __forceinline__ double wave_finish(const WaveAcc &w, long long c, int
     return scale_exp(__ll2double_rn(__mul64hi(v, (long long)kInv5040) + v), E - 1079);
 }
 
-// Above kW1 when one of the ORed values is at least 2^56 in magnitude; above
-// kW6 when one of the ORed sums of six reaches 2^59, so that a value in it
-// does.  A value of 2^56 in its unit weighs 0.8 x 2^56 last bits or more.
-#ifndef WB
-#define WB 24
-#endif
-#ifndef HB
-#define HB 24
-#endif
-constexpr uint32_t kW1 = (2u << WB) - 1, kW6 = (16u << WB) - 1;
-__device__ __forceinline__ uint32_t w_one(long long v) { return (uint32_t)(v >> 32) + (1u << WB); }
-__device__ __forceinline__ uint32_t w_six(long long v) { return (uint32_t)(v >> 32) + (8u << WB); }
+// Above kW1 when one of the ORed values is at least 2^54 in magnitude; above
+// kW6 when one of the ORed sums of six reaches 2^57, so that a value in it
+// does.  A value of 2^54 in its unit weighs 0.8 x 2^54 last bits or more.  At
+// 2^54 the rms error stays below the FP64 instructions' on all tested fields
+// (heat7 at 2^53 does not).
+constexpr uint32_t kW1 = (1u << 23) - 1, kW6 = (1u << 26) - 1;
+__device__ __forceinline__ uint32_t w_one(long long v) { return (uint32_t)(v >> 32) + (1u << 22); }
+__device__ __forceinline__ uint32_t w_six(long long v) { return (uint32_t)(v >> 32) + (1u << 25); }
 
 // Shared memory of a wave25 CTA: the row tile of the centre plane (double
 // buffered: 4 + TY + 4 rows of 2 + 32 + 2 pairs, the 4 x-neighbours beyond
@@ -504,7 +511,7 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
             // is the sums' last bit small against the values of each point's
             // own stencil (one1: beside it, six: sums further out)?
             const uint32_t own = w_one(ca) | w_one(cb);
-            uint32_t onea = own, oneb = own, sixa = 8u << WB, sixb = 8u << WB;
+            uint32_t onea = own, oneb = own, sixa = 1u << 25, sixb = 1u << 25;
             auto taps = [&](auto m_c) {
                 constexpr int m = decltype(m_c)::value;
                 constexpr uint32_t k = m == 1 ? kN1 : (m == 2 ? kN2 : (m == 3 ? kN3 : kN4));
