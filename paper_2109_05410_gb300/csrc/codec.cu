@@ -13,19 +13,30 @@
 // GPU design: one thread per 4^3 block.  The 64 values stay in registers
 // (16 coalesced 128-bit loads: neighbouring threads own neighbouring blocks
 // along x).  The bit-plane stage turns the 64 negabinary words into 32
-// 64-bit plane masks with two in-register 32x32 bit transposes; the encoder
-// then writes each plane with at most three 64-bit ORs (its significance
-// part from a 256-entry table of "doubled ones", whatever its number of new
-// coefficients), and the decoder parses all group-test segments inside a
-// 32-bit stream window from one register.  The encoder
-// stages its CTA's compressed words in shared memory and writes them with
-// coalesced 32-bit stores; the decoder reads each block's words straight
-// from the stream through L1, one word ahead of their use.
+// 64-bit plane masks with two in-register 32x32 bit transposes; a plane is
+// then coded (code_plane) or parsed (parse_plane) as a whole, its new ones
+// together, so that the lanes of a warp, whose blocks have them in different
+// planes and numbers, run the same instructions.  The compressed words of a
+// warp's blocks are staged in shared memory and move to and from the stream
+// with coalesced 16-byte accesses; the plane masks pass through shared memory
+// 16 planes at a time.
+//
+// The kernels are bound by the integer ALU pipe (78-80 % busy, against 23-27 %
+// of DRAM), which issues half of what the schedulers do.  56 planes of 1024^2,
+// R = 8, 16, 24, us: encode 196, 224, 241 -> 138, 150, 165; decode 196, 236,
+// 261 -> 142, 166, 179, against a plane loop that wrote its fields by
+// read-modify-write and parsed the new ones segment by segment (22 of 32
+// lanes active).  The transform and the transposes alone take 92 and 80 us.
+// What did not pay for the decoder: the plane loop unrolled with the masks in
+// registers (no shared memory for them, but its code overflows the
+// instruction cache: 230 us; with a plane as a called function 208), all 32
+// masks of a block in shared memory at once (16 warps per SM instead of 24:
+// 216).
 //
 // Also here: dense-field kernels for any shape (partial blocks padded with
 // the nearest inside value) and the variable-size fixed-precision and
-// fixed-accuracy modes, with a prefix sum that turns block sizes into
-// offsets.
+// fixed-accuracy modes, which find their blocks' offsets by a decoupled
+// look-back.
 #include <utility>
 
 #include "common.cuh"
@@ -40,7 +51,7 @@ namespace {
 
 constexpr int kPrec = 26;  // block-floating-point precision (bits)
 constexpr int kThreads = 128;
-constexpr int kPlaneStride = 65;  // words per thread for its plane masks
+constexpr int kHalfStride = 33;   // words per thread for 16 planes' masks (odd: different banks)
 constexpr int kSlack = 8;         // words past a block's 2R that a coder may touch
 
 // ---- sequency order ---------------------------------------------------------
@@ -63,20 +74,22 @@ __host__ __device__ constexpr int order_at(int r)
     return -1;
 }
 
+// Negabinary of q is (q + kNB) ^ kNB; the XOR happens in the plane masks
+// (to_planes32, from_planes32).
 constexpr uint32_t kNB = 0xAAAAAAAAu;
 
 template <int... R>
 __device__ __forceinline__ void to_coding_order(uint32_t (&u)[64], const int32_t (&q)[64],
                                                 std::integer_sequence<int, R...>)
 {
-    ((u[R] = ((uint32_t)q[std::integral_constant<int, order_at(R)>::value] + kNB) ^ kNB), ...);
+    ((u[R] = (uint32_t)q[std::integral_constant<int, order_at(R)>::value] + kNB), ...);
 }
 
 template <int... R>
 __device__ __forceinline__ void from_coding_order(int32_t (&q)[64], const uint32_t (&u)[64],
                                                   std::integer_sequence<int, R...>)
 {
-    ((q[std::integral_constant<int, order_at(R)>::value] = (int32_t)((u[R] ^ kNB) - kNB)), ...);
+    ((q[std::integral_constant<int, order_at(R)>::value] = (int32_t)(u[R] - kNB)), ...);
 }
 
 // ---- wrapping int32 lifting ---------------------------------------------------
@@ -167,21 +180,28 @@ __device__ __forceinline__ void transform_inv(int32_t (&c)[64])
 }
 
 // ---- 32x32 bit transpose of a[OFF .. OFF+31] in registers --------------------
-// Afterwards bit i of a[OFF + p] is the former bit p of a[OFF + i].
-template <int OFF, int J, uint32_t M>
+// Afterwards bit i of a[OFF + p] is the former bit p of a[OFF + i].  Each
+// stage swaps one bit of the row index with that bit of the column index, so
+// the stages commute.  The 16- and 8-bit stages are pure byte moves (one byte
+// permute per word), the others a shift and a bit select per word.  With NIN
+// (NOUT) the rows of odd index are complemented on the way in (out): the
+// negabinary offset's XOR with 0xAAAAAAAA, in the plane masks, for free.
+template <int OFF, int J, uint32_t M, bool NIN, bool NOUT>
 __device__ __forceinline__ void transpose_stage(uint32_t (&a)[64])
 {
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
         if (!(k & J)) {
-            const uint32_t t = ((a[OFF + k] >> J) ^ a[OFF + k + J]) & M;
-            a[OFF + k + J] ^= t;
-            a[OFF + k] ^= t << J;
+            const uint32_t x = a[OFF + k], y = a[OFF + k + J];
+            static_assert(J == 1 || (!NIN && !NOUT), "odd rows are one operand of the stage J = 1");
+            const uint32_t hi = y << J;
+            a[OFF + k] = NIN ? (x & M) | (~hi & ~M) : (x & M) | (hi & ~M);
+            const uint32_t lo = x >> J;
+            a[OFF + k + J] = NIN ? (lo & M) | (~y & ~M) : (NOUT ? ~((lo & M) | (y & ~M)) : (lo & M) | (y & ~M));
         }
     }
 }
 
-// The 16- and 8-bit stages are pure byte moves: one byte permute per word.
 template <int OFF>
 __device__ __forceinline__ void transpose_stage16(uint32_t (&a)[64])
 {
@@ -206,14 +226,25 @@ __device__ __forceinline__ void transpose_stage8(uint32_t (&a)[64])
     }
 }
 
+// Coefficients (plus kNB) to plane masks, and back.
 template <int OFF>
-__device__ __forceinline__ void transpose32(uint32_t (&a)[64])
+__device__ __forceinline__ void to_planes32(uint32_t (&a)[64])
 {
     transpose_stage16<OFF>(a);
     transpose_stage8<OFF>(a);
-    transpose_stage<OFF, 4, 0x0F0F0F0Fu>(a);
-    transpose_stage<OFF, 2, 0x33333333u>(a);
-    transpose_stage<OFF, 1, 0x55555555u>(a);
+    transpose_stage<OFF, 4, 0x0F0F0F0Fu, false, false>(a);
+    transpose_stage<OFF, 2, 0x33333333u, false, false>(a);
+    transpose_stage<OFF, 1, 0x55555555u, false, true>(a);
+}
+
+template <int OFF>
+__device__ __forceinline__ void from_planes32(uint32_t (&a)[64])
+{
+    transpose_stage<OFF, 1, 0x55555555u, true, false>(a);
+    transpose_stage<OFF, 2, 0x33333333u, false, false>(a);
+    transpose_stage<OFF, 4, 0x0F0F0F0Fu, false, false>(a);
+    transpose_stage8<OFF>(a);
+    transpose_stage16<OFF>(a);
 }
 
 // ---- bit writer / reader over a thread's shared-memory words ------------------
@@ -222,92 +253,57 @@ __device__ __forceinline__ uint32_t low_mask(int l)  // l in [0, 32]
     return (uint32_t)((1ull << l) - 1ull);
 }
 
-// Reads bit fields of a thread's words through a 64-bit buffer holding at
-// least 32 unread bits; it loads one shared-memory word per 32 bits read.
-// The words past the block's 2R are zero (slack), so bits past the budget
-// read as 0, which is what a truncated stream means; only the implied-one
-// rule needs the budget.
-// Reads a block's words straight from the stream (through the L1 cache);
-// words past the block's nwords read as 0, so bits past the budget are 0.
-struct BitReader {
-    const uint32_t *src;
-    uint64_t buf;  // unread bits, least significant first
-    int avail;     // valid bits in buf, >= 32
-    int wnext;     // index of the word held in `pre`
-    int pos;       // bits consumed
-    int nwords;    // words of the block
-    uint32_t pre;  // word wnext, loaded one refill ahead so its latency hides
+// A block's stream words in shared memory, followed by kZeroWords zero words:
+// bits past the budget read as 0, which is what a truncated stream means;
+// only the implied-one rule needs the budget.
+constexpr int kZeroWords = 4;
 
-    __device__ __forceinline__ uint32_t word(int i) const { return i < nwords ? __ldg(src + i) : 0u; }
-    __device__ __forceinline__ void init(const uint32_t *s, int start, int n)
-    {
-        src = s;
-        nwords = n;
-        const int w = start >> 5, sh = start & 31;
-        buf = ((uint64_t)word(w) | ((uint64_t)word(w + 1) << 32)) >> sh;
-        avail = 64 - sh;
-        wnext = w + 2;
-        pos = start;
-        pre = word(wnext);
-    }
-    __device__ __forceinline__ void skip(int len)  // len in [0, 32]
-    {
-        buf >>= len;
-        avail -= len;
-        pos += len;
-        if (avail < 32) {
-            buf |= (uint64_t)pre << avail;
-            avail += 32;
-            pre = word(++wnext);
-        }
-    }
-    __device__ __forceinline__ uint32_t peek32() const { return (uint32_t)buf; }
-    __device__ __forceinline__ uint32_t get(int len)  // len in [0, 32]
-    {
-        const uint32_t v = (uint32_t)buf & low_mask(len);
-        skip(len);
-        return v;
-    }
-};
-
-// OR a 64-bit field into a thread's zeroed words at bit offset `off`
-// (least significant bit first); touches words off/32 .. off/32 + 2.
-__device__ __forceinline__ void or_bits(uint32_t *w, int off, uint64_t v)
+__device__ __forceinline__ uint64_t shl64(uint64_t v, int n)  // n >= 0; 0 for n >= 64
 {
-    const int i = off >> 5, sh = off & 31;
-    const uint32_t a = (uint32_t)v, b = (uint32_t)(v >> 32);
-    w[i] |= a << sh;
-    w[i + 1] |= __funnelshift_l(a, b, sh);
-    w[i + 2] |= __funnelshift_l(b, 0u, sh);
+    uint64_t r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
 }
 
-// Significance parts are written with "doubled ones": the bits of x with
-// every one followed by an extra one.  In a plane's significance part each
-// new one is followed by the group bit 1 of the next segment, so the part
-// after its first group bit is the doubled bits before the last new one,
-// then that one.  dtab[b] holds the doubled bits of byte b (8 + popc(b) <= 16
-// bits); a CTA fills it once.
-__device__ __forceinline__ void init_dup_table(uint16_t *dtab)
+// The 32 bits from bit position pos on (0 past the block's nwords words).
+__device__ __forceinline__ uint32_t bits_at(const uint32_t *w, int nwords, int pos)
 {
-    for (int b = threadIdx.x; b < 256; b += blockDim.x) {
-        uint32_t d = 0u;
-        int k = 0;
-        for (int i = 0; i < 8; ++i)
-            if ((b >> i) & 1) {
-                d |= 3u << (i + k);
-                ++k;
-            }
-        dtab[b] = (uint16_t)d;
-    }
+    const int i = min(pos >> 5, nwords);
+    return __funnelshift_r(w[i], w[i + 1], pos);
 }
 
-// Doubled ones of a 32-bit word: 32 + popc(x) <= 64 bits.
-__device__ __forceinline__ uint64_t dup_ones(uint32_t x, const uint16_t *dtab)
+// Bit fields appended to a thread's words in shared memory: the word that
+// holds bit `off` keeps its bits below off, and the words behind it are
+// written, not read, so the buffer needs no zeros beforehand.  A field's bits
+// past its length are zero, so that what is written past the new end is too.
+__device__ __forceinline__ void put64(uint32_t *w, int off, uint32_t lo, uint32_t hi)
 {
-    const uint32_t b0 = x & 0xFFu, b2 = (x >> 16) & 0xFFu;
-    const uint32_t lo = (uint32_t)dtab[b0] | ((uint32_t)dtab[(x >> 8) & 0xFFu] << (8 + __popc(b0)));
-    const uint32_t hi = (uint32_t)dtab[b2] | ((uint32_t)dtab[x >> 24] << (8 + __popc(b2)));
-    return (uint64_t)lo | ((uint64_t)hi << (16 + __popc(x & 0xFFFFu)));
+    uint32_t *p = w + (off >> 5);
+    const uint32_t k = p[0];
+    p[0] = k | __funnelshift_l(0u, lo, off);
+    p[1] = __funnelshift_l(lo, hi, off);
+    p[2] = __funnelshift_l(hi, 0u, off);
+}
+
+__device__ __forceinline__ void put32(uint32_t *w, int off, uint32_t v)
+{
+    uint32_t *p = w + (off >> 5);
+    const uint32_t k = p[0];
+    p[0] = k | __funnelshift_l(0u, v, off);
+    p[1] = __funnelshift_l(v, 0u, off);
+}
+
+// A plane's new ones are written as its bits with every one followed by the
+// group bit 1 of the next segment: inserts a one behind each one of `at`
+// (a subset of v's, lowest first; the result fits 32 bits).
+__device__ __forceinline__ uint32_t insert_ones(uint32_t v, uint32_t at)
+{
+    do {  // with `at` 0 a pass changes nothing
+        const uint32_t a1 = at - 1u, upto = at ^ a1;
+        v = (v & upto) | ((v << 1) & ~upto);
+        at = (at & a1) << 1;
+    } while (at != 0u);
+    return v;
 }
 
 // ---- one block ----------------------------------------------------------------
@@ -326,89 +322,95 @@ __device__ __forceinline__ int plane_floor(int mode, int mparam, int emax)
     return 0;
 }
 
-// The bit-plane coder shared by FR4 (NP = 32 planes) and FR4D (NP = 64):
-// pm[p] and pm[NP + p] hold bit p of coefficients 0..31 and 32..63; the
-// planes NP-1 .. pmin are written from bit `off` of the zeroed words dst
-// until the budget is spent.  Returns the coded length in bits.
+// The bit-plane coder shared by FR4 and FR4D.
 //
-// Plane p (NP-1 .. 0) is written as: the refinement bits of the n
-// significant coefficients; then, for each new one at offset t past n,
-// a group bit 1, the zeros before it and the one itself; then a closing
-// group bit 0 if coefficients remain.  When a new one is the last
-// coefficient its one is implied and not written.
+// Plane p is written as: the refinement bits of the n significant
+// coefficients; then, for each new one at offset t past n, a group bit 1, the
+// zeros before it and the one itself; then a closing group bit 0 if
+// coefficients remain.  When a new one is the last coefficient its one is
+// implied and not written.
 //
-// With rest = the plane's bits past n and tl its highest one, the part
-// after the refinement bits is the group bit 1, the doubled bits of rest
-// below tl, and the one at tl: the one of segment j lands at t_j + j past
-// the first group bit, and the next segment's group bit right after it.
-// Each plane is written with at most three 64-bit ORs, whatever its
-// number of new ones.
-template <int NP>
-__device__ __forceinline__ int code_planes(const uint32_t *pm, uint32_t *dst, int off, int budget, int pmin,
-                                           const uint16_t *dtab)
+// With rest = the plane's bits past n and tl its highest one, the part after
+// the refinement bits is the group bit 1, the bits of rest below tl with
+// every one doubled (the one itself and the next segment's group bit 1), and
+// the one at tl.  n after the plane is the larger of n and the plane's bit
+// length.
+struct CodePos {
+    int n, off;
+};
+
+// New ones that take more than 32 bits: 16 bits of rest at a time.
+__device__ __noinline__ CodePos code_long(uint32_t *dst, uint64_t rest, int n, int off)
 {
-    int n = 0;
-#pragma unroll 1
-    for (int p = NP - 1; p >= pmin && off < budget; --p) {
-        const uint64_t X = ((uint64_t)pm[NP + p] << 32) | pm[p];
-        if (n >= 64) {
-            or_bits(dst, off, X);
-            off += 64;
-            continue;
-        }
-        const uint64_t refine = X & ((1ull << n) - 1ull);
-        const uint64_t rest = X >> n;
-        if (rest == 0ull) {
-            if (n > 0)
-                or_bits(dst, off, refine);
-            off += n + 1;  // refinement bits and the closing group bit 0
-            continue;
-        }
-        or_bits(dst, off, refine | (1ull << n));  // ... and the first group bit
-        const int m = __popcll((long long)rest);
-        const int tl = 63 - __clzll((long long)rest);  // offset of the last new one
-        const int n_new = n + tl + 1;
-        const int at = off + n + 1;  // first bit past the first group bit
-        const uint64_t before = rest ^ (1ull << tl);
-        const uint64_t last = n_new == 64 ? 0ull : 1ull;  // the last coefficient's one is implied
-        const int rel = tl + m - 1;                        // the last one's position past `at`
-        if (tl < 32) {
-            or_bits(dst, at, dup_ones((uint32_t)before, dtab) | (last << rel));
-        } else {
-            const uint32_t lo = (uint32_t)before;
-            const int hs = 32 + __popc(lo);
-            or_bits(dst, at, dup_ones(lo, dtab));
-            or_bits(dst, at + hs, dup_ones((uint32_t)(before >> 32), dtab) | (last << (rel - hs)));
-        }
-        // n refinement bits, m group bits 1, tl + 1 scanned bits (the last
-        // one implied when it is coefficient 63), a closing 0 if n_new < 64
-        off += n + m + tl + 1 - (n_new == 64 ? 1 : 0) + (n_new < 64 ? 1 : 0);
-        n = n_new;
+    const int tl = 63 - __clzll((long long)rest), n_new = n + tl + 1;
+    put32(dst, off, 1u);
+    ++off;
+    uint64_t before = rest ^ (1ull << tl);
+    for (int i = 0; i < tl; i += 16) {
+        const int c = tl - i < 16 ? tl - i : 16;
+        const uint32_t v = (uint32_t)before & 0xFFFFu;
+        put32(dst, off, insert_ones(v, v));
+        off += c + __popc(v);
+        before >>= 16;
     }
-    return off;
+    if (n_new < 64) {
+        put32(dst, off, 1u);
+        off += 2;
+    }
+    return CodePos{n_new, off};
+}
+
+// One plane (bits xl of coefficients 0..31, xh of 32..63) from bit `off` on.
+__device__ __forceinline__ CodePos code_plane(uint32_t *dst, uint32_t xl, uint32_t xh, int n, int off)
+{
+    const uint64_t keep = shl64(~0ull, n);
+    put64(dst, off, xl & ~(uint32_t)keep, xh & ~(uint32_t)(keep >> 32));
+    off += n;
+    const int len = xh != 0u ? 64 - __clz((int)xh) : 32 - __clz((int)xl);
+    if (n >= 64)
+        return CodePos{n, off};
+    if (len <= n) {  // the closing group bit; the word of `off` is written already
+        return CodePos{n, off + 1};
+    }
+    const uint32_t s = (uint32_t)((((uint64_t)xh << 32) | xl) >> n);
+    const int tl = len - n - 1, bits = tl + __popc(s);  // bits: up to and with the last one
+    if (tl > 31 || bits > 30)
+        return code_long(dst, (((uint64_t)xh << 32) | xl) >> n, n, off);
+    const uint32_t last = 1u << tl;
+    uint32_t v = insert_ones(s, s ^ last);
+    const bool open = len < 64;
+    if (!open)  // the last coefficient's one is implied
+        v ^= 1u << (bits - 1);
+    put32(dst, off, 1u | (v << 1));
+    return CodePos{len, off + bits + (open ? 2 : 0)};
+}
+
+// The words behind the coded bits up to the block's `words`.
+__device__ __forceinline__ void clear_tail(uint32_t *dst, int off, int words)
+{
+    for (int i = (off >> 5) + 1; i < words; ++i)
+        dst[i] = 0u;
 }
 
 // Encode one block into dst[0 .. words) (a bit budget of 32 words; words =
 // 2R at a fixed rate) with the plane range of `mode`.  Returns the coded
 // length in bits (exact for the variable-size modes, whose budget never
-// binds).
+// binds).  The planes go through the thread's 32 words at pm, 16 at a time:
+// half the shared memory of all 32 planes, for 24 warps per SM instead of 16.
 __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mode, int mparam, uint32_t *dst,
-                                            uint32_t *pm, const uint16_t *dtab)
+                                            uint32_t *pm)
 {
     uint32_t mx = 0;
 #pragma unroll
     for (int i = 0; i < 64; ++i)
         mx = max(mx, v[i] & 0x7FFFFFFFu);
     const int budget = 32 * words;
-    // The coder ORs bit fields into a zeroed buffer of `words` words plus
-    // slack; bits it writes past the budget land in the slack and are not
-    // kept.
-    for (int i = 0; i < words + kSlack; ++i)
-        dst[i] = 0u;
-    if (mx == 0u)
+    if (mx == 0u) {
+        dst[0] = 0u;
+        clear_tail(dst, 0, words);
         return 1;
+    }
     const int emax = (int)(mx >> 23) - 126;  // largest frexp exponent, >= -126
-    dst[0] = 1u | ((uint32_t)((emax + 127) & 0xFF) << 1);
     const int pmin = plane_floor(mode, mparam, emax);
 
     // q = trunc(x * 2^(26 - emax)), with the power of two split in two
@@ -425,126 +427,150 @@ __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mo
 
     transform_fwd(q);
     to_coding_order(v, q, std::make_integer_sequence<int, 64>{});
-    transpose32<0>(v);   // v[p]      = bits p of coefficients 0..31
-    transpose32<32>(v);  // v[32 + p] = bits p of coefficients 32..63
-    // The plane coder stays a compact loop (no unrolling) and reads the
-    // plane masks from this thread's shared-memory slot.
+    // the leading planes without a one, a group bit 0 each
+    uint32_t any = 0u;
 #pragma unroll
     for (int i = 0; i < 64; ++i)
-        pm[i] = v[i];
-
-    return code_planes<32>(pm, dst, 9, budget, pmin, dtab);
-}
-
-// The plane parser shared by FR4 (NP = 32 planes) and FR4D (NP = 64): reads
-// planes NP-1 .. pmin from r (positioned past the header) within `budget`
-// bits into pm[p] (bit p of coefficients 0..31) and pm[NP + p] (32..63);
-// planes not received are zero.
-template <int NP>
-__device__ __forceinline__ void parse_planes(BitReader &r, int budget, int pmin, uint32_t *pm)
-{
-    int n = 0;
-    int p = NP - 1;
+        any |= v[i] ^ kNB;
+    const int skip = min(__clz((int)any), 32 - pmin);
+    to_planes32<0>(v);   // v[p]      = bits p of coefficients 0..31
+    to_planes32<32>(v);  // v[32 + p] = bits p of coefficients 32..63
+    dst[0] = 1u | ((uint32_t)((emax + 127) & 0xFF) << 1);
+    dst[1] = 0u;
+    CodePos c{0, 9 + skip};
+    int p = 31 - skip;
+    auto code_half = [&](int base) {  // planes base + 15 .. base
+        const int stop = max(pmin, base);
+        const uint32_t *pb = pm - base;
 #pragma unroll 1
-    for (; p >= pmin && r.pos < budget; --p) {
-        const int n1 = n < 32 ? n : 32;
-        uint32_t xl = r.get(n1);
-        uint32_t xh = n > 32 ? r.get(n - 32) : 0u;
-        if (n < 64) {
-            uint64_t X = 0ull;  // the plane's new ones
-            for (;;) {
-                // The segments (group bit, scan) that end inside the next 32
-                // stream bits are parsed from one register, k bits in; the
-                // reader then advances once.  A segment that reaches past
-                // the window is parsed again from a fresh window, and from
-                // the long-scan path below when even that is too short.
-                const uint32_t wv = r.peek32();
-                int k = 0;
-                int state = 0;  // 0: window used up; 1: plane done; 2: segment reaches past the window
-                while (k < 32) {
-                    const uint32_t w = wv >> k;
-                    if ((w & 1u) == 0u) {  // group test: nothing more in this plane
-                        ++k;
-                        state = 1;
-                        break;
-                    }
-                    const int len = 63 - n;  // explicit scan bits at most (after the group bit)
-                    const uint32_t sc = w >> 1;  // the 31 - k scan bits inside the window
-                    const int t = __ffs((int)sc) - 1;
-                    if (sc != 0u && t < len) {
-                        X |= 1ull << (n + t);
-                        n += t + 1;
-                        k += t + 2;
-                        continue;
-                    }
-                    if (len <= 31 - k) {  // the len scan bits are zero: the last coefficient's one is implied
-                        if (r.pos + k + 1 + len <= budget) {
-                            X |= 1ull << 63;
-                            n = 64;
-                        }
-                        k += 1 + len;
-                        state = 1;
-                        break;
-                    }
-                    state = 2;
-                    break;
-                }
-                r.skip(k);
-                if (state == 1)
-                    break;
-                if (state == 0 || k > 0)
-                    continue;
-                // long scan: group bit 1, then 31 zero bits of a scan of len > 31
-                const int len = 63 - n;
-                r.skip(32);
-                int done = 31;
-                bool found = false;
-                for (;;) {
-                    const int rem = len - done;
-                    const int mm = rem < 32 ? rem : 32;
-                    const uint32_t s2 = r.peek32() & low_mask(mm);
-                    if (s2 != 0u) {
-                        const int f = __ffs((int)s2);
-                        const int t = done + f - 1;
-                        r.skip(f);
-                        X |= 1ull << (n + t);
-                        n += t + 1;
-                        found = true;
-                        break;
-                    }
-                    if (rem <= 32) {
-                        if (r.pos + rem <= budget) {
-                            X |= 1ull << 63;
-                            n = 64;
-                        }
-                        r.skip(rem);
-                        break;
-                    }
-                    r.skip(32);
-                    done += 32;
-                }
-                if (!found)
-                    break;
-            }
-            xl |= (uint32_t)X;
-            xh |= (uint32_t)(X >> 32);
-        }
-        pm[p] = xl;
-        pm[NP + p] = xh;
+        for (; p >= stop && c.off < budget; --p)
+            c = code_plane(dst, pb[p], pb[16 + p], c.n, c.off);
+    };
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        pm[i] = v[16 + i];
+        pm[16 + i] = v[48 + i];
     }
-    for (; p >= 0; --p) {  // planes past the budget or below the coded range
-        pm[p] = 0u;
-        pm[NP + p] = 0u;
+    code_half(16);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        pm[i] = v[i];
+        pm[16 + i] = v[32 + i];
     }
+    code_half(0);
+    clear_tail(dst, c.off, words);
+    return c.off;
 }
 
-// Decode one block of `nwords` words (2R at a fixed rate) with the plane
-// range of `mode`.
-__device__ __forceinline__ void decode_block(const uint32_t *src, int nwords, int mode, int mparam,
-                                             float (&out)[64], uint32_t *pm)
+struct Plane {
+    uint32_t xl, xh;  // bits of coefficients 0..31 and 32..63
+    int n, pos;       // significant coefficients and stream position behind it
+};
+
+// A plane's new ones, segment by segment, from the group bit at `pos` on: a
+// group bit 1, zeros, a one; a 0 group bit ends the plane.  Any stream.
+__device__ __noinline__ Plane parse_segments(const uint32_t *w, int nwords, int n, int pos)
+{
+    uint64_t X = 0ull;
+    for (;;) {
+        const uint32_t wv = bits_at(w, nwords, pos);
+        if ((wv & 1u) == 0u) {  // group test: nothing more in this plane
+            ++pos;
+            break;
+        }
+        const int len = 63 - n;  // explicit scan bits at most (after the group bit)
+        uint32_t sc = wv >> 1;   // 31 of them
+        int t = __ffs((int)sc) - 1;
+        if (sc == 0u && len > 31) {  // a longer scan
+            const int mm = len - 31 < 32 ? len - 31 : 32;
+            sc = bits_at(w, nwords, pos + 32) & low_mask(mm);
+            t = 30 + __ffs((int)sc);
+        }
+        if (sc != 0u && t < len) {
+            X |= 1ull << (n + t);
+            n += t + 1;
+            pos += t + 2;
+            continue;
+        }
+        // the scan bits are zero: the last coefficient's one is implied
+        if (pos + 1 + len <= 32 * nwords) {
+            X |= 1ull << 63;
+            n = 64;
+        }
+        pos += 1 + len;
+        break;
+    }
+    return Plane{(uint32_t)X, (uint32_t)(X >> 32), n, pos};
+}
+
+// One bit plane of a block: `n` refinement bits of the significant
+// coefficients, then the new ones (see code_planes for the form).
+//
+// The new ones of a plane are found together.  Past the first group bit the
+// stream holds the plane's bits with every one followed by the group bit of
+// the next segment, so in a run of ones they alternate: value, group, value
+// ..; the plane ends after the first run of odd length, whose last one has
+// the group bit 0 behind it.  Runs that start on an even bit are told from
+// the others by one addition that ripples through them (`ec`), which gives
+// every group one at once (`gr`); removing those below the end leaves the
+// plane's bits.  A plane has few new ones (20 in the 32 planes of a block of
+// the benchmark's field), but some lane of a warp has some in nearly every
+// plane, so all lanes go through it.  A plane whose end does not lie in the
+// 32-bit window, or that reaches the last coefficient (once per block), is
+// parsed by parse_segments.
+__device__ __forceinline__ Plane parse_plane(const uint32_t *w, int nwords, int n, int pos)
+{
+    const uint32_t *p = w + (pos >> 5);
+    const uint32_t a0 = p[0], a1 = p[1], a2 = p[2];
+    const int at = pos + n;
+    const uint32_t *ps = w + (at >> 5);
+    const uint32_t s = __funnelshift_r(ps[0], ps[1], at);  // from the group bit on
+    const bool rest = n < 64, has = (s & 1u) != 0u && rest;
+    const uint32_t sc = has ? s >> 1 : 0u;
+    const uint32_t ec = sc + (sc & ~(sc << 1) & 0x55555555u);  // starts of runs: a one after a zero
+    const uint32_t gr = sc & (ec ^ 0xAAAAAAAAu);
+    const uint32_t odd = sc & ~(sc >> 1) & ~gr;  // value ones with a group bit 0 behind (bit 30: perhaps)
+    const uint32_t upto = odd ^ (odd - 1u);      // bits up to the first of them
+    uint32_t v = sc & upto, g = gr & upto;
+    const int k = __popc(upto);
+    const int nv = k - __popc(g);  // coefficients scanned
+    const uint64_t keep = shl64(~0ull, n);  // of the refinement bits: those below
+    Plane r;
+    r.xl = __funnelshift_r(a0, a1, pos) & ~(uint32_t)keep;
+    r.xh = __funnelshift_r(a1, a2, pos) & ~(uint32_t)(keep >> 32);
+    r.n = has ? n + nv : n;
+    r.pos = at + (has ? k + 2 : (rest ? 1 : 0));  // with both group bits
+    if (has && (k > 30 || n + nv > 63)) {
+        const Plane t = parse_segments(w, nwords, n, at);
+        r.xl |= t.xl;
+        r.xh |= t.xh;
+        r.n = t.n;
+        r.pos = t.pos;
+        return r;
+    }
+    // take the group ones out, lowest first; the first removal without a test
+    // (with no group one left it changes nothing)
+    do {
+        const uint32_t g1 = g - 1u, below = g1 & ~g;
+        v = (v & below) | ((v >> 1) & ~below);
+        g = (g & g1) >> 1;
+    } while (g != 0u);
+    const uint64_t y = shl64(v, n);
+    r.xl |= (uint32_t)y;
+    r.xh |= (uint32_t)(y >> 32);
+    return r;
+}
+
+// Decode one block of `nwords` words (2R at a fixed rate), held in shared
+// memory with kZeroWords zeros behind, with the plane range of `mode`.  The
+// planes are parsed 16 at a time into the thread's 32 words at pm and taken
+// from there into registers, half transposed: half the shared memory of all
+// 32 planes, for 24 warps per SM instead of 16.
+__device__ __forceinline__ void decode_block(const uint32_t *w, int nwords, int mode, int mparam, float (&out)[64],
+                                             uint32_t *pm)
 {
     const int budget = 32 * nwords;
-    const uint32_t w0 = nwords > 0 ? __ldg(src) : 0u;
+    const uint32_t w0 = w[0];
     if ((w0 & 1u) == 0u) {
 #pragma unroll
         for (int i = 0; i < 64; ++i)
@@ -553,43 +579,157 @@ __device__ __forceinline__ void decode_block(const uint32_t *src, int nwords, in
     }
     const int emax = (int)((w0 >> 1) & 0xFFu) - 127;
     const int pmin = plane_floor(mode, mparam, emax);
-    BitReader r;
-    r.init(src, 9, nwords);
-    parse_planes<32>(r, budget, pmin, pm);
-    uint32_t u[64];
+    // the leading planes without a one, a group bit 0 each (up to 16 of them)
+    const uint32_t lead = __funnelshift_r(w0, w[1], 9) | 0x10000u;
+    const int skip = min(__ffs((int)lead) - 1, budget - 9);
+    int pos = 9 + skip, n = 0, p = 31 - skip;
+    auto parse_half = [&](int base) {  // planes base + 15 .. base
+        const int stop = max(pmin, base);
+        uint32_t *pb = pm - base;
 #pragma unroll
-    for (int i = 0; i < 64; ++i)
+        for (int i = 0; i < 32; ++i)
+            pm[i] = 0u;
+#pragma unroll 1
+        for (; p >= stop && pos < budget; --p) {
+            const Plane r = parse_plane(w, nwords, n, pos);
+            pb[p] = r.xl;
+            pb[16 + p] = r.xh;
+            n = r.n;
+            pos = r.pos;
+        }
+    };
+    uint32_t u[64];
+    parse_half(16);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        u[16 + i] = pm[i];
+        u[48 + i] = pm[16 + i];
+    }
+    parse_half(0);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
         u[i] = pm[i];
-    transpose32<0>(u);
-    transpose32<32>(u);
+        u[32 + i] = pm[16 + i];
+    }
+    const int k = emax - kPrec;
+    from_planes32<0>(u);
+    from_planes32<32>(u);
     int32_t q[64];
     from_coding_order(q, u, std::make_integer_sequence<int, 64>{});
     transform_inv(q);
     // x = RN(RN(q) * 2^(emax - 26)): one exact or correctly rounded scaling.
-    const int k = emax - kPrec;
     const bool split = k < -126;
     const float sa = __int_as_float(((split ? k + 64 : k) + 127) << 23);
-    const float sb = __int_as_float((-64 + 127) << 23);
 #pragma unroll
-    for (int i = 0; i < 64; ++i) {
-        float f = __fmul_rn(__int2float_rn(q[i]), sa);
-        if (split)
-            f = __fmul_rn(f, sb);
-        out[i] = f;
+    for (int i = 0; i < 64; ++i)
+        out[i] = __fmul_rn(__int2float_rn(q[i]), sa);
+    if (split) {
+        const float sb = __int_as_float((-64 + 127) << 23);
+#pragma unroll
+        for (int i = 0; i < 64; ++i)
+            out[i] = __fmul_rn(out[i], sb);
     }
 }
 
-// ---- kernels ------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) fr4_encode_kernel(ConstRing in, int64_t nx, int64_t ny, int64_t z0,
-                                                             int64_t nblk, int rate, uint32_t *__restrict__ out)
+// Words per block in the decoder's shared memory: odd, so that the threads'
+// blocks start in different banks.
+__host__ __device__ constexpr int decode_stride(int words) { return (words + kZeroWords) | 1; }
+
+// A warp's `nv` consecutive blocks of `words` words from the stream at `src`
+// into its part of shared memory.
+__device__ __forceinline__ void stage_blocks(const uint32_t *__restrict__ src, int nv, int words, int stride,
+                                             uint32_t *dst)
 {
-    extern __shared__ uint32_t smem[];
-    __shared__ uint16_t dtab[256];
-    init_dup_table(dtab);
-    __syncthreads();
-    const int words = 2 * rate, stride = words + kSlack + 1;
-    const int64_t first = (int64_t)blockIdx.x * kThreads;
-    const int64_t b = first + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    if ((words & 3) == 0 && ((uintptr_t)src & 15) == 0) {
+        // chunk c of 4 words is words 4 (c mod q) .. of block c / q
+        const int q = words >> 2;
+        int blk = lane / q, ch = lane - blk * q;
+        const int step_blk = 32 / q, step_ch = 32 - step_blk * q;
+        for (int c = lane; c < nv * q; c += 32) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src) + c);
+            uint32_t *d = dst + blk * stride + 4 * ch;
+            d[0] = v.x;
+            d[1] = v.y;
+            d[2] = v.z;
+            d[3] = v.w;
+            blk += step_blk;
+            ch += step_ch;
+            if (ch >= q) {
+                ch -= q;
+                ++blk;
+            }
+        }
+    } else {
+        int blk = lane / words, wd = lane - blk * words;
+        const int step_blk = 32 / words, step_wd = 32 - step_blk * words;
+        for (int o = lane; o < nv * words; o += 32) {
+            dst[blk * stride + wd] = __ldg(src + o);
+            blk += step_blk;
+            wd += step_wd;
+            if (wd >= words) {
+                wd -= words;
+                ++blk;
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kZeroWords; ++i)
+        dst[lane * stride + words + i] = 0u;
+    __syncwarp();
+}
+
+// ---- kernels ------------------------------------------------------------------
+// Words per block in the encoder's shared memory: odd, so that the threads'
+// blocks start in different banks.
+__host__ __device__ constexpr int encode_stride(int words) { return (words + kSlack) | 1; }
+
+// A warp's `nv` consecutive blocks of `words` words from its part of shared
+// memory to the stream at `dst`.
+__device__ __forceinline__ void store_blocks(uint32_t *dst, int nv, int words, int stride, const uint32_t *src)
+{
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    if ((words & 3) == 0 && ((uintptr_t)dst & 15) == 0) {
+        // chunk c of 4 words is words 4 (c mod q) .. of block c / q
+        const int q = words >> 2;
+        int blk = lane / q, ch = lane - blk * q;
+        const int step_blk = 32 / q, step_ch = 32 - step_blk * q;
+        for (int c = lane; c < nv * q; c += 32) {
+            const uint32_t *w = src + blk * stride + 4 * ch;
+            reinterpret_cast<uint4 *>(dst)[c] = make_uint4(w[0], w[1], w[2], w[3]);
+            blk += step_blk;
+            ch += step_ch;
+            if (ch >= q) {
+                ch -= q;
+                ++blk;
+            }
+        }
+        return;
+    }
+    int blk = lane / words, wd = lane - blk * words;
+    const int step_blk = 32 / words, step_wd = 32 - step_blk * words;
+    for (int o = lane; o < nv * words; o += 32) {
+        dst[o] = src[blk * stride + wd];
+        blk += step_blk;
+        wd += step_wd;
+        if (wd >= words) {
+            wd -= words;
+            ++blk;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 6) fr4_encode_kernel(ConstRing in, int64_t nx, int64_t ny, int64_t z0,
+                                                                 int64_t nblk, int rate, uint32_t *__restrict__ out)
+{
+    extern __shared__ uint32_t smem[];  // each thread's block, then each thread's planes
+    const int words = 2 * rate, stride = encode_stride(words);
+    const int64_t b = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    const int64_t first = b - (threadIdx.x & 31);
+    if (first >= nblk)
+        return;
+    uint32_t *mine = smem + threadIdx.x * stride;
     if (b < nblk) {
         const int64_t nbx = nx >> 2, nby = ny >> 2;
         const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
@@ -606,60 +746,31 @@ __global__ void __launch_bounds__(kThreads) fr4_encode_kernel(ConstRing in, int6
                 v[16 * k + 4 * j + 2] = __float_as_uint(f.z);
                 v[16 * k + 4 * j + 3] = __float_as_uint(f.w);
             }
-        encode_block(v, words, OOC_FR4_RATE, 0, smem + threadIdx.x * stride,
-                     smem + kThreads * stride + threadIdx.x * kPlaneStride, dtab);
+        encode_block(v, words, OOC_FR4_RATE, 0, mine, smem + kThreads * stride + threadIdx.x * kHalfStride);
     }
-    __syncthreads();
-    const int64_t left = nblk - first;
-    const int nvalid = left < kThreads ? (int)left : kThreads;
-    uint32_t *dst = out + first * words;
-    if ((words & 3) == 0 && ((uintptr_t)out & 15) == 0) {
-        // 16-byte stores: chunk c of the CTA's output is words 4 (c mod q) ..
-        // of block c / q, q = words / 4; c advances by kThreads
-        const int q = words >> 2;
-        int blk = threadIdx.x / q, ch = threadIdx.x - blk * q;
-        const int step_blk = kThreads / q, step_ch = kThreads - step_blk * q;
-        for (int c = threadIdx.x; c < nvalid * q; c += kThreads) {
-            const uint32_t *w = smem + blk * stride + 4 * ch;
-            reinterpret_cast<uint4 *>(dst)[c] = make_uint4(w[0], w[1], w[2], w[3]);
-            blk += step_blk;
-            ch += step_ch;
-            if (ch >= q) {
-                ch -= q;
-                ++blk;
-            }
-        }
-        return;
-    }
-    // word o of the CTA's output is word (o mod words) of block (o / words);
-    // o advances by kThreads, so block and word advance incrementally
-    int blk = threadIdx.x / words, wd = threadIdx.x - blk * words;
-    const int step_blk = kThreads / words, step_wd = kThreads - step_blk * words;
-    for (int o = threadIdx.x; o < nvalid * words; o += kThreads) {
-        dst[o] = smem[blk * stride + wd];
-        blk += step_blk;
-        wd += step_wd;
-        if (wd >= words) {
-            wd -= words;
-            ++blk;
-        }
-    }
+    store_blocks(out + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
+                 mine - (threadIdx.x & 31) * stride);
 }
 
-// MINB CTAs per SM: 6 (80 registers) for rates up to 16, 5 (96 registers,
-// more L1 beside the plane masks) above.  1024^3 decode, 6 against 5:
-// R = 8 3.35 against 3.60 ms, R = 16 4.19 against 4.30, R = 24 4.90
-// against 4.59.
+// MINB CTAs per SM: 6 (80 registers) up to R = 16; above, where the staged
+// blocks leave room for 5, 5 (96 registers).
 template <int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) fr4_decode_kernel(const uint32_t *__restrict__ in, int64_t nx, int64_t ny,
                                                              int64_t z0, int64_t nblk, int rate, Ring out)
 {
-    extern __shared__ uint32_t smem[];  // each thread's plane masks
+    extern __shared__ uint32_t smem[];  // each thread's block
+    const int words = 2 * rate, stride = decode_stride(words);
     const int64_t b = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    const int64_t first = b - (threadIdx.x & 31);
+    if (first >= nblk)
+        return;
+    uint32_t *mine = smem + threadIdx.x * stride;
+    stage_blocks(in + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
+                 mine - (threadIdx.x & 31) * stride);
     if (b >= nblk)
         return;
     float f[64];
-    decode_block(in + b * (2 * rate), 2 * rate, OOC_FR4_RATE, 0, f, smem + threadIdx.x * kPlaneStride);
+    decode_block(mine, words, OOC_FR4_RATE, 0, f, smem + kThreads * stride + threadIdx.x * kHalfStride);
     const int64_t nbx = nx >> 2, nby = ny >> 2;
     const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
     const int64_t slot = ring_slot(z0 + 4 * bz, out.zbase, out.nslot);
@@ -775,8 +886,8 @@ template <int... R>
 __device__ __forceinline__ void to_coding_order64(uint32_t (&lo)[64], uint32_t (&hi)[64], const int64_t (&q)[64],
                                                   std::integer_sequence<int, R...>)
 {
-    ((lo[R] = (uint32_t)(((uint64_t)q[std::integral_constant<int, order_at(R)>::value] + kNB64) ^ kNB64),
-      hi[R] = (uint32_t)((((uint64_t)q[std::integral_constant<int, order_at(R)>::value] + kNB64) ^ kNB64) >> 32)),
+    ((lo[R] = (uint32_t)((uint64_t)q[std::integral_constant<int, order_at(R)>::value] + kNB64),
+      hi[R] = (uint32_t)(((uint64_t)q[std::integral_constant<int, order_at(R)>::value] + kNB64) >> 32)),
      ...);
 }
 
@@ -785,7 +896,7 @@ __device__ __forceinline__ void from_coding_order64(int64_t (&q)[64], const uint
                                                     const uint32_t (&hi)[64], std::integer_sequence<int, R...>)
 {
     ((q[std::integral_constant<int, order_at(R)>::value] =
-          (int64_t)(((((uint64_t)hi[R] << 32) | lo[R]) ^ kNB64) - kNB64)),
+          (int64_t)((((uint64_t)hi[R] << 32) | lo[R]) - kNB64)),
      ...);
 }
 
@@ -793,10 +904,10 @@ __device__ __forceinline__ void from_coding_order64(int64_t (&q)[64], const uint
 // 0..31) and pm[64 + p] (32..63) for p = 0..63, and back.
 __device__ __forceinline__ void words_to_planes64(uint32_t (&lo)[64], uint32_t (&hi)[64], uint32_t *pm)
 {
-    transpose32<0>(lo);
-    transpose32<32>(lo);
-    transpose32<0>(hi);
-    transpose32<32>(hi);
+    to_planes32<0>(lo);
+    to_planes32<32>(lo);
+    to_planes32<0>(hi);
+    to_planes32<32>(hi);
 #pragma unroll
     for (int p = 0; p < 32; ++p) {
         pm[p] = lo[p];
@@ -815,10 +926,10 @@ __device__ __forceinline__ void planes_to_words64(const uint32_t *pm, uint32_t (
         lo[32 + p] = pm[64 + p];
         hi[32 + p] = pm[96 + p];
     }
-    transpose32<0>(lo);
-    transpose32<32>(lo);
-    transpose32<0>(hi);
-    transpose32<32>(hi);
+    from_planes32<0>(lo);
+    from_planes32<32>(lo);
+    from_planes32<0>(hi);
+    from_planes32<32>(hi);
 }
 
 __device__ __forceinline__ uint64_t umax64(uint64_t a, uint64_t b) { return a > b ? a : b; }
@@ -830,20 +941,19 @@ __device__ __forceinline__ double pow2d(int k)  // k in [-1022, 1023]
 
 // Encode one FP64 block (bit patterns v) into dst[0 .. words) at a fixed
 // rate: words = 2R, a budget of 64R bits.
-__device__ __forceinline__ void encode_block64(const uint64_t (&v)[64], int words, uint32_t *dst, uint32_t *pm,
-                                               const uint16_t *dtab)
+__device__ __forceinline__ void encode_block64(const uint64_t (&v)[64], int words, uint32_t *dst, uint32_t *pm)
 {
     uint64_t mx = 0;
 #pragma unroll
     for (int i = 0; i < 64; ++i)
         mx = umax64(mx, v[i] & 0x7FFFFFFFFFFFFFFFull);
-    for (int i = 0; i < words + kSlack; ++i)
-        dst[i] = 0u;
-    if (mx == 0ull)
+    if (mx == 0ull) {
+        dst[0] = 0u;
+        clear_tail(dst, 0, words);
         return;
+    }
     // largest frexp exponent (biased exponent - 1022; subnormals clamp to -1022)
     const int emax = (int)(mx >> 52) - 1022;
-    dst[0] = 1u | ((uint32_t)(emax + 1023) << 1);
     // q = trunc(x * 2^(58 - emax)) in integer arithmetic on the bits (the
     // FP64 pipe is scarce on this GPU): x = m 2^e with the 53-bit significand
     // m, so |q| = m shifted by e + 58 - emax (left by at most 5, since |x| <
@@ -863,12 +973,18 @@ __device__ __forceinline__ void encode_block64(const uint64_t (&v)[64], int word
     uint32_t lo[64], hi[64];
     to_coding_order64(lo, hi, q, std::make_integer_sequence<int, 64>{});
     words_to_planes64(lo, hi, pm);
-    code_planes<64>(pm, dst, 12, 32 * words, 0, dtab);
+    dst[0] = 1u | ((uint32_t)(emax + 1023) << 1);
+    dst[1] = 0u;
+    CodePos c{0, 12};
+#pragma unroll 1
+    for (int p = 63; p >= 0 && c.off < 32 * words; --p)
+        c = code_plane(dst, pm[p], pm[64 + p], c.n, c.off);
+    clear_tail(dst, c.off, words);
 }
 
-__device__ __forceinline__ void decode_block64(const uint32_t *src, int nwords, double (&out)[64], uint32_t *pm)
+__device__ __forceinline__ void decode_block64(const uint32_t *w, int nwords, double (&out)[64], uint32_t *pm)
 {
-    const uint32_t w0 = nwords > 0 ? __ldg(src) : 0u;
+    const uint32_t w0 = w[0];
     if ((w0 & 1u) == 0u) {
 #pragma unroll
         for (int i = 0; i < 64; ++i)
@@ -876,9 +992,20 @@ __device__ __forceinline__ void decode_block64(const uint32_t *src, int nwords, 
         return;
     }
     const int emax = (int)((w0 >> 1) & 0x7FFu) - 1023;
-    BitReader r;
-    r.init(src, 12, nwords);
-    parse_planes<64>(r, 32 * nwords, 0, pm);
+    const int budget = 32 * nwords;
+    int pos = 12, n = 0, p = 63;
+#pragma unroll 1
+    for (; p >= 0 && pos < budget; --p) {
+        const Plane r = parse_plane(w, nwords, n, pos);
+        pm[p] = r.xl;
+        pm[64 + p] = r.xh;
+        n = r.n;
+        pos = r.pos;
+    }
+    for (; p >= 0; --p) {  // planes past the budget
+        pm[p] = 0u;
+        pm[64 + p] = 0u;
+    }
     uint32_t lo[64], hi[64];
     planes_to_words64(pm, lo, hi);
     int64_t q[64];
@@ -901,13 +1028,13 @@ __device__ __forceinline__ void decode_block64(const uint32_t *src, int nwords, 
 __global__ void __launch_bounds__(kThreads64) fr4d_encode_kernel(DConstRing in, int64_t nx, int64_t ny, int64_t z0,
                                                                  int64_t nblk, int rate, uint32_t *__restrict__ out)
 {
-    extern __shared__ uint32_t smem[];
-    __shared__ uint16_t dtab[256];
-    init_dup_table(dtab);
-    __syncthreads();
-    const int words = 2 * rate, stride = words + kSlack + 1;
-    const int64_t first = (int64_t)blockIdx.x * kThreads64;
-    const int64_t b = first + threadIdx.x;
+    extern __shared__ uint32_t smem[];  // each thread's block, then each thread's planes
+    const int words = 2 * rate, stride = encode_stride(words);
+    const int64_t b = (int64_t)blockIdx.x * kThreads64 + threadIdx.x;
+    const int64_t first = b - (threadIdx.x & 31);
+    if (first >= nblk)
+        return;
+    uint32_t *mine = smem + threadIdx.x * stride;
     if (b < nblk) {
         const int64_t nbx = nx >> 2, nby = ny >> 2;
         const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
@@ -925,28 +1052,29 @@ __global__ void __launch_bounds__(kThreads64) fr4d_encode_kernel(DConstRing in, 
                 v[16 * k + 4 * j + 2] = (uint64_t)__double_as_longlong(c.x);
                 v[16 * k + 4 * j + 3] = (uint64_t)__double_as_longlong(c.y);
             }
-        encode_block64(v, words, smem + threadIdx.x * stride, smem + kThreads64 * stride + threadIdx.x * kPlaneStride64,
-                       dtab);
+        encode_block64(v, words, mine, smem + kThreads64 * stride + threadIdx.x * kPlaneStride64);
     }
-    __syncthreads();
-    const int64_t left = nblk - first;
-    const int nvalid = left < kThreads64 ? (int)left : kThreads64;
-    uint32_t *dst = out + first * words;
-    // word o of the CTA's output is word (o mod words) of block (o / words)
-    for (int o = threadIdx.x; o < nvalid * words; o += kThreads64)
-        dst[o] = smem[(o / words) * stride + (o % words)];
+    store_blocks(out + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
+                 mine - (threadIdx.x & 31) * stride);
 }
 
 __global__ void __launch_bounds__(kThreads64) fr4d_decode_kernel(const uint32_t *__restrict__ in, int64_t nx,
                                                                  int64_t ny, int64_t z0, int64_t nblk, int rate,
                                                                  DRing out)
 {
-    extern __shared__ uint32_t smem[];  // each thread's plane words
+    extern __shared__ uint32_t smem[];  // each thread's block and plane words
+    const int words = 2 * rate, stride = decode_stride(words);
     const int64_t b = (int64_t)blockIdx.x * kThreads64 + threadIdx.x;
+    const int64_t first = b - (threadIdx.x & 31);
+    if (first >= nblk)
+        return;
+    uint32_t *mine = smem + threadIdx.x * stride;
+    stage_blocks(in + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
+                 mine - (threadIdx.x & 31) * stride);
     if (b >= nblk)
         return;
     double f[64];
-    decode_block64(in + b * (2 * rate), 2 * rate, f, smem + threadIdx.x * kPlaneStride64);
+    decode_block64(mine, words, f, smem + kThreads64 * stride + threadIdx.x * kPlaneStride64);
     const int64_t nbx = nx >> 2, nby = ny >> 2;
     const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
     const int64_t slot = ring_slot(z0 + 4 * bz, out.zbase, out.nslot);
@@ -964,8 +1092,8 @@ __global__ void __launch_bounds__(kThreads64) fr4d_decode_kernel(const uint32_t 
 size_t smem_bytes64(int rate, bool encoder)
 {
     if (!encoder)
-        return (size_t)kThreads64 * kPlaneStride64 * sizeof(uint32_t);
-    return ((size_t)kThreads64 * (2 * rate + kSlack + 1) + (size_t)kThreads64 * kPlaneStride64) * sizeof(uint32_t);
+        return (size_t)kThreads64 * (decode_stride(2 * rate) + kPlaneStride64) * sizeof(uint32_t);
+    return (size_t)kThreads64 * (encode_stride(2 * rate) + kPlaneStride64) * sizeof(uint32_t);
 }
 
 cudaError_t ensure_smem_attr64()
@@ -1010,35 +1138,21 @@ __global__ void __launch_bounds__(kThreads)
                             uint32_t *__restrict__ out)
 {
     extern __shared__ uint32_t smem[];
-    __shared__ uint16_t dtab[256];
-    init_dup_table(dtab);
-    __syncthreads();
-    const int stride = words + kSlack + 1;
-    const int64_t first = (int64_t)blockIdx.x * kThreads;
-    const int64_t b = first + threadIdx.x;
+    const int stride = encode_stride(words);
+    const int64_t b = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    const int64_t first = b - (threadIdx.x & 31);
+    if (first >= nblk)
+        return;
     uint32_t *mine = smem + threadIdx.x * stride;
     if (b < nblk) {
         const int64_t nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
         const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
         uint32_t v[64];
         gather_clamped(in, nx, ny, nz, bx, by, bz, v);
-        encode_block(v, words, OOC_FR4_RATE, 0, mine, smem + kThreads * stride + threadIdx.x * kPlaneStride, dtab);
+        encode_block(v, words, OOC_FR4_RATE, 0, mine, smem + kThreads * stride + threadIdx.x * kHalfStride);
     }
-    __syncthreads();
-    const int64_t left = nblk - first;
-    const int nvalid = left < kThreads ? (int)left : kThreads;
-    uint32_t *dst = out + first * words;
-    int blk = threadIdx.x / words, wd = threadIdx.x - blk * words;
-    const int step_blk = kThreads / words, step_wd = kThreads - step_blk * words;
-    for (int o = threadIdx.x; o < nvalid * words; o += kThreads) {
-        dst[o] = smem[blk * stride + wd];
-        blk += step_blk;
-        wd += step_wd;
-        if (wd >= words) {
-            wd -= words;
-            ++blk;
-        }
-    }
+    store_blocks(out + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
+                 mine - (threadIdx.x & 31) * stride);
 }
 
 // Fixed rate: block b is words [b * words, (b + 1) * words).  Variable-size:
@@ -1049,25 +1163,36 @@ __global__ void __launch_bounds__(kThreads)
                             int64_t nx, int64_t ny, int64_t nz, int64_t nblk, int words, int mode, int mparam,
                             float *__restrict__ out)
 {
-    extern __shared__ uint32_t smem[];  // each thread's plane masks
+    extern __shared__ uint32_t smem[];  // each thread's block
+    const int stride = decode_stride(words);
     const int64_t b = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    if (b >= nblk)
-        return;
-    const uint32_t *src;
-    int nw;
+    uint32_t *mine = smem + threadIdx.x * stride;
+    int nw = words;
     if (mode == OOC_FR4_RATE) {
-        src = in + b * words;
-        nw = words;
+        const int64_t first = b - (threadIdx.x & 31);
+        if (first >= nblk)
+            return;
+        stage_blocks(in + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
+                     mine - (threadIdx.x & 31) * stride);
+        if (b >= nblk)
+            return;
     } else {
+        if (b >= nblk)
+            return;
         uint64_t lo = __ldg(index + b), hi = __ldg(index + b + 1);
         lo = lo < (uint64_t)in_words ? lo : (uint64_t)in_words;
         hi = hi < (uint64_t)in_words ? hi : (uint64_t)in_words;
         const uint64_t n = hi > lo ? hi - lo : 0;
         nw = (int)(n < (uint64_t)kVarWords ? n : (uint64_t)kVarWords);
-        src = in + lo;
+        const uint32_t *src = in + lo;
+        for (int i = 0; i < nw; ++i)
+            mine[i] = __ldg(src + i);
+#pragma unroll
+        for (int i = 0; i < kZeroWords; ++i)
+            mine[nw + i] = 0u;
     }
     float f[64];
-    decode_block(src, nw, mode, mparam, f, smem + threadIdx.x * kPlaneStride);
+    decode_block(mine, nw, mode, mparam, f, smem + kThreads * stride + threadIdx.x * kHalfStride);
     const int64_t nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
     const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
 #pragma unroll
@@ -1115,7 +1240,6 @@ __global__ void __launch_bounds__(kThreads)
                           unsigned long long *scratch)
 {
     extern __shared__ uint32_t smem[];
-    __shared__ uint16_t dtab[256];
     __shared__ uint64_t warp_tot[kThreads / 32];
     __shared__ int64_t s_tile;
     __shared__ uint64_t s_prefix;
@@ -1125,10 +1249,9 @@ __global__ void __launch_bounds__(kThreads)
         s_tile = (int64_t)atomicAdd(scratch, 1ull);
         s_fail = 0;
     }
-    init_dup_table(dtab);
     __syncthreads();
     const int64_t tile = s_tile;
-    constexpr int stride = kVarWords + kSlack + 1;
+    constexpr int stride = encode_stride(kVarWords);
     const int64_t b = tile * kThreads + threadIdx.x;
     uint32_t *mine = smem + threadIdx.x * stride;
     uint64_t nw = 0;
@@ -1138,7 +1261,7 @@ __global__ void __launch_bounds__(kThreads)
         uint32_t v[64];
         gather_clamped(in, nx, ny, nz, bx, by, bz, v);
         const int bits = encode_block(v, kVarWords, mode, mparam, mine,
-                                      smem + kThreads * stride + threadIdx.x * kPlaneStride, dtab);
+                                      smem + kThreads * stride + threadIdx.x * kHalfStride);
         nw = (uint64_t)((bits + 31) >> 5);
     }
     // exclusive scan of the word counts over the CTA
@@ -1207,8 +1330,8 @@ __global__ void __launch_bounds__(kThreads)
 size_t dense_smem_bytes(int words, bool encoder)
 {
     if (!encoder)
-        return (size_t)kThreads * kPlaneStride * sizeof(uint32_t);
-    return (size_t)kThreads * (words + kSlack + 1 + kPlaneStride) * sizeof(uint32_t);
+        return (size_t)kThreads * (decode_stride(words) + kHalfStride) * sizeof(uint32_t);
+    return (size_t)kThreads * (encode_stride(words) + kHalfStride) * sizeof(uint32_t);
 }
 
 cudaError_t ensure_dense_smem_attr()
@@ -1234,9 +1357,9 @@ cudaError_t ensure_dense_smem_attr()
 // (stride 65).  The decoder keeps only the plane masks.
 size_t smem_bytes(int rate, bool encoder)
 {
-    if (!encoder)  // the decoder reads its words from the stream directly
-        return (size_t)kThreads * kPlaneStride * sizeof(uint32_t);
-    return ((size_t)kThreads * (2 * rate + kSlack + 1) + (size_t)kThreads * kPlaneStride) * sizeof(uint32_t);
+    if (!encoder)
+        return (size_t)kThreads * (decode_stride(2 * rate) + kHalfStride) * sizeof(uint32_t);
+    return (size_t)kThreads * (encode_stride(2 * rate) + kHalfStride) * sizeof(uint32_t);
 }
 
 cudaError_t ensure_smem_attr()
