@@ -407,7 +407,8 @@ __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mo
     const int budget = 32 * words;
     if (mx == 0u) {
         dst[0] = 0u;
-        clear_tail(dst, 0, words);
+        if (mode == OOC_FR4_RATE)
+            clear_tail(dst, 0, words);
         return 1;
     }
     const int emax = (int)(mx >> 23) - 126;  // largest frexp exponent, >= -126
@@ -458,7 +459,8 @@ __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mo
         pm[16 + i] = v[32 + i];
     }
     code_half(0);
-    clear_tail(dst, c.off, words);
+    if (mode == OOC_FR4_RATE)
+        clear_tail(dst, c.off, words);
     return c.off;
 }
 
@@ -1111,10 +1113,19 @@ cudaError_t ensure_smem_attr64()
 }
 
 // ---- dense fields of any shape, fixed rate and variable-size modes -------------
-constexpr int kVarWords = 130;  // largest variable-size block (9 + 32 * 129 bits)
+constexpr int kVarWords = 130;  // most words of a variable-size block that a decoder takes
+
+// Most words of a block coded without a budget down to plane pmin: 9 header
+// bits; per plane, the refinement and scanned bits are at most one per
+// coefficient and the closing group bit one more; every coefficient costs one
+// group bit 1.  68 words for all 32 planes.
+__host__ __device__ constexpr int var_block_words(int pmin) { return (9 + (32 - pmin) * 65 + 64 + 31) / 32; }
 
 // Block (bx, by, bz) of a dense field; a block reaching past the field takes
-// the value of the nearest point inside it (each coordinate clamped).
+// the value of the nearest point inside it (each coordinate clamped).  VEC:
+// nx is a multiple of 4 and the field 16-byte aligned, so a row of the block
+// is one 16-byte access.
+template <bool VEC>
 __device__ __forceinline__ void gather_clamped(const float *in, int64_t nx, int64_t ny, int64_t nz, int64_t bx,
                                                int64_t by, int64_t bz, uint32_t (&v)[64])
 {
@@ -1124,16 +1135,52 @@ __device__ __forceinline__ void gather_clamped(const float *in, int64_t nx, int6
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const float *row = in + (z * ny + min(4 * by + j, ny - 1)) * nx;
+            if (VEC) {
+                const float4 f = __ldg(reinterpret_cast<const float4 *>(row + 4 * bx));
+                v[16 * k + 4 * j + 0] = __float_as_uint(f.x);
+                v[16 * k + 4 * j + 1] = __float_as_uint(f.y);
+                v[16 * k + 4 * j + 2] = __float_as_uint(f.z);
+                v[16 * k + 4 * j + 3] = __float_as_uint(f.w);
+            } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                v[16 * k + 4 * j + i] = __float_as_uint(__ldg(row + min(4 * bx + i, nx - 1)));
+                for (int i = 0; i < 4; ++i)
+                    v[16 * k + 4 * j + i] = __float_as_uint(__ldg(row + min(4 * bx + i, nx - 1)));
+            }
         }
     }
 }
 
+// The points of block (bx, by, bz) that lie inside the field; VEC as above.
+template <bool VEC>
+__device__ __forceinline__ void scatter_inside(float *out, int64_t nx, int64_t ny, int64_t nz, int64_t bx, int64_t by,
+                                               int64_t bz, const float (&f)[64])
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int64_t z = 4 * bz + k, y = 4 * by + j;
+            if (z < nz && y < ny) {
+                float *row = out + (z * ny + y) * nx + 4 * bx;
+                if (VEC) {
+                    *reinterpret_cast<float4 *>(row) = make_float4(f[16 * k + 4 * j], f[16 * k + 4 * j + 1],
+                                                                   f[16 * k + 4 * j + 2], f[16 * k + 4 * j + 3]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (4 * bx + i < nx)
+                            row[i] = f[16 * k + 4 * j + i];
+                }
+            }
+        }
+}
+
+inline bool vec_rows(const void *field, int64_t nx) { return nx % 4 == 0 && (uintptr_t)field % 16 == 0; }
+
 // Fixed rate for any shape: `words` words per block, the CTA's output
 // staged and written with coalesced stores.
-__global__ void __launch_bounds__(kThreads)
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads, 6)
     fr4_encode_dense_kernel(const float *__restrict__ in, int64_t nx, int64_t ny, int64_t nz, int64_t nblk, int words,
                             uint32_t *__restrict__ out)
 {
@@ -1148,63 +1195,91 @@ __global__ void __launch_bounds__(kThreads)
         const int64_t nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
         const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
         uint32_t v[64];
-        gather_clamped(in, nx, ny, nz, bx, by, bz, v);
+        gather_clamped<VEC>(in, nx, ny, nz, bx, by, bz, v);
         encode_block(v, words, OOC_FR4_RATE, 0, mine, smem + kThreads * stride + threadIdx.x * kHalfStride);
     }
     store_blocks(out + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
                  mine - (threadIdx.x & 31) * stride);
 }
 
-// Fixed rate: block b is words [b * words, (b + 1) * words).  Variable-size:
-// words [index[b], index[b + 1]), clamped to the stream and to kVarWords.
-// Only the points inside the field are written.
-__global__ void __launch_bounds__(kThreads)
-    fr4_decode_dense_kernel(const uint32_t *__restrict__ in, int64_t in_words, const uint64_t *__restrict__ index,
-                            int64_t nx, int64_t ny, int64_t nz, int64_t nblk, int words, int mode, int mparam,
-                            float *__restrict__ out)
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads, 6)
+    fr4_decode_dense_kernel(const uint32_t *__restrict__ in, int64_t nx, int64_t ny, int64_t nz, int64_t nblk,
+                            int words, float *__restrict__ out)
 {
-    extern __shared__ uint32_t smem[];  // each thread's block
+    extern __shared__ uint32_t smem[];  // each thread's block, then each thread's planes
     const int stride = decode_stride(words);
     const int64_t b = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    const int64_t first = b - (threadIdx.x & 31);
+    if (first >= nblk)
+        return;
     uint32_t *mine = smem + threadIdx.x * stride;
-    int nw = words;
-    if (mode == OOC_FR4_RATE) {
-        const int64_t first = b - (threadIdx.x & 31);
-        if (first >= nblk)
-            return;
-        stage_blocks(in + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
-                     mine - (threadIdx.x & 31) * stride);
-        if (b >= nblk)
-            return;
-    } else {
-        if (b >= nblk)
-            return;
+    stage_blocks(in + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
+                 mine - (threadIdx.x & 31) * stride);
+    if (b >= nblk)
+        return;
+    float f[64];
+    decode_block(mine, words, OOC_FR4_RATE, 0, f, smem + kThreads * stride + threadIdx.x * kHalfStride);
+    const int64_t nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
+    const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
+    scatter_inside<VEC>(out, nx, ny, nz, bx, by, bz, f);
+}
+
+// Variable-size: block b is words [index[b], index[b + 1]), clamped to the
+// stream and to kVarWords.  A warp stages its blocks one behind the other in
+// kVarBuf words (38 per block: 6 CTAs per SM; slots of the largest block's
+// size leave 2), those that fit first and the rest in further rounds.
+constexpr int kVarBuf = 32 * 38;
+static_assert(kVarBuf >= kVarWords + kZeroWords, "any block fits alone");
+
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads, 6)
+    fr4_decode_var_kernel(const uint32_t *__restrict__ in, int64_t in_words, const uint64_t *__restrict__ index,
+                          int64_t nx, int64_t ny, int64_t nz, int64_t nblk, int mode, int mparam,
+                          float *__restrict__ out)
+{
+    extern __shared__ uint32_t smem[];  // the warps' blocks, then each thread's planes
+    const int lane = threadIdx.x & 31;
+    uint32_t *buf = smem + (threadIdx.x >> 5) * kVarBuf;
+    uint32_t *pm = smem + (kThreads / 32) * kVarBuf + threadIdx.x * kHalfStride;
+    const int64_t b = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    bool todo = b < nblk;
+    const uint32_t *src = in;
+    int nw = 0;
+    if (todo) {
         uint64_t lo = __ldg(index + b), hi = __ldg(index + b + 1);
         lo = lo < (uint64_t)in_words ? lo : (uint64_t)in_words;
         hi = hi < (uint64_t)in_words ? hi : (uint64_t)in_words;
         const uint64_t n = hi > lo ? hi - lo : 0;
         nw = (int)(n < (uint64_t)kVarWords ? n : (uint64_t)kVarWords);
-        const uint32_t *src = in + lo;
-        for (int i = 0; i < nw; ++i)
-            mine[i] = __ldg(src + i);
-#pragma unroll
-        for (int i = 0; i < kZeroWords; ++i)
-            mine[nw + i] = 0u;
+        src = in + lo;
     }
-    float f[64];
-    decode_block(mine, nw, mode, mparam, f, smem + kThreads * stride + threadIdx.x * kHalfStride);
     const int64_t nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
     const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
+    while (__any_sync(0xffffffffu, todo)) {
+        const int need = todo ? nw + kZeroWords : 0;
+        int end = need;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+        for (int d = 1; d < 32; d <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, end, d);
+            if (lane >= d)
+                end += t;
+        }
+        const bool now = todo && end <= kVarBuf;
+        if (now) {
+            uint32_t *w = buf + (end - need);
+            for (int i = 0; i < nw; ++i)
+                w[i] = __ldg(src + i);
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int64_t z = 4 * bz + k, y = 4 * by + j, x = 4 * bx + i;
-                if (z < nz && y < ny && x < nx)
-                    out[(z * ny + y) * nx + x] = f[16 * k + 4 * j + i];
-            }
+            for (int i = 0; i < kZeroWords; ++i)
+                w[nw + i] = 0u;
+            float f[64];
+            decode_block(w, nw, mode, mparam, f, pm);
+            scatter_inside<VEC>(out, nx, ny, nz, bx, by, bz, f);
+        }
+        todo = todo && !now;
+        __syncwarp();  // the next round's blocks take this one's places
+    }
 }
 
 // ---- variable-size modes: one pass with a decoupled look-back ---------------------
@@ -1233,11 +1308,13 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned l
 
 // Block b's words at out + index[b]; index[nblk] = total words.  A block is
 // written only if it ends within out_words.  scratch: the tile counter, then
-// one status word per tile, all zero at launch.
-__global__ void __launch_bounds__(kThreads)
+// one status word per tile, all zero at launch.  `cap`: words of shared
+// memory for a block (var_block_words of the lowest plane).
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads, 5)
     fr4_encode_var_kernel(const float *__restrict__ in, int64_t nx, int64_t ny, int64_t nz, int64_t nblk, int mode,
-                          int mparam, uint32_t *__restrict__ out, uint64_t out_words, uint64_t *__restrict__ index,
-                          unsigned long long *scratch)
+                          int mparam, int cap, uint32_t *__restrict__ out, uint64_t out_words,
+                          uint64_t *__restrict__ index, unsigned long long *scratch)
 {
     extern __shared__ uint32_t smem[];
     __shared__ uint64_t warp_tot[kThreads / 32];
@@ -1251,7 +1328,7 @@ __global__ void __launch_bounds__(kThreads)
     }
     __syncthreads();
     const int64_t tile = s_tile;
-    constexpr int stride = encode_stride(kVarWords);
+    const int stride = encode_stride(cap);
     const int64_t b = tile * kThreads + threadIdx.x;
     uint32_t *mine = smem + threadIdx.x * stride;
     uint64_t nw = 0;
@@ -1259,8 +1336,8 @@ __global__ void __launch_bounds__(kThreads)
         const int64_t nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
         const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
         uint32_t v[64];
-        gather_clamped(in, nx, ny, nz, bx, by, bz, v);
-        const int bits = encode_block(v, kVarWords, mode, mparam, mine,
+        gather_clamped<VEC>(in, nx, ny, nz, bx, by, bz, v);
+        const int bits = encode_block(v, cap, mode, mparam, mine,
                                       smem + kThreads * stride + threadIdx.x * kHalfStride);
         nw = (uint64_t)((bits + 31) >> 5);
     }
@@ -1283,37 +1360,48 @@ __global__ void __launch_bounds__(kThreads)
             before += warp_tot[w];
         total += warp_tot[w];
     }
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
+        // the look-back, 32 tiles at a time: lane l reads tile - 1 - l
         uint64_t prefix = 0;
-        if (tile == 0) {
-            st_relaxed_u64(&status[0], kTilePrefix | total);
-        } else {
-            st_relaxed_u64(&status[tile], kTileAgg | total);
-            bool failed = false;
-            for (int64_t j = tile - 1;; --j) {  // tile 0 publishes a prefix, so j stays >= 0
-                uint64_t v = ld_relaxed_u64(&status[j]);
+        bool failed = false;
+        if (lane == 0)
+            st_relaxed_u64(&status[tile], (tile == 0 ? kTilePrefix : kTileAgg) | total);
+        for (int64_t j = tile - 1 - lane; tile > 0; j -= 32) {
+            uint64_t v = kTilePrefix;  // before tile 0: nothing
+            if (j >= 0) {
+                v = ld_relaxed_u64(&status[j]);
                 for (int spins = 0; (v >> 62) == 0 && spins < kLookbackSpins; ++spins) {
                     __nanosleep(64);
                     v = ld_relaxed_u64(&status[j]);
                 }
-                const uint64_t state = v & ~kTileValue;
-                if (state == 0 || state == kTileFailed) {
-                    failed = true;
-                    break;
-                }
-                prefix += v & kTileValue;
-                if (state == kTilePrefix)
-                    break;
             }
+            const uint64_t state = v & ~kTileValue;
+            const uint32_t done = __ballot_sync(0xffffffffu, state == kTilePrefix);
+            const uint32_t bad = __ballot_sync(0xffffffffu, state == 0 || state == kTileFailed);
+            const int last = done ? __ffs((int)done) - 1 : 31;  // tiles up to the nearest prefix count
+            const uint32_t counted = last == 31 ? 0xffffffffu : (2u << last) - 1u;
+            if (bad & counted) {
+                failed = true;
+                break;
+            }
+            uint64_t sum = lane <= last ? v & kTileValue : 0;
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1)
+                sum += __shfl_xor_sync(0xffffffffu, sum, d);
+            prefix += sum;
+            if (done)
+                break;
+        }
+        if (lane == 0) {
             if (failed) {
                 st_relaxed_u64(&status[tile], kTileFailed);  // later tiles stop at once
                 atomicOr(&g_codec_fault, 1u);
                 s_fail = 1;
-            } else {
+            } else if (tile > 0) {
                 st_relaxed_u64(&status[tile], kTilePrefix | (prefix + total));
             }
+            s_prefix = prefix;
         }
-        s_prefix = prefix;
     }
     __syncthreads();
     if (s_fail || b >= nblk)
@@ -1334,19 +1422,31 @@ size_t dense_smem_bytes(int words, bool encoder)
     return (size_t)kThreads * (encode_stride(words) + kHalfStride) * sizeof(uint32_t);
 }
 
+// Shared memory of the variable-size kernels.
+size_t var_encode_smem(int cap) { return dense_smem_bytes(cap, true); }
+constexpr size_t kVarDecodeSmem = (size_t)((kThreads / 32) * kVarBuf + kThreads * kHalfStride) * sizeof(uint32_t);
+
 cudaError_t ensure_dense_smem_attr()
 {
     // set once per process (thread-safe); the attribute is per function
     static const cudaError_t once = [] {
-        cudaError_t e = cudaFuncSetAttribute(fr4_encode_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)dense_smem_bytes(kVarWords, true));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fr4_encode_var_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)dense_smem_bytes(kVarWords, true));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fr4_decode_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)dense_smem_bytes(kVarWords, false));
-        return e;
+        struct {
+            const void *fn;
+            size_t bytes;
+        } const a[] = {{(const void *)fr4_encode_dense_kernel<false>, dense_smem_bytes(128, true)},
+                       {(const void *)fr4_encode_dense_kernel<true>, dense_smem_bytes(128, true)},
+                       {(const void *)fr4_decode_dense_kernel<false>, dense_smem_bytes(128, false)},
+                       {(const void *)fr4_decode_dense_kernel<true>, dense_smem_bytes(128, false)},
+                       {(const void *)fr4_encode_var_kernel<false>, var_encode_smem(var_block_words(0))},
+                       {(const void *)fr4_encode_var_kernel<true>, var_encode_smem(var_block_words(0))},
+                       {(const void *)fr4_decode_var_kernel<false>, kVarDecodeSmem},
+                       {(const void *)fr4_decode_var_kernel<true>, kVarDecodeSmem}};
+        for (const auto &x : a) {
+            const cudaError_t e = cudaFuncSetAttribute(x.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)x.bytes);
+            if (e != cudaSuccess)
+                return e;
+        }
+        return cudaSuccess;
     }();
     return once;
 }
@@ -1452,14 +1552,14 @@ cudaError_t launch_fr4_encode_dense(const float *in, int64_t nx, int64_t ny, int
     const int64_t nblk = fr4_blocks(nx, ny, nz);
     if (nblk <= 0)
         return cudaSuccess;
-    if (words < 1 || words > kVarWords)
+    if (words < 1 || words > 128)
         return cudaErrorInvalidValue;
     cudaError_t e = ensure_dense_smem_attr();
     if (e != cudaSuccess)
         return e;
     const int64_t grid = (nblk + kThreads - 1) / kThreads;
-    fr4_encode_dense_kernel<<<(unsigned)grid, kThreads, dense_smem_bytes(words, true), st>>>(in, nx, ny, nz, nblk,
-                                                                                             words, out);
+    const auto kernel = vec_rows(in, nx) ? fr4_encode_dense_kernel<true> : fr4_encode_dense_kernel<false>;
+    kernel<<<(unsigned)grid, kThreads, dense_smem_bytes(words, true), st>>>(in, nx, ny, nz, nblk, words, out);
     return cudaGetLastError();
 }
 
@@ -1476,8 +1576,10 @@ cudaError_t launch_fr4_encode_var(const float *in, int64_t nx, int64_t ny, int64
     if (e != cudaSuccess)
         return e;
     const int64_t grid = (nblk + kThreads - 1) / kThreads;
-    fr4_encode_var_kernel<<<(unsigned)grid, kThreads, dense_smem_bytes(kVarWords, true), st>>>(
-        in, nx, ny, nz, nblk, mode, mparam, out, out_words, index, (unsigned long long *)scratch);
+    const int cap = var_block_words(mode == OOC_FR4_PRECISION ? 32 - mparam : 0);
+    const auto kernel = vec_rows(in, nx) ? fr4_encode_var_kernel<true> : fr4_encode_var_kernel<false>;
+    kernel<<<(unsigned)grid, kThreads, var_encode_smem(cap), st>>>(in, nx, ny, nz, nblk, mode, mparam, cap, out,
+                                                                   out_words, index, (unsigned long long *)scratch);
     return cudaGetLastError();
 }
 
@@ -1504,8 +1606,16 @@ cudaError_t launch_fr4_decode_dense(const uint32_t *in, int64_t in_words, const 
     if (e != cudaSuccess)
         return e;
     const int64_t grid = (nblk + kThreads - 1) / kThreads;
-    fr4_decode_dense_kernel<<<(unsigned)grid, kThreads, dense_smem_bytes(words, false), st>>>(
-        in, in_words, index, nx, ny, nz, nblk, words, mode, mparam, out);
+    if (mode == OOC_FR4_RATE) {
+        if (words < 1 || words > 128)
+            return cudaErrorInvalidValue;
+        const auto kernel = vec_rows(out, nx) ? fr4_decode_dense_kernel<true> : fr4_decode_dense_kernel<false>;
+        kernel<<<(unsigned)grid, kThreads, dense_smem_bytes(words, false), st>>>(in, nx, ny, nz, nblk, words, out);
+    } else {
+        const auto kernel = vec_rows(out, nx) ? fr4_decode_var_kernel<true> : fr4_decode_var_kernel<false>;
+        kernel<<<(unsigned)grid, kThreads, kVarDecodeSmem, st>>>(in, in_words, index, nx, ny, nz, nblk, mode, mparam,
+                                                                 out);
+    }
     return cudaGetLastError();
 }
 
