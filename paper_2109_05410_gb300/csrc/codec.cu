@@ -789,11 +789,17 @@ __global__ void __launch_bounds__(kThreads, MINB) fr4_decode_kernel(const uint32
 // 58-bit block floating point (emax clamped at -1022, 11 header bits), the
 // FR4 lifting in wrapping int64, the same coding order, 64-bit negabinary
 // and 64 bit planes through the shared plane coder and parser.  One thread
-// owns one block; a CTA of 64 threads keeps each thread's 128 plane words
-// (and, encoding, its staged output) in shared memory.
+// owns one block; a CTA of 64 threads keeps each thread's staged words and 16
+// planes at a time in shared memory.  The high words' 32 planes are transposed
+// and coded first; the low words' only when the budget reaches them (it ends
+// about there at 24 of 64 bits on smooth fields).  56 planes of 1024^2, R = 24
+// and 32, us, against all 128 plane words per thread in shared memory (8 warps
+// per SM): encode 474, 505 -> 388, 396 (12 warps, 168 registers); decode 647,
+// 678 -> 443, 470 (16 warps at 128 registers with spills; 12 warps without,
+// 460, 484), with the scaling as an addition to the exponent instead of a
+// second FP64 instruction per value.
 constexpr int kPrec64 = 58;
 constexpr int kThreads64 = 64;
-constexpr int kPlaneStride64 = 129;  // 128 plane words, odd stride
 constexpr uint64_t kNB64 = 0xAAAAAAAAAAAAAAAAull;
 
 __device__ __forceinline__ int64_t wadd64(int64_t a, int64_t b) { return (int64_t)((uint64_t)a + (uint64_t)b); }
@@ -902,38 +908,6 @@ __device__ __forceinline__ void from_coding_order64(int64_t (&q)[64], const uint
      ...);
 }
 
-// 64 coefficients' low and high words -> pm[p] (bit p of coefficients
-// 0..31) and pm[64 + p] (32..63) for p = 0..63, and back.
-__device__ __forceinline__ void words_to_planes64(uint32_t (&lo)[64], uint32_t (&hi)[64], uint32_t *pm)
-{
-    to_planes32<0>(lo);
-    to_planes32<32>(lo);
-    to_planes32<0>(hi);
-    to_planes32<32>(hi);
-#pragma unroll
-    for (int p = 0; p < 32; ++p) {
-        pm[p] = lo[p];
-        pm[32 + p] = hi[p];
-        pm[64 + p] = lo[32 + p];
-        pm[96 + p] = hi[32 + p];
-    }
-}
-
-__device__ __forceinline__ void planes_to_words64(const uint32_t *pm, uint32_t (&lo)[64], uint32_t (&hi)[64])
-{
-#pragma unroll
-    for (int p = 0; p < 32; ++p) {
-        lo[p] = pm[p];
-        hi[p] = pm[32 + p];
-        lo[32 + p] = pm[64 + p];
-        hi[32 + p] = pm[96 + p];
-    }
-    from_planes32<0>(lo);
-    from_planes32<32>(lo);
-    from_planes32<0>(hi);
-    from_planes32<32>(hi);
-}
-
 __device__ __forceinline__ uint64_t umax64(uint64_t a, uint64_t b) { return a > b ? a : b; }
 
 __device__ __forceinline__ double pow2d(int k)  // k in [-1022, 1023]
@@ -974,13 +948,39 @@ __device__ __forceinline__ void encode_block64(const uint64_t (&v)[64], int word
     transform_fwd64(q);
     uint32_t lo[64], hi[64];
     to_coding_order64(lo, hi, q, std::make_integer_sequence<int, 64>{});
-    words_to_planes64(lo, hi, pm);
+    // the leading planes without a one, a group bit 0 each (up to 32 of them)
+    uint32_t any = 0u;
+#pragma unroll
+    for (int i = 0; i < 64; ++i)
+        any |= hi[i] ^ kNB;
+    const int skip = min(__clz((int)any), 32 * words - 12);
     dst[0] = 1u | ((uint32_t)(emax + 1023) << 1);
     dst[1] = 0u;
-    CodePos c{0, 12};
+    CodePos c{0, 12 + skip};
+    int p = 63 - skip;
+    // planes base + 15 .. base, whose masks are in a[at ..] and a[at + 32 ..]
+    auto code_part = [&](int base, const uint32_t (&a)[64], auto at_c) {
+        constexpr int at = decltype(at_c)::value;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            pm[i] = a[at + i];
+            pm[16 + i] = a[32 + at + i];
+        }
+        const uint32_t *pb = pm - base;
 #pragma unroll 1
-    for (int p = 63; p >= 0 && c.off < 32 * words; --p)
-        c = code_plane(dst, pm[p], pm[64 + p], c.n, c.off);
+        for (; p >= base && c.off < 32 * words; --p)
+            c = code_plane(dst, pb[p], pb[16 + p], c.n, c.off);
+    };
+    to_planes32<0>(hi);
+    to_planes32<32>(hi);
+    code_part(48, hi, std::integral_constant<int, 16>{});
+    code_part(32, hi, std::integral_constant<int, 0>{});
+    if (c.off < 32 * words) {
+        to_planes32<0>(lo);
+        to_planes32<32>(lo);
+        code_part(16, lo, std::integral_constant<int, 16>{});
+        code_part(0, lo, std::integral_constant<int, 0>{});
+    }
     clear_tail(dst, c.off, words);
 }
 
@@ -995,27 +995,62 @@ __device__ __forceinline__ void decode_block64(const uint32_t *w, int nwords, do
     }
     const int emax = (int)((w0 >> 1) & 0x7FFu) - 1023;
     const int budget = 32 * nwords;
-    int pos = 12, n = 0, p = 63;
+    // the leading planes without a one, a group bit 0 each (up to 20 of them)
+    const uint32_t lead = __funnelshift_r(w0, w[1], 12) | 0x100000u;
+    const int skip = min(__ffs((int)lead) - 1, budget - 12);
+    int pos = 12 + skip, n = 0, p = 63 - skip;
+    // planes base + 15 .. base into a[at ..] and a[at + 32 ..]
+    auto parse_part = [&](int base, uint32_t (&a)[64], auto at_c) {
+        constexpr int at = decltype(at_c)::value;
+        uint32_t *pb = pm - base;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            pm[i] = 0u;
 #pragma unroll 1
-    for (; p >= 0 && pos < budget; --p) {
-        const Plane r = parse_plane(w, nwords, n, pos);
-        pm[p] = r.xl;
-        pm[64 + p] = r.xh;
-        n = r.n;
-        pos = r.pos;
-    }
-    for (; p >= 0; --p) {  // planes past the budget
-        pm[p] = 0u;
-        pm[64 + p] = 0u;
-    }
+        for (; p >= base && pos < budget; --p) {
+            const Plane r = parse_plane(w, nwords, n, pos);
+            pb[p] = r.xl;
+            pb[16 + p] = r.xh;
+            n = r.n;
+            pos = r.pos;
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            a[at + i] = pm[i];
+            a[32 + at + i] = pm[16 + i];
+        }
+    };
     uint32_t lo[64], hi[64];
-    planes_to_words64(pm, lo, hi);
+    parse_part(48, hi, std::integral_constant<int, 16>{});
+    parse_part(32, hi, std::integral_constant<int, 0>{});
+    from_planes32<0>(hi);
+    from_planes32<32>(hi);
+    if (pos < budget) {
+        parse_part(16, lo, std::integral_constant<int, 16>{});
+        parse_part(0, lo, std::integral_constant<int, 0>{});
+        from_planes32<0>(lo);
+        from_planes32<32>(lo);
+    } else {  // the budget ended in the high planes
+#pragma unroll
+        for (int i = 0; i < 64; ++i)
+            lo[i] = kNB;
+    }
     int64_t q[64];
     from_coding_order64(q, lo, hi, std::make_integer_sequence<int, 64>{});
     transform_inv64(q);
-    // x = RN(RN(q) * 2^(emax - 58)): one exact or correctly rounded scaling
-    // (on the FP64 pipe: the same in integer arithmetic measured slower)
+    // x = RN(RN(q) * 2^(emax - 58)): one exact or correctly rounded scaling.
+    // Away from both ends of the range it is an addition to the exponent; the
+    // conversion stays on the FP64 pipe (16 clocks per warp each).
     const int k = emax - kPrec64;
+    if (k >= -1022 && k <= 960) {
+#pragma unroll
+        for (int i = 0; i < 64; ++i) {
+            const double f = __ll2double_rn((long long)q[i]);
+            const int h = __double2hiint(f);
+            out[i] = __hiloint2double(h != 0 ? h + (k << 20) : 0, __double2loint(f));
+        }
+        return;
+    }
     const bool split = k < -1022;
     const double sa = pow2d(split ? k + 64 : k), sb = pow2d(-64);
 #pragma unroll
@@ -1027,7 +1062,7 @@ __device__ __forceinline__ void decode_block64(const uint32_t *w, int nwords, do
     }
 }
 
-__global__ void __launch_bounds__(kThreads64) fr4d_encode_kernel(DConstRing in, int64_t nx, int64_t ny, int64_t z0,
+__global__ void __launch_bounds__(kThreads64, 6) fr4d_encode_kernel(DConstRing in, int64_t nx, int64_t ny, int64_t z0,
                                                                  int64_t nblk, int rate, uint32_t *__restrict__ out)
 {
     extern __shared__ uint32_t smem[];  // each thread's block, then each thread's planes
@@ -1054,13 +1089,13 @@ __global__ void __launch_bounds__(kThreads64) fr4d_encode_kernel(DConstRing in, 
                 v[16 * k + 4 * j + 2] = (uint64_t)__double_as_longlong(c.x);
                 v[16 * k + 4 * j + 3] = (uint64_t)__double_as_longlong(c.y);
             }
-        encode_block64(v, words, mine, smem + kThreads64 * stride + threadIdx.x * kPlaneStride64);
+        encode_block64(v, words, mine, smem + kThreads64 * stride + threadIdx.x * kHalfStride);
     }
     store_blocks(out + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
                  mine - (threadIdx.x & 31) * stride);
 }
 
-__global__ void __launch_bounds__(kThreads64) fr4d_decode_kernel(const uint32_t *__restrict__ in, int64_t nx,
+__global__ void __launch_bounds__(kThreads64, 7) fr4d_decode_kernel(const uint32_t *__restrict__ in, int64_t nx,
                                                                  int64_t ny, int64_t z0, int64_t nblk, int rate,
                                                                  DRing out)
 {
@@ -1076,7 +1111,7 @@ __global__ void __launch_bounds__(kThreads64) fr4d_decode_kernel(const uint32_t 
     if (b >= nblk)
         return;
     double f[64];
-    decode_block64(mine, words, f, smem + kThreads64 * stride + threadIdx.x * kPlaneStride64);
+    decode_block64(mine, words, f, smem + kThreads64 * stride + threadIdx.x * kHalfStride);
     const int64_t nbx = nx >> 2, nby = ny >> 2;
     const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
     const int64_t slot = ring_slot(z0 + 4 * bz, out.zbase, out.nslot);
@@ -1094,8 +1129,8 @@ __global__ void __launch_bounds__(kThreads64) fr4d_decode_kernel(const uint32_t 
 size_t smem_bytes64(int rate, bool encoder)
 {
     if (!encoder)
-        return (size_t)kThreads64 * (decode_stride(2 * rate) + kPlaneStride64) * sizeof(uint32_t);
-    return (size_t)kThreads64 * (encode_stride(2 * rate) + kPlaneStride64) * sizeof(uint32_t);
+        return (size_t)kThreads64 * (decode_stride(2 * rate) + kHalfStride) * sizeof(uint32_t);
+    return (size_t)kThreads64 * (encode_stride(2 * rate) + kHalfStride) * sizeof(uint32_t);
 }
 
 cudaError_t ensure_smem_attr64()
