@@ -70,9 +70,13 @@ constexpr int kX2tNW = OOC_HEATX2T_NW;
 using X2t = X2tShape<kX2tR, kX2tNW>;
 // 5 stages and 3 CTAs per SM (72 KB of shared memory and at most 85
 // registers each), loop unrolled 3 times (the z-queues rotate without
-// copies).  In the 1024^3 FR4-16 pipeline (56-plane windows), per launch:
-// 110.4 us; 112.4 us not unrolled; 6 stages and 2 CTAs per SM 128.6 us
-// (120.6 us unrolled); heat7x2r_kernel 146.2 us.
+// copies).  Bound by instruction issue and the plane barrier (issue 65 %
+// active, 51-54 % of DRAM).  56 planes of 1024^2, us per launch: 98.7; with
+// planes outside the grid tested for instead of copied as zeros 104.7 (13 %
+// more instructions in the loop); 4 stages 100.5; unrolled 4 and 6 times 102.5
+// and 98.5; 6 stages and 2 CTAs per SM 118.9; a check of the tile's position
+// in place of the select after level s 101.5.  512^3: 217.8, with 120-column
+// tiles and the tests 256.
 #ifndef OOC_HEATX2T_NS
 #define OOC_HEATX2T_NS 5
 #endif
@@ -85,10 +89,25 @@ using X2t = X2tShape<kX2tR, kX2tNW>;
 constexpr int kX2tNS = OOC_HEATX2T_NS;
 size_t heat7x2t_smem_bytes()
 {
-    return (size_t)kX2tNS * X2t::stage_floats * 4 + 3 * (size_t)X2t::l1_float4 * 16 + kX2tNS * 8;
+    return (size_t)kX2tNS * X2t::stage_floats * 4 + 3 * (size_t)X2t::l1_float4 * 16 + kX2tNS * 8 +
+           3 * (size_t)X2t::rows * 2 * 4;
 }
 
-template <int NS, int R, int NW>
+// Tile widths.  EDGE = false: a warp's 128 level-s columns give 120 columns of
+// level s+1, four fewer on each side.  EDGE = true: 128 columns; level s of the
+// two columns beside the tile is computed point by point, 32 points a plane,
+// by one warp in turn.  That costs about a tenth more per tile, so it is for
+// widths where it saves an eighth of the tiles: 512 columns take 4 tiles
+// instead of 5 (us per pair, 120 and 128: 512^3 256 and 232; 384^3 118 and 109),
+// 1024 take 8 instead of 9 (56 planes of 1024^2: 105 and 107).
+template <bool EDGE>
+__host__ __device__ constexpr int64_t x2t_tiles(int64_t nx)
+{
+    return EDGE ? (nx + kSeg - 1) / kSeg : (nx + kSeg - 9) / (kSeg - 8);
+}
+inline bool x2t_edge(int64_t nx) { return 8 * x2t_tiles<true>(nx) <= 7 * x2t_tiles<false>(nx); }
+
+template <int NS, int R, int NW, bool EDGE>
 __global__ void __launch_bounds__(kTX *NW, OOC_HEATX2T_MINB)
     heat7x2t_kernel(const __grid_constant__ CUtensorMap tin, float *__restrict__ out, int nslot, int64_t zbase,
                     Grid3 g, int64_t z0, int64_t z1, int64_t ntiles, int64_t nfull, int64_t zchunk, int64_t lo64,
@@ -102,6 +121,7 @@ __global__ void __launch_bounds__(kTX *NW, OOC_HEATX2T_MINB)
     float4 *l1 = reinterpret_cast<float4 *>(smem_raw + (size_t)NS * S::stage_floats * 4);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + (size_t)NS * S::stage_floats * 4 +
                                                  3 * (size_t)S::l1_float4 * 16);
+    float *l1x = reinterpret_cast<float *>(bar + NS);  // [3][rows][2]
     const int lane = threadIdx.x, w = threadIdx.y;
     const bool leader = lane == 0 && w == 0;
     int64_t tile, zs64, ze64;
@@ -115,8 +135,8 @@ __global__ void __launch_bounds__(kTX *NW, OOC_HEATX2T_MINB)
         zs64 = z0 + (j / rest) * zchunk;
         ze64 = min(zs64 + zchunk, z1);
     }
-    const int64_t gx = (g.nx + kSeg - 9) / (kSeg - 8);  // x tiles; tile = by * gx + bx
-    const int64_t xs = (tile % gx) * (kSeg - 8) - 4;     // first level-s column
+    const int64_t gx = x2t_tiles<EDGE>(g.nx);  // x tiles; tile = by * gx + bx
+    const int64_t xs = EDGE ? (tile % gx) * kSeg : (tile % gx) * (kSeg - 8) - 4;  // first level-s column
     const int64_t x4 = xs + 4 * lane;
     const int64_t y0 = (tile / gx) * TYO;
     const int L0 = R * w;  // this warp's first level-s row in the tile (row y0 - 1 + L0)
@@ -125,7 +145,7 @@ __global__ void __launch_bounds__(kTX *NW, OOC_HEATX2T_MINB)
     const int zs = (int)zs64, ze = (int)ze64;
     const int64_t plane = g.plane;
     const bool xin = x4 >= 0 && x4 < g.nx;
-    const bool lin = lane >= 1 && lane <= kTX - 2;
+    const bool lin = EDGE || (lane >= 1 && lane <= kTX - 2);
     bool in[R], own[R];
     int64_t off[R];
 #pragma unroll
@@ -136,6 +156,14 @@ __global__ void __launch_bounds__(kTX *NW, OOC_HEATX2T_MINB)
         own[j] = in[j] && lin && L0 + j >= 1 && L0 + j <= S::rows - 2;  // level s+1 stored here
     }
     const float4 z4 = zero4();
+    // the point beside the tile that this lane takes when its warp's turn
+    // comes: row lane / 2, left or right
+    static_assert(!EDGE || 2 * S::rows == kTX, "one lane per point beside the tile");
+    const int64_t hx = (lane & 1) ? xs + kSeg : xs - 1, hy = y0 - 1 + (lane >> 1);
+    const bool hin = hx >= 0 && hx < g.nx && hy >= 0 && hy < g.ny;
+    const int64_t hoff = hin ? hy * g.nx + hx : 0;
+    const int hat = ((lane >> 1) + 1) * S::scols + ((lane & 1) ? kSeg + 4 : 3);
+    const bool xedge = lane == 0 || lane == kTX - 1;
 
     // staged planes zs-2 .. ze+1: stage index i holds plane zs - 2 + i in
     // slot i mod NS, completing phase (i / NS) of that slot's mbarrier
@@ -146,12 +174,9 @@ __global__ void __launch_bounds__(kTX *NW, OOC_HEATX2T_MINB)
     int islot = (int)ring_slot(zfirst, zbase, nslot);
     auto issue = [&](int i) {  // copies plane zfirst + i; i advances by one per call
         const int zp = zfirst + i, sl = i % NS;
-        if (zp >= 0 && zp < nz) {
-            mbar_arrive_tx(&bar[sl], (unsigned)S::copy_bytes);
-            tma_load_3d(stages + sl * S::stage_floats, &tin, tx, ty, islot, &bar[sl]);
-        } else {
-            mbar_arrive(&bar[sl]);  // a plane outside the grid: nothing to copy, the phase completes at once
-        }
+        // a plane outside the grid is the out-of-range slot nslot: zeros
+        mbar_arrive_tx(&bar[sl], (unsigned)S::copy_bytes);
+        tma_load_3d(stages + sl * S::stage_floats, &tin, tx, ty, zp >= 0 && zp < nz ? islot : nslot, &bar[sl]);
         islot = wrap_add(islot, 1, nslot);
     };
     if (leader) {
@@ -174,17 +199,17 @@ __global__ void __launch_bounds__(kTX *NW, OOC_HEATX2T_MINB)
     unsigned fail = 0;
     fail |= mbar_wait(&bar[0], 0) ? 0u : 1u;
     fail |= mbar_wait(&bar[1 % NS], (1 / NS) & 1) ? 0u : 1u;
-    // level s-1 queue z-1, z, z+1 of the thread's rows (zero outside the
-    // grid: the copies fill zeros there, and planes outside are not read)
+    // level s-1 queue z-1, z, z+1 of the thread's rows (the copies fill zeros
+    // outside the grid)
     float4 pq[R], cq[R], s2[R], s1[R];
 #pragma unroll
     for (int j = 0; j < R; ++j) {
-        pq[j] = (!fail && zfirst >= 0) ? s4(0, L0 + j + 1) : z4;
-        cq[j] = (!fail && zfirst + 1 >= 0 && zfirst + 1 < nz) ? s4(1 % NS, L0 + j + 1) : z4;
+        pq[j] = s4(0, L0 + j + 1);
+        cq[j] = s4(1 % NS, L0 + j + 1);
         s2[j] = z4;  // level s at planes z-2, z-1
         s1[j] = z4;
     }
-    int sc = 1 % NS, sn = 2 % NS;                      // stages of planes z and z+1
+    int sp = 0, sc = 1 % NS, sn = 2 % NS;              // stages of planes z-1, z and z+1
     int l1c = 0;                                       // level-s ring plane of z
     int oslot = (int)ring_slot(zs - 2, zbase, nslot);  // output ring slot of plane z-1
 OOC_PRAGMA(unroll OOC_HEATX2T_UNROLL)
@@ -193,10 +218,28 @@ OOC_PRAGMA(unroll OOC_HEATX2T_UNROLL)
         if (!mbar_wait(&bar[sn], (unsigned)(((i + 1) / NS) & 1)))
             fail = 1u;
         float4 nq[R], sv[R];
+        float ye[R];  // level s of plane z-1 beside the tile (edge lanes)
+        const int lp = l1c == 0 ? 2 : l1c - 1;
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+            ye[j] = EDGE && xedge ? l1x[(lp * S::rows + L0 + j) * 2 + (lane & 1)] : 0.0f;
 #pragma unroll
         for (int j = 0; j < R; ++j) {
-            nq[j] = z + 1 < nz ? s4(sn, L0 + j + 1) : z4;
+            nq[j] = s4(sn, L0 + j + 1);
             sv[j] = z4;
+        }
+        // level s on the columns beside the tile: the warps take turns
+        if (EDGE && w == (i & (NW - 1))) {
+            float v = 0.0f;
+            if (hin) {
+                const float *pc = stages + sc * S::stage_floats + hat;
+                if (z >= lo && z < hi)
+                    v = heat_pt(pc[0], pc[-1], pc[1], pc[-S::scols], pc[S::scols],
+                                stages[sp * S::stage_floats + hat], stages[sn * S::stage_floats + hat], r);
+                else if (band_in != nullptr && z >= bin_lo && z < bin_lo + 2)
+                    v = __ldg(band_in + (int64_t)(z - bin_lo) * plane + hoff);
+            }
+            l1x[l1c * 2 * S::rows + lane] = v;
         }
         // level s at plane z (z is uniform over the CTA); a row's neighbours
         // on the thread's other rows come from registers
@@ -250,14 +293,17 @@ OOC_PRAGMA(unroll OOC_HEATX2T_UNROLL)
         }
         // level s+1 at plane z-1 from level s at planes z-2, z-1, z
         if (z - 1 >= zs) {
-            const int lp = l1c == 0 ? 2 : l1c - 1;
             const float4 upo = w >= 1 ? l1[lp * S::l1_float4 + (L0 - 1) * kTX + lane] : z4;
             const float4 dno = w <= NW - 2 ? l1[lp * S::l1_float4 + (L0 + R) * kTX + lane] : z4;
             float *op = out + (int64_t)oslot * plane;
 #pragma unroll
             for (int j = 0; j < R; ++j) {
-                const float yl = __shfl_up_sync(0xffffffffu, s1[j].w, 1);
-                const float yr = __shfl_down_sync(0xffffffffu, s1[j].x, 1);
+                float yl = __shfl_up_sync(0xffffffffu, s1[j].w, 1);
+                float yr = __shfl_down_sync(0xffffffffu, s1[j].x, 1);
+                if (EDGE && lane == 0)
+                    yl = ye[j];
+                if (EDGE && lane == kTX - 1)
+                    yr = ye[j];
                 const float4 o = OOC_HEATX2T_PT(s1[j], yl, yr, j == 0 ? upo : s1[j - 1], j == R - 1 ? dno : s1[j + 1],
                                           s2[j], sv[j], r);
                 if (own[j])
@@ -271,6 +317,7 @@ OOC_PRAGMA(unroll OOC_HEATX2T_UNROLL)
             pq[j] = cq[j];
             cq[j] = nq[j];
         }
+        sp = sc;
         sc = sn;
         sn = sn + 1 == NS ? 0 : sn + 1;
         l1c = l1c == 2 ? 0 : l1c + 1;
@@ -368,16 +415,22 @@ cudaError_t launch_heat7x2(ConstRing in, Ring out, int64_t nx, int64_t ny, int64
     constexpr int NW = kX2tNW;
     constexpr int TYO = X2t::tyo;
     const size_t smem = heat7x2t_smem_bytes();
-    // set once (thread-safe); 0 if the attribute could not be set
+    // resident CTAs of both kernels; set once (thread-safe), 0 if an attribute
+    // could not be set
     static const int res = [smem]() -> int {
-        if (cudaFuncSetAttribute(heat7x2t_kernel<kX2tNS, kX2tR, kX2tNW>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return 0;
-        return resident((const void *)heat7x2t_kernel<kX2tNS, kX2tR, kX2tNW>, kTX * NW, smem);
+        int n = 0;
+        for (const void *fn : {(const void *)heat7x2t_kernel<kX2tNS, kX2tR, kX2tNW, false>,
+                               (const void *)heat7x2t_kernel<kX2tNS, kX2tR, kX2tNW, true>}) {
+            if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+                return 0;
+            n = resident(fn, kTX * NW, smem);
+        }
+        return n;
     }();
     if (res <= 0)
         return cudaErrorInvalidValue;
-    const int64_t gx = (nx + kSeg - 9) / (kSeg - 8), gy = (ny + TYO - 1) / TYO;
+    const bool edge = x2t_edge(nx);
+    const int64_t gx = edge ? x2t_tiles<true>(nx) : x2t_tiles<false>(nx), gy = (ny + TYO - 1) / TYO;
     const int64_t chunk = choose_chunk(gx * gy, z1 - z0, 8, 5, res);
     if (in.nslot != out.nslot || in.zbase != out.zbase || in.nslot > (1ll << 30) || in.base == out.base ||
         gx * gy > 0x7fffffffll || nz > (1ll << 30))
@@ -385,17 +438,19 @@ cudaError_t launch_heat7x2(ConstRing in, Ring out, int64_t nx, int64_t ny, int64
     const FusedGrid fg = fused_grid(gx * gy, z1 - z0, chunk, res);
     if (fg.ncta > 0x7fffffffll)
         return cudaErrorInvalidValue;
-    // the TMA x coordinate (first column - 8) is a multiple of 4 floats:
-    // tiles start at multiples of 120; ring strides are multiples of 16 bytes
+    // the TMA x coordinate (the tile's first column - 4) is a multiple of 4
+    // floats; ring strides are multiples of 16 bytes
     if (nx % 4 || ((uintptr_t)in.base % 16) || nx > 0x7fffffffll || ny > 0x7fffffffll)
         return cudaErrorInvalidValue;
     CUtensorMap map;
     cudaError_t e = ring_tensor_map(in.base, nx, ny, in.nslot, X2t::scols, X2t::srows, &map);
     if (e != cudaSuccess)
         return e;
-    heat7x2t_kernel<kX2tNS, kX2tR, kX2tNW><<<(unsigned)fg.ncta, dim3(kTX, NW), smem, st>>>(
-        map, out.base, (int)in.nslot, in.zbase, Grid3{nx, ny, nz, nx * ny}, z0, z1, gx * gy, fg.nfull, fg.zch, lo, hi,
-        band_in, bin_lo, band_out, bout_lo, r);
+    const auto kernel = edge ? heat7x2t_kernel<kX2tNS, kX2tR, kX2tNW, true>
+                             : heat7x2t_kernel<kX2tNS, kX2tR, kX2tNW, false>;
+    kernel<<<(unsigned)fg.ncta, dim3(kTX, NW), smem, st>>>(map, out.base, (int)in.nslot, in.zbase,
+                                                           Grid3{nx, ny, nz, nx * ny}, z0, z1, gx * gy, fg.nfull,
+                                                           fg.zch, lo, hi, band_in, bin_lo, band_out, bout_lo, r);
     return cudaGetLastError();
 #endif
 }
