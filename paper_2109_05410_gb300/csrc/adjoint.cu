@@ -173,11 +173,12 @@ __global__ void __launch_bounds__(kTX *kTY, 2)
 __global__ void gather_kernel(const float *__restrict__ f, int64_t size, const int64_t *__restrict__ idx, int64_t n,
                               float *__restrict__ out)
 {
+    pdl_begin();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
-        const int64_t j = idx[i];
+        const int64_t j = __ldca(idx + i);
         if (j >= 0 && j < size) {
-            out[i] = f[j];
+            out[i] = __ldca(f + j);
         } else {
             out[i] = 0.0f;
             atomicOr(&g_index_fault, 1u);
@@ -203,11 +204,12 @@ __global__ void scatter_add_kernel(float *f, int64_t size, const int64_t *__rest
 __global__ void scatter_add_scaled_kernel(float *f, int64_t size, const int64_t *__restrict__ idx, int64_t n,
                                           const float *__restrict__ v, const float *__restrict__ kap)
 {
+    pdl_begin();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
-        const int64_t j = idx[i];
+        const int64_t j = __ldca(idx + i);
         if (j >= 0 && j < size)
-            f[j] += v[i] * kap[j];
+            f[j] += __ldca(v + i) * __ldca(kap + j);
         else
             atomicOr(&g_index_fault, 1u);
     }
@@ -509,13 +511,13 @@ ooc_status ooc_wave25_forward_ckpt(const float *d_kappa, int64_t nx, int64_t ny,
             TRY_CUDA(cudaEventRecord(ev.e[2 + bi], sD));
         }
         TRY_CUDA(launch_wave25(ConstRing{p, nz, 0}, Ring{pp, nz, 0}, ConstRing{d_kappa, nz, 0}, nx, ny, nz, 0, nz,
-                               src ? sx : -1, sy, sz, src ? h_w[s] : 0.0f, sC));
+                               src ? sx : -1, sy, sz, src ? h_w[s] : 0.0f, sC, WaveSrcTable{}, true));
         float *t = p;  // pp now holds p^{s+1}
         p = pp;
         pp = t;
         if (nrec > 0)
-            TRY_CUDA(ooc_gather(p, n, d_rec, nrec, d_traces + s * nrec, sC) == OOC_OK ? cudaSuccess
-                                                                                     : cudaErrorUnknown);
+            TRY_CUDA(launch(true, gather_kernel, dim3((unsigned)((nrec + 255) / 256)), dim3(256), 0, sC, p, n, d_rec, nrec,
+                            d_traces + s * nrec));
     }
     TRY_CUDA(cudaEventRecord(ev.e[4], sC));
     TRY_CUDA(cudaEventRecord(ev.e[5], sD));
@@ -591,16 +593,16 @@ ooc_status ooc_wave25_backward_ckpt(const float *d_kappa, int64_t nx, int64_t ny
             const int64_t s = n0 + j - 1;
             TRY_CUDA(launch_wave25_to(ConstRing{hist(j), nz, 0}, ConstRing{hist(j - 1), nz, 0}, Ring{hist(j + 1), nz, 0},
                                       ConstRing{d_kappa, nz, 0}, nx, ny, nz, 0, nz, src ? sx : -1, sy, sz,
-                                      src ? h_w[s] : 0.0f, sC));
+                                      src ? h_w[s] : 0.0f, sC, WaveSrcTable{}, true));
         }
         // adjoint through the segment, on w = kappa mu (mu1 / mu2 hold w)
         for (int64_t m = n1; m >= n0 + 1; --m) {
             TRY_CUDA(launch_wave25_to(ConstRing{mu1, nz, 0}, ConstRing{mu2, nz, 0}, Ring{mu2, nz, 0},
-                                      ConstRing{d_kappa, nz, 0}, nx, ny, nz, 0, nz, -1, -1, -1, 0.0f, sC));
+                                      ConstRing{d_kappa, nz, 0}, nx, ny, nz, 0, nz, -1, -1, -1, 0.0f, sC,
+                                      WaveSrcTable{}, true));
             if (nrec > 0) {  // + kappa S^T res[m-1]
-                scatter_add_scaled_kernel<<<(unsigned)((nrec + 255) / 256), 256, 0, sC>>>(
-                    mu2, n, d_rec, nrec, d_res + (m - 1) * nrec, d_kappa);
-                TRY_CUDA(cudaGetLastError());
+                TRY_CUDA(launch(true, scatter_add_scaled_kernel, dim3((unsigned)((nrec + 255) / 256)), dim3(256), 0, sC,
+                                mu2, n, d_rec, nrec, d_res + (m - 1) * nrec, d_kappa));
             }
             // += w^m L(p^{m-1}), in FP32 within the segment
             TRY_CUDA(launch_wave25_grad32(hist(m - n0), mu2, gacc, nx, ny, nz, sC));

@@ -101,6 +101,37 @@ __global__ void bf16_unpack_flat(const uint16_t *in, float *out, int64_t n)
             out[j] = __uint_as_float((uint32_t)in[j] << 16);
 }
 
+// nsteps heat7 steps in place on d_u.  Pairs of steps in one launch where one
+// pair takes less time than two steps, that is on all grids but small ones
+// (us per pair and per two steps: 512^3 218 and 340, 256^3 39 and 53; at
+// 192^3 and below single steps are faster, 28 and 19).  The launches alternate
+// between the two fields, so their number is made even by running up to three
+// steps singly (10 steps of 512^3: 4 pairs and 2 steps, no copy back).
+ooc_status heat7_run(float *d_u, float *d_tmp, int64_t nx, int64_t ny, int64_t nz, float r, int64_t nsteps,
+                     cudaStream_t st)
+{
+    int64_t pairs = heat7_small(nx, ny, nz) ? 0 : nsteps / 2;
+    if (pairs > 0 && ((nsteps - pairs) & 1))
+        --pairs;
+    float *a = d_u, *b = d_tmp;
+    for (int64_t s = 0, j = 0; s < nsteps; ++j) {
+        const bool pair = j < pairs;
+        const cudaError_t e =
+            pair ? launch_heat7x2(ConstRing{a, nz, 0}, Ring{b, nz, 0}, nx, ny, nz, 0, nz, 0, nz, nullptr, 0, nullptr, 0, r,
+                                  st)
+                 : launch_heat7(ConstRing{a, nz, 0}, Ring{b, nz, 0}, nx, ny, nz, 0, nz, r, st, true);
+        if (e != cudaSuccess)
+            return OOC_E_CUDA;
+        s += pair ? 2 : 1;
+        float *t = a;
+        a = b;
+        b = t;
+    }
+    if (a != d_u)
+        return cuda_status(cudaMemcpyAsync(d_u, a, sizeof(float) * nx * ny * nz, cudaMemcpyDeviceToDevice, st));
+    return OOC_OK;
+}
+
 unsigned flat_grid(int64_t n)
 {
     int64_t b = (n / 4 + 255) / 256;
@@ -307,19 +338,7 @@ ooc_status ooc_heat7_steps(float *d_u, float *d_tmp, int64_t nx, int64_t ny, int
     if (!d_u || !d_tmp || d_u == d_tmp || !dims_ok(nx, ny, nz) || nsteps < 0 || !aligned(d_u, 16) ||
         !aligned(d_tmp, 16))
         return OOC_E_INVALID;
-    cudaStream_t st = (cudaStream_t)stream;
-    float *a = d_u, *b = d_tmp;
-    for (int64_t s = 0; s < nsteps; ++s) {
-        cudaError_t e = launch_heat7(ConstRing{a, nz, 0}, Ring{b, nz, 0}, nx, ny, nz, 0, nz, (float)r, st);
-        if (e != cudaSuccess)
-            return OOC_E_CUDA;
-        float *t = a;
-        a = b;
-        b = t;
-    }
-    if (a != d_u)
-        return cuda_status(cudaMemcpyAsync(d_u, a, sizeof(float) * nx * ny * nz, cudaMemcpyDeviceToDevice, st));
-    return OOC_OK;
+    return heat7_run(d_u, d_tmp, nx, ny, nz, (float)r, nsteps, (cudaStream_t)stream);
 }
 
 ooc_status ooc_heat7_steps_f64(double *d_u, double *d_tmp, int64_t nx, int64_t ny, int64_t nz, double r,
@@ -345,25 +364,7 @@ ooc_status ooc_heat7_steps_f64(double *d_u, double *d_tmp, int64_t nx, int64_t n
 ooc_status ooc_heat7_steps_fused(float *d_u, float *d_tmp, int64_t nx, int64_t ny, int64_t nz, double r,
                                  int64_t nsteps, void *stream)
 {
-    if (!d_u || !d_tmp || !dims_ok(nx, ny, nz) || nsteps < 0 || d_u == d_tmp || !aligned(d_u, 16) ||
-        !aligned(d_tmp, 16))
-        return OOC_E_INVALID;
-    cudaStream_t st = (cudaStream_t)stream;
-    float *a = d_u, *b = d_tmp;
-    for (int64_t s = 0; s < nsteps; s += 2) {
-        cudaError_t e = s + 2 <= nsteps
-                            ? launch_heat7x2(ConstRing{a, nz, 0}, Ring{b, nz, 0}, nx, ny, nz, 0, nz, 0, nz, nullptr, 0,
-                                             nullptr, 0, (float)r, st)
-                            : launch_heat7(ConstRing{a, nz, 0}, Ring{b, nz, 0}, nx, ny, nz, 0, nz, (float)r, st);
-        if (e != cudaSuccess)
-            return OOC_E_CUDA;
-        float *t = a;
-        a = b;
-        b = t;
-    }
-    if (a != d_u)
-        return cuda_status(cudaMemcpyAsync(d_u, a, sizeof(float) * nx * ny * nz, cudaMemcpyDeviceToDevice, st));
-    return OOC_OK;
+    return ooc_heat7_steps(d_u, d_tmp, nx, ny, nz, r, nsteps, stream);
 }
 
 ooc_status ooc_wave25_steps(float *d_p, float *d_pprev, const float *d_kappa, int64_t nx, int64_t ny, int64_t nz,
@@ -379,7 +380,7 @@ ooc_status ooc_wave25_steps(float *d_p, float *d_pprev, const float *d_kappa, in
         const bool src = sx >= 0 && h_w != nullptr;
         const float w = src ? h_w[t + s] : 0.0f;
         cudaError_t e = launch_wave25(ConstRing{a, nz, 0}, Ring{b, nz, 0}, ConstRing{d_kappa, nz, 0}, nx, ny, nz, 0,
-                                      nz, src ? sx : -1, sy, sz, w, st);
+                                      nz, src ? sx : -1, sy, sz, w, st, WaveSrcTable{}, true);
         if (e != cudaSuccess)
             return OOC_E_CUDA;
         float *tmp = a;  // b now holds p^{n+1}

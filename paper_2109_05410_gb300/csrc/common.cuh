@@ -42,6 +42,41 @@ __host__ __device__ inline int64_t ring_slot(int64_t z, int64_t zbase, int64_t n
     return s < 0 ? s + nslot : s;
 }
 
+// Programmatic dependent launch, for the step loops of the in-core calls.  A
+// kernel launched with `pdl` may start while the kernel before it in the stream
+// still runs, so its first statement is pdl_begin(), in every block and before
+// any early return: it lets the next kernel start in turn (once all blocks of
+// this one have) and waits until the kernels before have completed and their
+// writes are visible.  What overlaps is the launch itself: between two
+// dependent kernels without it the GPU idles for up to 2.05 us (kernel starts
+// fall on a grid of about that step; a 64^3 heat7 step takes 4.17 us without
+// and 2.4 us with it).  Such a kernel must not read through the non-coherent
+// path (__ldg, or a const __restrict__ pointer's plain loads): that is for data
+// that nothing writes while the kernel is resident, and a block that waits is.
+// Its loads are __ldca or copies through L2 (cp.async of 16 bytes).
+__device__ __forceinline__ void pdl_begin()
+{
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+}
+
+template <typename... P, typename... A>
+cudaError_t launch(bool pdl, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // Stencil coefficients of the 8th-order central second difference.
 constexpr float kC0 = -205.0f / 72.0f;
 constexpr float kC1 = 8.0f / 5.0f;
@@ -60,8 +95,12 @@ struct WaveSrcTable {
 
 // Kernel launchers (stream-ordered, no synchronisation).  All return
 // cudaGetLastError() of the launch.
+// `pdl`: see launch().
 cudaError_t launch_heat7(ConstRing in, Ring out, int64_t nx, int64_t ny, int64_t nz, int64_t z0, int64_t z1,
-                         float r, cudaStream_t st);
+                         float r, cudaStream_t st, bool pdl = false);
+// Whether launch_heat7 runs a window of this size without a march (see
+// heat7_direct_kernel).
+bool heat7_small(int64_t nx, int64_t ny, int64_t nplanes);
 // g[i] += (double) mu[i] * (double) L(p)[i] over whole dense fields (the
 // 25-point Laplacian without kappa); g 32-byte aligned.
 cudaError_t launch_wave25_grad(const float *p, const float *mu, double *g, int64_t nx, int64_t ny, int64_t nz,
@@ -96,11 +135,11 @@ cudaError_t launch_wave25_f64(DConstRing p, DRing pprev_out, DConstRing kappa, i
                               WaveSrcTable tab = WaveSrcTable{});
 cudaError_t launch_wave25(ConstRing p, Ring pprev_out, ConstRing kappa, int64_t nx, int64_t ny, int64_t nz,
                           int64_t z0, int64_t z1, int64_t sx, int64_t sy, int64_t sz, float w, cudaStream_t st,
-                          WaveSrcTable tab = WaveSrcTable{});
+                          WaveSrcTable tab = WaveSrcTable{}, bool pdl = false);
 // Same step with p_prev read from `pprev` and p' written to `pnew` (may alias).
 cudaError_t launch_wave25_to(ConstRing p, ConstRing pprev, Ring pnew, ConstRing kappa, int64_t nx, int64_t ny,
                              int64_t nz, int64_t z0, int64_t z1, int64_t sx, int64_t sy, int64_t sz, float w,
-                             cudaStream_t st, WaveSrcTable tab = WaveSrcTable{});
+                             cudaStream_t st, WaveSrcTable tab = WaveSrcTable{}, bool pdl = false);
 // Reads and clears the device word that a stencil kernel sets when one of
 // its bounded waits gives up (nonzero: that launch left planes unwritten).
 cudaError_t take_stencil_fault(unsigned *fault);

@@ -113,7 +113,7 @@ extern "C" ooc_status ooc_heat7_steps_noalloc(float *d_u, int64_t nx, int64_t ny
     cudaStream_t st = (cudaStream_t)stream;
     float *a = d_u, *b = tmp;
     for (int64_t i = 0; i < nsteps; ++i) {
-        if (launch_heat7(ConstRing{a, nz, 0}, Ring{b, nz, 0}, nx, ny, nz, 0, nz, (float)r, st) != cudaSuccess)
+        if (launch_heat7(ConstRing{a, nz, 0}, Ring{b, nz, 0}, nx, ny, nz, 0, nz, (float)r, st, true) != cudaSuccess)
             return OOC_E_CUDA;
         float *t = a;
         a = b;

@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(kTX *kHeatTY)
                  int64_t z0, int64_t z1, int64_t zchunk, float r)
 {
     __shared__ float4 tile[2][kHeatTY + 2][kTX];
+    pdl_begin();
     const int lane = threadIdx.x, ty = threadIdx.y;
     const int64_t gx = (g.nx + kSeg - 1) / kSeg;  // x tiles; blockIdx.x = by * gx + bx
     const int64_t xs = (int64_t)(blockIdx.x % gx) * kSeg;
@@ -115,8 +116,8 @@ __global__ void __launch_bounds__(kTX *kHeatTY)
     float4 nn = (inside && za + 2 < nz) ? ldg4(p2 + off) : z4;
     float4 hyv = (hrow && za < nz) ? ldg4(p0 + hoff) : z4;
     float4 hyv1 = (hrow && za + 1 < nz) ? ldg4(p1 + hoff) : z4;
-    float hx = (hcol && za < nz) ? __ldg(p0 + xoff) : 0.f;
-    float hx1 = (hcol && za + 1 < nz) ? __ldg(p1 + xoff) : 0.f;
+    float hx = (hcol && za < nz) ? __ldca(p0 + xoff) : 0.f;
+    float hx1 = (hcol && za + 1 < nz) ? __ldca(p1 + xoff) : 0.f;
     int64_t z = za;
     // unrolled twice so that the register queue rotates by renaming
 OOC_PRAGMA(unroll OOC_HEAT_UNROLL)
@@ -127,7 +128,7 @@ OOC_PRAGMA(unroll OOC_HEAT_UNROLL)
         const float4 pfv = (inside && z + 3 < nz) ? ldg4(q3 + off) : z4;
         const bool v2 = z + 2 < nz;
         const float4 hyv2 = (hrow && v2) ? ldg4(q2 + hoff) : z4;
-        const float hx2 = (hcol && v2) ? __ldg(q2 + xoff) : 0.f;
+        const float hx2 = (hcol && v2) ? __ldca(q2 + xoff) : 0.f;
 
         const int b = i & 1;
         tile[b][ty + 1][lane] = cur;
@@ -159,6 +160,74 @@ OOC_PRAGMA(unroll OOC_HEAT_UNROLL)
     }
 }
 
+
+// One heat7 step without a march: a thread owns four consecutive x points of
+// ZR consecutive planes and reads their neighbours straight from memory (x
+// from the adjacent lanes), all loads at once.  The rows that neighbouring
+// threads read again come from L1 and L2, so this is for windows that L2
+// holds, where the march's chain of planes is what takes the time.
+//
+// Up to kHeatDirectMax points (88 MiB for both levels: L2 holds them): us per
+// step, march and direct, both with overlapped launches: 64^3 6.2 and 2.4,
+// 128^3 8.3 and 3.7, 192^3 16.4 and 9.6; 256^3 26.4 and 27.2, 512^3 170 and
+// 197.  ZR = 4: at 128^3 2 takes 4.4 and 8 the same as 4, at 192^3 12.0 and
+// 13.8 against 9.6.
+constexpr int kHeatZR = 4;
+constexpr int64_t kHeatDirectMax = 11ll << 20;
+__global__ void __launch_bounds__(256)
+    heat7_direct_kernel(const float *__restrict__ in, float *__restrict__ out, int nslot, int64_t zbase, Grid3 g,
+                        int64_t z0, int64_t z1, float r)
+{
+    const int64_t qpp = g.plane >> 2, q = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const int nxq = (int)(g.nx >> 2), lane = threadIdx.x & 31;
+    const int64_t za = z0 + (int64_t)blockIdx.y * kHeatZR;
+    const int cnt = (int)min((int64_t)kHeatZR, z1 - za);
+    const bool inside = q < qpp;
+    const int64_t off = inside ? 4 * q : 0;
+    const int xq = inside ? (int)(q % nxq) : 0;
+    const bool up_in = inside && q >= nxq, dn_in = inside && q + nxq < qpp;
+    const float4 z4 = zero4();
+    int s = (int)ring_slot(za, zbase, nslot);
+    const float *p[kHeatZR + 2];  // planes za - 1 .. za + ZR
+    bool v[kHeatZR + 2];
+    s = s == 0 ? nslot - 1 : s - 1;
+#pragma unroll
+    for (int j = 0; j < kHeatZR + 2; ++j) {
+        const int64_t z = za - 1 + j;
+        v[j] = z >= 0 && z < g.nz && j <= cnt + 1;
+        p[j] = in + (int64_t)s * g.plane + off;
+        s = wrap_add(s, 1, nslot);
+    }
+    pdl_begin();
+    float4 c[kHeatZR + 2], up[kHeatZR], dn[kHeatZR];
+    float xe[kHeatZR], xf[kHeatZR];  // beyond the warp's first and last point
+#pragma unroll
+    for (int j = 0; j < kHeatZR + 2; ++j)
+        c[j] = inside && v[j] ? ldg4(p[j]) : z4;
+#pragma unroll
+    for (int j = 0; j < kHeatZR; ++j) {
+        const bool w = j < cnt;
+        up[j] = up_in && w ? ldg4(p[j + 1] - g.nx) : z4;
+        dn[j] = dn_in && w ? ldg4(p[j + 1] + g.nx) : z4;
+        xe[j] = inside && w && lane == 0 && xq > 0 ? __ldca(p[j + 1] - 1) : 0.0f;
+        xf[j] = inside && w && lane == 31 && xq < nxq - 1 ? __ldca(p[j + 1] + 4) : 0.0f;
+    }
+#pragma unroll
+    for (int j = 0; j < kHeatZR; ++j) {
+        float xl = __shfl_up_sync(0xffffffffu, c[j + 1].w, 1), xr = __shfl_down_sync(0xffffffffu, c[j + 1].x, 1);
+        if (lane == 0)
+            xl = xe[j];
+        if (lane == 31)
+            xr = xf[j];
+        if (xq == 0)
+            xl = 0.0f;
+        if (xq == nxq - 1)
+            xr = 0.0f;
+        const float4 o = heat_pt4(c[j + 1], xl, xr, up[j], dn[j], c[j], c[j + 2], r);
+        if (inside && j < cnt)
+            *reinterpret_cast<float4 *>(out + (p[j + 1] - in)) = o;
+    }
+}
 
 // Two heat7 steps per launch: levels s and s+1 of a pair, with level s kept
 // on chip (temporal blocking inside the kernel, so HBM carries 8 bytes per
@@ -221,8 +290,8 @@ __global__ void __launch_bounds__(kTX *(TYO + 2), OOC_HEATX2_MINB)
     float4 nn = (inside && z + 2 < nz) ? ldg4(p2 + off) : z4;
     float4 hyv = (hrow && z >= 0) ? ldg4(p0 + hoff) : z4;
     float4 hyv1 = (hrow && z + 1 < nz) ? ldg4(p1 + hoff) : z4;
-    float hx = (hcol && z >= 0) ? __ldg(p0 + xoff) : 0.f;
-    float hx1 = (hcol && z + 1 < nz) ? __ldg(p1 + xoff) : 0.f;
+    float hx = (hcol && z >= 0) ? __ldca(p0 + xoff) : 0.f;
+    float hx1 = (hcol && z + 1 < nz) ? __ldca(p1 + xoff) : 0.f;
     float4 sm2 = z4, sm1 = z4;  // level s at planes z-2, z-1
 OOC_PRAGMA(unroll OOC_HEATX2_UNROLL)
     for (int i = 0; i < cnt + 2; ++i, ++z) {
@@ -230,7 +299,7 @@ OOC_PRAGMA(unroll OOC_HEATX2_UNROLL)
         const float4 pfv = (inside && z + 3 < nz) ? ldg4(in + (int64_t)s3 * plane + off) : z4;
         const bool v2 = z + 2 >= 0 && z + 2 < nz;
         const float4 hyv2 = (hrow && v2) ? ldg4(in + (int64_t)s2 * plane + hoff) : z4;
-        const float hx2 = (hcol && v2) ? __ldg(in + (int64_t)s2 * plane + xoff) : 0.f;
+        const float hx2 = (hcol && v2) ? __ldca(in + (int64_t)s2 * plane + xoff) : 0.f;
 
         const int b = i & 1;
         ta[b][w + 1][lane] = cur;
@@ -353,8 +422,8 @@ __global__ void __launch_bounds__(kTX *NW, 2)
     float4 nna = (ina && z + 2 < nz) ? ldg4(p2 + offa) : z4, nnb = (inb && z + 2 < nz) ? ldg4(p2 + offb) : z4;
     float4 hyv = (hrow && z >= 0) ? ldg4(p0 + hoff) : z4;
     float4 hyv1 = (hrow && z + 1 < nz) ? ldg4(p1 + hoff) : z4;
-    float hxa = (hca && z >= 0) ? __ldg(p0 + xoffa) : 0.f, hxb = (hcb && z >= 0) ? __ldg(p0 + xoffb) : 0.f;
-    float hxa1 = (hca && z + 1 < nz) ? __ldg(p1 + xoffa) : 0.f, hxb1 = (hcb && z + 1 < nz) ? __ldg(p1 + xoffb) : 0.f;
+    float hxa = (hca && z >= 0) ? __ldca(p0 + xoffa) : 0.f, hxb = (hcb && z >= 0) ? __ldca(p0 + xoffb) : 0.f;
+    float hxa1 = (hca && z + 1 < nz) ? __ldca(p1 + xoffa) : 0.f, hxb1 = (hcb && z + 1 < nz) ? __ldca(p1 + xoffb) : 0.f;
     float4 s2a = z4, s1a = z4, s2b = z4, s1b = z4;  // level s at planes z-2, z-1
 OOC_PRAGMA(unroll OOC_HEATX2_UNROLL)
     for (int i = 0; i < cnt + 2; ++i, ++z) {
@@ -365,8 +434,8 @@ OOC_PRAGMA(unroll OOC_HEATX2_UNROLL)
         const float4 pfa = (ina && v3) ? ldg4(q3 + offa) : z4;
         const float4 pfb = (inb && v3) ? ldg4(q3 + offb) : z4;
         const float4 hyv2 = (hrow && v2) ? ldg4(q2 + hoff) : z4;
-        const float hxa2 = (hca && v2) ? __ldg(q2 + xoffa) : 0.f;
-        const float hxb2 = (hcb && v2) ? __ldg(q2 + xoffb) : 0.f;
+        const float hxa2 = (hca && v2) ? __ldca(q2 + xoffa) : 0.f;
+        const float hxb2 = (hcb && v2) ? __ldca(q2 + xoffb) : 0.f;
 
         const int bb = i & 1;
         ta[bb][2 * w + 1][lane] = ca;
@@ -489,6 +558,7 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
     static_assert(kWavePS == 2 * R + 1 && kWavePS % kWaveKS == 0 && kWaveLead == kWavePS - 1, "stage geometry");
     extern __shared__ __align__(16) unsigned char wave_smem[];
     WaveSmem &sm = *reinterpret_cast<WaveSmem *>(wave_smem);
+    pdl_begin();
     const int lane = threadIdx.x, ty = threadIdx.y;
     const int64_t gx = (g.nx + kSeg - 1) / kSeg;  // x tiles; blockIdx.x = by * gx + bx
     const int64_t xs = (int64_t)(blockIdx.x % gx) * kSeg;
@@ -716,20 +786,28 @@ __global__ void swap_kernel(float *a, float *b, int64_t n)
 
 }  // namespace
 
+bool heat7_small(int64_t nx, int64_t ny, int64_t nplanes) { return nx * ny <= kHeatDirectMax / nplanes; }
+
 cudaError_t launch_heat7(ConstRing in, Ring out, int64_t nx, int64_t ny, int64_t nz, int64_t z0, int64_t z1,
-                         float r, cudaStream_t st)
+                         float r, cudaStream_t st, bool pdl)
 {
     if (z1 <= z0)
         return cudaSuccess;
+    if (heat7_small(nx, ny, z1 - z0) && in.nslot == out.nslot && in.zbase == out.zbase &&
+        in.nslot <= (1ll << 30) && (z1 - z0 + kHeatZR - 1) / kHeatZR <= 65535) {
+        const int64_t bx = (nx * ny / 4 + 255) / 256;
+        return launch(pdl, heat7_direct_kernel, dim3((unsigned)bx, (unsigned)((z1 - z0 + kHeatZR - 1) / kHeatZR)),
+                          dim3(256), 0, st, in.base, out.base, (int)in.nslot, in.zbase, Grid3{nx, ny, nz, nx * ny}, z0,
+                          z1, r);
+    }
     static const int res = resident((const void *)heat7_kernel, kTX * kHeatTY);  // once, thread-safe
     const int64_t gx = (nx + kSeg - 1) / kSeg, gy = (ny + kHeatTY - 1) / kHeatTY;
     const int64_t chunk = choose_chunk(gx * gy, z1 - z0, 8, 3, res);
     const int64_t gz = (z1 - z0 + chunk - 1) / chunk;
     if (in.nslot != out.nslot || in.zbase != out.zbase || in.nslot > (1ll << 30) || gx * gy > 0x7fffffffll)
         return cudaErrorInvalidValue;
-    heat7_kernel<<<dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kHeatTY), 0, st>>>(
-        in.base, out.base, (int)in.nslot, in.zbase, Grid3{nx, ny, nz, nx * ny}, z0, z1, chunk, r);
-    return cudaGetLastError();
+    return launch(pdl, heat7_kernel, dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kHeatTY), 0, st, in.base,
+                      out.base, (int)in.nslot, in.zbase, Grid3{nx, ny, nz, nx * ny}, z0, z1, chunk, r);
 }
 
 // The fused pairs of the register-loading kernels (build option
@@ -774,7 +852,7 @@ cudaError_t launch_heat7x2_regs(ConstRing in, Ring out, int64_t nx, int64_t ny, 
 #if !OOC_WAVE_TMA
 cudaError_t launch_wave25_to(ConstRing p, ConstRing pprev, Ring pnew, ConstRing kappa, int64_t nx, int64_t ny,
                              int64_t nz, int64_t z0, int64_t z1, int64_t sx, int64_t sy, int64_t sz, float w,
-                             cudaStream_t st, WaveSrcTable tab)
+                             cudaStream_t st, WaveSrcTable tab, bool pdl)
 {
     if (z1 <= z0)
         return cudaSuccess;
@@ -793,10 +871,10 @@ cudaError_t launch_wave25_to(ConstRing p, ConstRing pprev, Ring pnew, ConstRing 
     if (p.nslot != pnew.nslot || p.zbase != pnew.zbase || p.nslot != kappa.nslot || p.zbase != kappa.zbase ||
         p.nslot != pprev.nslot || p.zbase != pprev.zbase || p.nslot > (1ll << 30) || gx * gy > 0x7fffffffll)
         return cudaErrorInvalidValue;
-    wave25_kernel<0><<<dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWaveTY), sizeof(WaveSmem), st>>>(
+    return launch(pdl, wave25_kernel<0>, dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWaveTY),
+                      sizeof(WaveSmem), st,
         p.base, pprev.base, pnew.base, kappa.base, (int)p.nslot, p.zbase, Grid3{nx, ny, nz, nx * ny}, z0, z1, chunk,
-        sx, sy, sz, w, nullptr, tab);
-    return cudaGetLastError();
+        sx, sy, sz, w, (double *)nullptr, tab, (float *)nullptr);
 }
 
 cudaError_t launch_wave25_grad(const float *p, const float *mu, double *g, int64_t nx, int64_t ny, int64_t nz,
@@ -816,10 +894,10 @@ cudaError_t launch_wave25_grad(const float *p, const float *mu, double *g, int64
     const int64_t gz = (nz + chunk - 1) / chunk;
     if (gx * gy > 0x7fffffffll || nz > (1ll << 30))
         return cudaErrorInvalidValue;
-    wave25_kernel<1><<<dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWaveTY), sizeof(WaveSmem), st>>>(
-        p, mu, nullptr, nullptr, (int)nz, 0, Grid3{nx, ny, nz, nx * ny}, 0, nz, chunk, -1, -1, -1, 0.0f, g,
-        WaveSrcTable{});
-    return cudaGetLastError();
+    return launch(false, wave25_kernel<1>, dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWaveTY),
+                      sizeof(WaveSmem), st,
+        p, mu, (float *)nullptr, (const float *)nullptr, (int)nz, 0, Grid3{nx, ny, nz, nx * ny}, 0, nz, chunk, -1, -1, -1, 0.0f, g,
+        WaveSrcTable{}, (float *)nullptr);
 }
 
 cudaError_t launch_wave25_grad32(const float *p, const float *mu, float *gacc, int64_t nx, int64_t ny, int64_t nz,
@@ -839,18 +917,18 @@ cudaError_t launch_wave25_grad32(const float *p, const float *mu, float *gacc, i
     const int64_t gz = (nz + chunk - 1) / chunk;
     if (gx * gy > 0x7fffffffll || nz > (1ll << 30))
         return cudaErrorInvalidValue;
-    wave25_kernel<2><<<dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWaveTY), sizeof(WaveSmem), st>>>(
-        p, mu, nullptr, nullptr, (int)nz, 0, Grid3{nx, ny, nz, nx * ny}, 0, nz, chunk, -1, -1, -1, 0.0f, nullptr,
+    return launch(true, wave25_kernel<2>, dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWaveTY),
+                      sizeof(WaveSmem), st,
+        p, mu, (float *)nullptr, (const float *)nullptr, (int)nz, 0, Grid3{nx, ny, nz, nx * ny}, 0, nz, chunk, -1, -1, -1, 0.0f, (double *)nullptr,
         WaveSrcTable{}, gacc);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_wave25(ConstRing p, Ring pprev_out, ConstRing kappa, int64_t nx, int64_t ny, int64_t nz,
                           int64_t z0, int64_t z1, int64_t sx, int64_t sy, int64_t sz, float w, cudaStream_t st,
-                          WaveSrcTable tab)
+                          WaveSrcTable tab, bool pdl)
 {
     return launch_wave25_to(p, ConstRing{pprev_out.base, pprev_out.nslot, pprev_out.zbase}, pprev_out, kappa, nx, ny,
-                            nz, z0, z1, sx, sy, sz, w, st, tab);
+                            nz, z0, z1, sx, sy, sz, w, st, tab, pdl);
 }
 
 #endif

@@ -40,7 +40,8 @@ __device__ __forceinline__ int wrap_add(int s, int d, int nslot)
     return s >= nslot ? s - nslot : s;
 }
 
-__device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+// coherent loads: the fields are written by the kernel before (pdl_begin)
+__device__ __forceinline__ float4 ldg4(const float *p) { return __ldca(reinterpret_cast<const float4 *>(p)); }
 
 // One heat7 point in a fixed operation order, written with rounding
 // intrinsics so that the compiler cannot contract or reorder it: every heat
@@ -85,13 +86,14 @@ __device__ __forceinline__ float4 heat_pt4x2(float4 c, float xl, float xr, float
     return o;
 }
 
-// z-chunk so that the grid fills whole waves: pick the chunk count (1..8,
+// z-chunk so that the grid fills whole waves: pick the chunk count (1..64,
 // chunks of at least min_chunk planes) minimising waves x (chunk + overhead).
+// (Up to 8, a field of few tiles, 112 x 112 x 1024, left half the chip idle.)
 inline int64_t choose_chunk(int64_t ntiles, int64_t height, int64_t min_chunk, int64_t overhead, int resident_ctas)
 {
     int64_t best_n = 1;
     double best_cost = 1e300;
-    for (int64_t n = 1; n <= 8; ++n) {
+    for (int64_t n = 1; n <= 64; ++n) {
         const int64_t chunk = (height + n - 1) / n;
         if (n > 1 && chunk < min_chunk)
             break;
