@@ -26,11 +26,10 @@
 // terms, in a device field); each segment's sum is then added to the FP64
 // total.  GB300's FP64 pipe made a per-step FP64 update (two conversions, a
 // multiply and an add per point) the slowest kernel of the backward pass.
-#include <chrono>
 #include <cstring>
-#include <thread>
 
 #include "common.cuh"
+#include "host_wait.cuh"
 
 using namespace ooc;
 
@@ -313,21 +312,6 @@ Layout make_layout(int64_t n, int64_t every, int rate)
     return L;
 }
 
-ooc_status wait_ev(cudaEvent_t ev, int64_t timeout_ms)
-{
-    const auto deadline = std::chrono::steady_clock::now() + std::chrono::milliseconds(timeout_ms);
-    for (;;) {
-        const cudaError_t e = cudaEventQuery(ev);
-        if (e == cudaSuccess)
-            return OOC_OK;
-        if (e != cudaErrorNotReady)
-            return OOC_E_CUDA;
-        if (std::chrono::steady_clock::now() > deadline)
-            return OOC_E_TIMEOUT;
-        std::this_thread::sleep_for(std::chrono::microseconds(50));
-    }
-}
-
 struct Events {
     cudaEvent_t e[8];
     int made = 0;
@@ -360,14 +344,14 @@ ooc_status check_receivers(const int64_t *d_rec, int64_t nrec, int64_t size, cud
     check_indices_kernel<<<(unsigned)((nrec + 255) / 256), 256, 0, st>>>(d_rec, nrec, size);
     if (cudaGetLastError() != cudaSuccess || cudaEventRecord(ev, st) != cudaSuccess)
         return OOC_E_CUDA;
-    const ooc_status w = wait_ev(ev, 600000);
+    const ooc_status w = wait_event(ev, 600000);
     if (w != OOC_OK)
         return w;
     unsigned bad = 0u;
     if (cudaMemcpyFromSymbolAsync(&bad, g_receivers_bad, sizeof(bad), 0, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaEventRecord(ev, st) != cudaSuccess)
         return OOC_E_CUDA;
-    const ooc_status w2 = wait_ev(ev, 600000);
+    const ooc_status w2 = wait_event(ev, 600000);
     if (w2 != OOC_OK)
         return w2;
     return bad ? OOC_E_INVALID : OOC_OK;
@@ -521,9 +505,9 @@ ooc_status ooc_wave25_forward_ckpt(const float *d_kappa, int64_t nx, int64_t ny,
     }
     TRY_CUDA(cudaEventRecord(ev.e[4], sC));
     TRY_CUDA(cudaEventRecord(ev.e[5], sD));
-    ooc_status st = wait_ev(ev.e[4], 600000);
+    ooc_status st = wait_event(ev.e[4], 600000);
     if (st == OOC_OK)
-        st = wait_ev(ev.e[5], 600000);
+        st = wait_event(ev.e[5], 600000);
     return st;
 }
 
@@ -618,9 +602,9 @@ ooc_status ooc_wave25_backward_ckpt(const float *d_kappa, int64_t nx, int64_t ny
     TRY_CUDA(cudaGetLastError());
     TRY_CUDA(cudaEventRecord(ev.e[4], sC));
     TRY_CUDA(cudaEventRecord(ev.e[5], sD));
-    ooc_status st = wait_ev(ev.e[4], 600000);
+    ooc_status st = wait_event(ev.e[4], 600000);
     if (st == OOC_OK)
-        st = wait_ev(ev.e[5], 600000);
+        st = wait_event(ev.e[5], 600000);
     return st;
 }
 

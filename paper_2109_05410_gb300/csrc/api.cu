@@ -1,10 +1,9 @@
 // api.cu -- stand-alone entry points of the C ABI: codec, BF16, in-core
 // stencil runs and status strings.  See include/ooc.h for the contract.
-#include <chrono>
 #include <cmath>
-#include <thread>
 
 #include "common.cuh"
+#include "host_wait.cuh"
 
 using namespace ooc;
 
@@ -30,19 +29,7 @@ ooc_status wait_stream(cudaStream_t st, int64_t timeout_ms)
     cudaEvent_t ev = nullptr;
     if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess)
         return OOC_E_CUDA;
-    ooc_status s = cudaEventRecord(ev, st) == cudaSuccess ? OOC_OK : OOC_E_CUDA;
-    const auto deadline = std::chrono::steady_clock::now() + std::chrono::milliseconds(timeout_ms);
-    while (s == OOC_OK) {
-        const cudaError_t e = cudaEventQuery(ev);
-        if (e == cudaSuccess)
-            break;
-        if (e != cudaErrorNotReady)
-            s = OOC_E_CUDA;
-        else if (std::chrono::steady_clock::now() > deadline)
-            s = OOC_E_TIMEOUT;
-        else
-            std::this_thread::sleep_for(std::chrono::microseconds(20));
-    }
+    const ooc_status s = cudaEventRecord(ev, st) == cudaSuccess ? wait_event(ev, timeout_ms) : OOC_E_CUDA;
     cudaEventDestroy(ev);
     return s;
 }
@@ -285,14 +272,16 @@ ooc_status ooc_compress_var(const float *d_in, int64_t nx, int64_t ny, int64_t n
     const ooc_status ws = wait_stream(st, kCallWaitMs);
     if (ws != OOC_OK)
         return ws;
-    unsigned fault = 0u;
-    if (take_codec_fault(&fault) != cudaSuccess)
+    // the last tile's status word: the total, unless a look-back gave up
+    uint64_t word = 0;
+    if (cudaMemcpy(&word, (const uint64_t *)d_scratch + var_total_word(nblk), sizeof(word), cudaMemcpyDeviceToHost) !=
+        cudaSuccess)
         return OOC_E_CUDA;
-    if (fault)
-        return OOC_E_TIMEOUT;
     uint64_t total = 0;
-    if (cudaMemcpy(&total, d_index + nblk, sizeof(total), cudaMemcpyDeviceToHost) != cudaSuccess)
-        return OOC_E_CUDA;
+    if (!var_total(word, &total)) {
+        unsigned fault = 0u;
+        return take_codec_fault(&fault) == cudaSuccess ? OOC_E_TIMEOUT : OOC_E_CUDA;
+    }
     *out_bytes = (size_t)total * 4;
     return *out_bytes > out_cap ? OOC_E_INVALID : OOC_OK;
 }

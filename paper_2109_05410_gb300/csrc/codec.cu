@@ -1654,6 +1654,14 @@ cudaError_t launch_fr4_decode_dense(const uint32_t *in, int64_t in_words, const 
     return cudaGetLastError();
 }
 
+int64_t var_total_word(int64_t nblk) { return (nblk + kThreads - 1) / kThreads; }
+
+bool var_total(uint64_t word, uint64_t *total)
+{
+    *total = word & kTileValue;
+    return (word & ~kTileValue) == kTilePrefix;
+}
+
 // the tile counter and one status word per tile of the variable-size encoder
 size_t var_scratch_bytes(int64_t nblk) { return sizeof(uint64_t) * (size_t)((nblk + kThreads - 1) / kThreads + 1); }
 

@@ -174,6 +174,10 @@ cudaError_t launch_fr4_encode_dense(const float *in, int64_t nx, int64_t ny, int
 cudaError_t launch_fr4_encode_var(const float *in, int64_t nx, int64_t ny, int64_t nz, int mode, int mparam,
                                   uint32_t *out, uint64_t out_words, uint64_t *index, void *scratch, cudaStream_t st);
 size_t var_scratch_bytes(int64_t nblk);
+// After it: the index of the 64-bit scratch word that holds the total, and the
+// total in that word (false if a bounded look-back gave up).
+int64_t var_total_word(int64_t nblk);
+bool var_total(uint64_t word, uint64_t *total);
 // Reads and clears the word set when the variable-size encoder's bounded
 // look-back gave up.
 cudaError_t take_codec_fault(unsigned *fault);

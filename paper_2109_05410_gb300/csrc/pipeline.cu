@@ -28,10 +28,10 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
-#include <thread>
 #include <vector>
 
 #include "common.cuh"
+#include "host_wait.cuh"
 
 using namespace ooc;
 
@@ -256,18 +256,7 @@ cudaError_t copy_ring(ooc_plan *p, int r, int64_t zbase, int64_t z0, int64_t z1,
 
 ooc_status wait_event(ooc_plan *p, cudaEvent_t ev)
 {
-    const int64_t ms = p->cfg.wait_timeout_ms > 0 ? p->cfg.wait_timeout_ms : 600000;
-    const auto deadline = std::chrono::steady_clock::now() + std::chrono::milliseconds(ms);
-    for (;;) {
-        const cudaError_t e = cudaEventQuery(ev);
-        if (e == cudaSuccess)
-            return OOC_OK;
-        if (e != cudaErrorNotReady)
-            return OOC_E_CUDA;
-        if (std::chrono::steady_clock::now() > deadline)
-            return OOC_E_TIMEOUT;
-        std::this_thread::sleep_for(std::chrono::microseconds(20));
-    }
+    return ooc::wait_event(ev, p->cfg.wait_timeout_ms > 0 ? p->cfg.wait_timeout_ms : 600000);
 }
 
 // debug_checks: every guard region back to kGuardByte and the flag to 0.
