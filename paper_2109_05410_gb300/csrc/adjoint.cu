@@ -26,6 +26,15 @@
 // terms, in a device field); each segment's sum is then added to the FP64
 // total.  GB300's FP64 pipe made a per-step FP64 update (two conversions, a
 // multiply and an add per point) the slowest kernel of the backward pass.
+//
+// The replay keeps L(p^n), which its steps compute anyway, in place of p^n,
+// so a term costs no Laplacian; and a term is added where its w is already on
+// chip: every second adjoint step holds two (its p and p_prev), the flush
+// takes the rest.  Per replayed step that is 20 + 24 bytes and two 25-point
+// sums in two launches, against 48 bytes and three sums in three launches
+// for a gradient kernel of its own: at 256^3, where a step is bound by the
+// sums' instructions (52 us against 40 us of traffic), forward and gradient
+// of 100 steps took 28.8 ms with it and 22.6 ms without.
 #include <cstring>
 
 #include "common.cuh"
@@ -222,13 +231,17 @@ __global__ void check_indices_kernel(const int64_t *__restrict__ idx, int64_t n,
         atomicOr(&g_receivers_bad, 1u);
 }
 
-// g[i] += (double) a[i]; a[i] = 0: a segment's FP32 gradient sum into the
-// FP64 total.
-__global__ void flush_segment_kernel(double *__restrict__ g, float *__restrict__ a, int64_t n)
+// A segment's FP32 gradient sum a (nullptr: 0) and its last one or two terms,
+// w1 l1 (w1 may be nullptr) and w0 l0, into the FP64 total g.
+__global__ void flush_segment_kernel(double *__restrict__ g, const float *__restrict__ a,
+                                     const float *__restrict__ w1, const float *__restrict__ l1,
+                                     const float *__restrict__ w0, const float *__restrict__ l0, int64_t n)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        g[i] += (double)a[i];
-        a[i] = 0.0f;
+        float s = a ? a[i] : 0.0f;
+        if (w1)
+            s = __fmaf_rn(w1[i], l1[i], s);
+        g[i] += (double)__fmaf_rn(w0[i], l0[i], s);
     }
 }
 
@@ -540,7 +553,6 @@ ooc_status ooc_wave25_backward_ckpt(const float *d_kappa, int64_t nx, int64_t ny
     TRY_CUDA(cudaMemsetAsync(mu1, 0, sizeof(float) * n, sC));
     TRY_CUDA(cudaMemsetAsync(mu2, 0, sizeof(float) * n, sC));
     TRY_CUDA(cudaMemsetAsync(d_grad, 0, sizeof(double) * n, sC));
-    TRY_CUDA(cudaMemsetAsync(gacc, 0, sizeof(float) * n, sC));
     const bool src = sx >= 0 && h_w != nullptr;
     const int64_t nseg = (nsteps + every - 1) / every;
     auto load = [&](int64_t k) -> cudaError_t {  // checkpoint k -> staging (k & 1), on sD
@@ -572,30 +584,41 @@ ooc_status ooc_wave25_backward_ckpt(const float *d_kappa, int64_t nx, int64_t ny
             TRY_CUDA(cudaStreamWaitEvent(sD, ev.e[2 + (1 - bi)], 0));
             TRY_CUDA(load(k - 1));
         }
-        // replay: hist[j + 1] = p^{n0 + j}, j = 1 .. len - 1
-        for (int64_t j = 1; j < len; ++j) {
-            const int64_t s = n0 + j - 1;
-            TRY_CUDA(launch_wave25_to(ConstRing{hist(j), nz, 0}, ConstRing{hist(j - 1), nz, 0}, Ring{hist(j + 1), nz, 0},
-                                      ConstRing{d_kappa, nz, 0}, nx, ny, nz, 0, nz, src ? sx : -1, sy, sz,
-                                      src ? h_w[s] : 0.0f, sC, WaveSrcTable{}, true));
+        // replay in place in hist[0] and hist[1]; L(p^{n0+j}) is kept in
+        // hist[j + 2], the last one (no step follows) in the older p buffer
+        float *p = hist(1), *pp = hist(0);
+        for (int64_t j = 0; j + 1 < len; ++j) {
+            TRY_CUDA(launch_wave25_lap(p, pp, pp, d_kappa, hist(j + 2), nx, ny, nz, src ? sx : -1, sy, sz,
+                                       src ? h_w[n0 + j] : 0.0f, sC));
+            float *t = p;
+            p = pp;
+            pp = t;
         }
-        // adjoint through the segment, on w = kappa mu (mu1 / mu2 hold w)
+        TRY_CUDA(launch_wave25_lap(p, pp, nullptr, d_kappa, pp, nx, ny, nz, -1, -1, -1, 0.0f, sC));
+        auto lap = [&](int64_t j) { return j + 1 < len ? hist(j + 2) : pp; };  // L(p^{n0+j})
+        // adjoint through the segment, on w = kappa mu (mu1 / mu2 hold w);
+        // the second, fourth, ... step, to w^m from w^{m+1} and w^{m+2}, also
+        // adds w^{m+2} L(p^{m+1}) + w^{m+1} L(p^m), in FP32 within the segment
         for (int64_t m = n1; m >= n0 + 1; --m) {
-            TRY_CUDA(launch_wave25_to(ConstRing{mu1, nz, 0}, ConstRing{mu2, nz, 0}, Ring{mu2, nz, 0},
-                                      ConstRing{d_kappa, nz, 0}, nx, ny, nz, 0, nz, -1, -1, -1, 0.0f, sC,
-                                      WaveSrcTable{}, true));
+            if (m < n1 && (n1 - m) % 2 == 0)
+                TRY_CUDA(launch_wave25_gacc(mu1, mu2, d_kappa, lap(m + 1 - n0), lap(m - n0), gacc, m == n1 - 2, nx, ny,
+                                            nz, sC));
+            else
+                TRY_CUDA(launch_wave25(ConstRing{mu1, nz, 0}, Ring{mu2, nz, 0}, ConstRing{d_kappa, nz, 0}, nx, ny, nz,
+                                       0, nz, -1, -1, -1, 0.0f, sC, WaveSrcTable{}, true));
             if (nrec > 0) {  // + kappa S^T res[m-1]
                 TRY_CUDA(launch(true, scatter_add_scaled_kernel, dim3((unsigned)((nrec + 255) / 256)), dim3(256), 0, sC,
                                 mu2, n, d_rec, nrec, d_res + (m - 1) * nrec, d_kappa));
             }
-            // += w^m L(p^{m-1}), in FP32 within the segment
-            TRY_CUDA(launch_wave25_grad32(hist(m - n0), mu2, gacc, nx, ny, nz, sC));
             float *t = mu1;
             mu1 = mu2;
             mu2 = t;
         }
-        // the segment's sum (at most `every` terms) into the FP64 total
-        flush_segment_kernel<<<grid1d(n, 256), 256, 0, sC>>>(d_grad, gacc, n);
+        // the segment's sum (at most `every` terms) into the FP64 total, with
+        // its last terms: w^{n0+2} L(p^{n0+1}) if len is even, w^{n0+1} L(p^{n0})
+        flush_segment_kernel<<<grid1d(n, 256), 256, 0, sC>>>(d_grad, len > 2 ? gacc : nullptr,
+                                                             len % 2 ? nullptr : mu2, len % 2 ? nullptr : lap(1), mu1,
+                                                             lap(0), n);
         TRY_CUDA(cudaGetLastError());
     }
     divide_by_kappa_kernel<<<grid1d(n, 256), 256, 0, sC>>>(d_grad, d_kappa, n);

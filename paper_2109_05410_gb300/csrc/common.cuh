@@ -105,10 +105,19 @@ bool heat7_small(int64_t nx, int64_t ny, int64_t nplanes);
 // 25-point Laplacian without kappa); g 32-byte aligned.
 cudaError_t launch_wave25_grad(const float *p, const float *mu, double *g, int64_t nx, int64_t ny, int64_t nz,
                                cudaStream_t st);
-// gacc[i] = fma(mu[i], L(p)[i], gacc[i]) in FP32 over whole dense fields
-// (gacc 16-byte aligned): the adjoint run's in-segment gradient sums.
-cudaError_t launch_wave25_grad32(const float *p, const float *mu, float *gacc, int64_t nx, int64_t ny, int64_t nz,
-                                 cudaStream_t st);
+// The two steps of the adjoint run's backward pass, on dense fields (all
+// pointers 16-byte aligned), launched as dependents (see launch()).
+// _lap: one step, p' to pnew (may be pprev; nullptr: no step, only the
+// Laplacian) and L(p) to lap (a buffer of its own, or pprev if pnew is null).
+// _gacc: one step with p_prev overwritten, and in FP32
+// gacc[i] = fma(p[i], lap_p[i], fma(p_prev[i], lap_pprev[i], gacc[i])), with 0
+// in place of gacc[i] if fresh.
+cudaError_t launch_wave25_lap(const float *p, const float *pprev, float *pnew, const float *kappa, float *lap,
+                              int64_t nx, int64_t ny, int64_t nz, int64_t sx, int64_t sy, int64_t sz, float w,
+                              cudaStream_t st);
+cudaError_t launch_wave25_gacc(const float *p, float *pprev_out, const float *kappa, const float *lap_pprev,
+                               const float *lap_p, float *gacc, bool fresh, int64_t nx, int64_t ny, int64_t nz,
+                               cudaStream_t st);
 // Two heat7 steps in one launch: level s on [lo, hi) computed on chip from
 // ring `in` (level s-1), level s+1 written to ring `out` on [z0, z1).  The
 // two level-s planes below lo are read from band_in (planes bin_lo,

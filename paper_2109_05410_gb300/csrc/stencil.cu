@@ -542,9 +542,13 @@ using IC = std::integral_constant<int, V>;
 
 // MODE 0: the leapfrog step above.  MODE 1 (gradient of the adjoint run):
 // gsum[own] += (double) pprev * (double) L(pin) in FP64, with `pprev` the
-// adjoint field and kappa, pout and the source unused.  MODE 2: the same
-// term accumulated in FP32, gacc[own] = fma(pprev, L(pin), gacc[own]) (the
-// adjoint run's short in-segment sums, added to an FP64 total per segment).
+// adjoint field and kappa, pout and the source unused.  MODE 2: the step,
+// with L(pin) also stored to lapf; pout == nullptr leaves the step itself out
+// (p_prev and kappa are then not read).  MODE 3: the step, and in FP32
+// gacc[own] = fma(pin, lap2, fma(pprev, lapf, gacc[own])) (0 for gacc[own]
+// with `fresh`): two of the adjoint run's gradient terms w L(p), from the
+// L(p) that its replay (MODE 2) kept.  Both w are in registers, so two terms
+// cost two reads and one update of gacc and no Laplacian.
 // The arithmetic is written with rounding intrinsics in a fixed order:
 //   L = 3 c0 p + sum_m c_m (((x-m + x+m) + (y-m + y+m)) + (z-m + z+m))
 //   p' = kappa L + (2 p - p_prev)
@@ -552,7 +556,8 @@ template <int MODE>
 __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
     wave25_kernel(const float *__restrict__ pin, const float *pprev, float *pout, const float *__restrict__ kap, int nslot,
                   int64_t zbase, Grid3 g, int64_t z0, int64_t z1, int64_t zchunk, int64_t sx, int64_t sy, int64_t sz,
-                  float w, double *__restrict__ gsum, WaveSrcTable tab, float *__restrict__ gacc = nullptr)
+                  float w, double *__restrict__ gsum, WaveSrcTable tab, float *lapf,
+                  const float *__restrict__ lap2, float *__restrict__ gacc, bool fresh)
 {
     constexpr int R = kWaveR;
     static_assert(kWavePS == 2 * R + 1 && kWavePS % kWaveKS == 0 && kWaveLead == kWavePS - 1, "stage geometry");
@@ -586,6 +591,7 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
     const bool hcol = (lane == 0 || lane == kTX - 1) && xh >= 0 && xh < g.nx && y < g.ny;
     const int64_t xoff = hcol ? y * g.nx + xh : 0;
     const bool src_here = inside && y == sy && sx >= x4 && sx < x4 + 4;
+    const bool step_on = MODE != 2 || pout != nullptr;
     const float4 z4 = zero4();
 
     // Copy group of plane gz into p stage ST and, with K, p_prev / kappa of
@@ -609,9 +615,9 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
         if (with_k) {
             if (gz - kWaveLead + 2 < zend) {
                 const int64_t kb = (int64_t)ks * plane;
-                cp_async16(&sm.pp[KST][ty][lane], pprev + kb + off, inside);
-                if (MODE == 0)
-                    cp_async16(&sm.kk[KST][ty][lane], kap + kb + off, inside);
+                cp_async16(&sm.pp[KST][ty][lane], pprev + kb + off, inside && step_on);
+                if (MODE != 1)
+                    cp_async16(&sm.kk[KST][ty][lane], kap + kb + off, inside && step_on);
             }
             ks = wrap_add(ks, 1, nslot);
         }
@@ -646,6 +652,11 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
         cp_async_wait<1>();  // groups up to plane z + 6 have landed (p tile of z + 4, p_prev / kappa of z)
         __syncthreads();     // ... for every thread; the stages of plane z - 1 are free
         issue(IC<(PH + kWaveLead) % kWavePS>{}, IC<(PH + 2) % kWaveKS>{}, z + kWaveLead, true);
+        // MODE 3: read here, used after the Laplacian
+        const int64_t own = (int64_t)os * plane + off;
+        const float4 la = MODE == 3 ? ldg4(lapf + own) : z4;
+        const float4 lb = MODE == 3 ? ldg4(lap2 + own) : z4;
+        float4 ga = MODE == 3 && !fresh ? *reinterpret_cast<const float4 *>(gacc + own) : z4;
         q[(PH + 2 * R) % kWavePS] = sm.p[(PH + R) % kWavePS][ty + R][lane];
         const float4 c = q[(PH + R) % kWavePS];
         float4 lf, rt;
@@ -662,7 +673,7 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
         if (lane == kTX - 1)
             rt = sm.xh[PH][ty][1];
         const float4 ppv = sm.pp[PH % kWaveKS][ty][lane];
-        const float4 kv = MODE == 0 ? sm.kk[PH % kWaveKS][ty][lane] : z4;
+        const float4 kv = MODE != 1 ? sm.kk[PH % kWaveKS][ty][lane] : z4;
         const float L[4] = {lf.x, lf.y, lf.z, lf.w};
         const float C[4] = {c.x, c.y, c.z, c.w};
         const float Rt[4] = {rt.x, rt.y, rt.z, rt.w};
@@ -717,7 +728,7 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
             }
         }
 #endif
-        if (MODE == 0) {
+        if (MODE != 1) {
             float o[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -733,18 +744,19 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
                     if (sx == x4 + j)
                         o[j] += ws;
             }
-            if (inside)
-                *reinterpret_cast<float4 *>(pout + (int64_t)os * plane + off) = make_float4(o[0], o[1], o[2], o[3]);
-        } else if (MODE == 2 && inside) {
-            float4 *ap = reinterpret_cast<float4 *>(gacc + (int64_t)os * plane + off);
-            float4 a = *ap;
-            a.x = __fmaf_rn(PP[0], lap[0], a.x);
-            a.y = __fmaf_rn(PP[1], lap[1], a.y);
-            a.z = __fmaf_rn(PP[2], lap[2], a.z);
-            a.w = __fmaf_rn(PP[3], lap[3], a.w);
-            *ap = a;
-        } else if (MODE == 1 && inside) {
-            double2 *gp = reinterpret_cast<double2 *>(gsum + (int64_t)os * plane + off);
+            if (inside && step_on)
+                *reinterpret_cast<float4 *>(pout + own) = make_float4(o[0], o[1], o[2], o[3]);
+            if (MODE == 2 && inside)
+                *reinterpret_cast<float4 *>(lapf + own) = make_float4(lap[0], lap[1], lap[2], lap[3]);
+            if (MODE == 3 && inside) {
+                ga.x = __fmaf_rn(C[0], lb.x, __fmaf_rn(PP[0], la.x, ga.x));
+                ga.y = __fmaf_rn(C[1], lb.y, __fmaf_rn(PP[1], la.y, ga.y));
+                ga.z = __fmaf_rn(C[2], lb.z, __fmaf_rn(PP[2], la.z, ga.z));
+                ga.w = __fmaf_rn(C[3], lb.w, __fmaf_rn(PP[3], la.w, ga.w));
+                *reinterpret_cast<float4 *>(gacc + own) = ga;
+            }
+        } else if (inside) {
+            double2 *gp = reinterpret_cast<double2 *>(gsum + own);
             double2 g0 = gp[0], g1 = gp[1];
             g0.x += (double)PP[0] * (double)lap[0];
             g0.y += (double)PP[1] * (double)lap[1];
@@ -850,77 +862,69 @@ cudaError_t launch_heat7x2_regs(ConstRing in, Ring out, int64_t nx, int64_t ny, 
 
 
 #if !OOC_WAVE_TMA
-cudaError_t launch_wave25_to(ConstRing p, ConstRing pprev, Ring pnew, ConstRing kappa, int64_t nx, int64_t ny,
-                             int64_t nz, int64_t z0, int64_t z1, int64_t sx, int64_t sy, int64_t sz, float w,
-                             cudaStream_t st, WaveSrcTable tab, bool pdl)
+namespace {
+// One launch of a wave25_kernel mode over planes [z0, z1) of rings that share
+// nslot and zbase.
+template <int MODE>
+cudaError_t run_wave25(bool pdl, const float *p, const float *pprev, float *pout, const float *kappa, int64_t nslot,
+                       int64_t zbase, int64_t nx, int64_t ny, int64_t nz, int64_t z0, int64_t z1, int64_t sx,
+                       int64_t sy, int64_t sz, float w, double *gsum, WaveSrcTable tab, float *lapf,
+                       const float *lap2, float *gacc, bool fresh, cudaStream_t st)
 {
     if (z1 <= z0)
         return cudaSuccess;
     // set once (thread-safe); 0 if the attribute could not be set
     static const int res = []() -> int {
-        if (cudaFuncSetAttribute(wave25_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(wave25_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(WaveSmem)) != cudaSuccess)
             return 0;
-        return resident((const void *)wave25_kernel<0>, kTX * kWaveTY, sizeof(WaveSmem));
+        return resident((const void *)wave25_kernel<MODE>, kTX * kWaveTY, sizeof(WaveSmem));
     }();
     if (res <= 0)
         return cudaErrorInvalidValue;
     const int64_t gx = (nx + kSeg - 1) / kSeg, gy = (ny + kWaveTY - 1) / kWaveTY;
     const int64_t chunk = choose_chunk(gx * gy, z1 - z0, 16, 9, res);
     const int64_t gz = (z1 - z0 + chunk - 1) / chunk;
-    if (p.nslot != pnew.nslot || p.zbase != pnew.zbase || p.nslot != kappa.nslot || p.zbase != kappa.zbase ||
-        p.nslot != pprev.nslot || p.zbase != pprev.zbase || p.nslot > (1ll << 30) || gx * gy > 0x7fffffffll)
+    if (nslot > (1ll << 30) || gx * gy > 0x7fffffffll)
         return cudaErrorInvalidValue;
-    return launch(pdl, wave25_kernel<0>, dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWaveTY),
-                      sizeof(WaveSmem), st,
-        p.base, pprev.base, pnew.base, kappa.base, (int)p.nslot, p.zbase, Grid3{nx, ny, nz, nx * ny}, z0, z1, chunk,
-        sx, sy, sz, w, (double *)nullptr, tab, (float *)nullptr);
+    return launch(pdl, wave25_kernel<MODE>, dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWaveTY),
+                  sizeof(WaveSmem), st, p, pprev, pout, kappa, (int)nslot, zbase, Grid3{nx, ny, nz, nx * ny}, z0, z1,
+                  chunk, sx, sy, sz, w, gsum, tab, lapf, lap2, gacc, fresh);
+}
+}  // namespace
+
+cudaError_t launch_wave25_to(ConstRing p, ConstRing pprev, Ring pnew, ConstRing kappa, int64_t nx, int64_t ny,
+                             int64_t nz, int64_t z0, int64_t z1, int64_t sx, int64_t sy, int64_t sz, float w,
+                             cudaStream_t st, WaveSrcTable tab, bool pdl)
+{
+    if (p.nslot != pnew.nslot || p.zbase != pnew.zbase || p.nslot != kappa.nslot || p.zbase != kappa.zbase ||
+        p.nslot != pprev.nslot || p.zbase != pprev.zbase)
+        return cudaErrorInvalidValue;
+    return run_wave25<0>(pdl, p.base, pprev.base, pnew.base, kappa.base, p.nslot, p.zbase, nx, ny, nz, z0, z1, sx, sy,
+                         sz, w, nullptr, tab, nullptr, nullptr, nullptr, false, st);
 }
 
 cudaError_t launch_wave25_grad(const float *p, const float *mu, double *g, int64_t nx, int64_t ny, int64_t nz,
                                cudaStream_t st)
 {
-    // set once (thread-safe); 0 if the attribute could not be set
-    static const int res = []() -> int {
-        if (cudaFuncSetAttribute(wave25_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(WaveSmem)) != cudaSuccess)
-            return 0;
-        return resident((const void *)wave25_kernel<1>, kTX * kWaveTY, sizeof(WaveSmem));
-    }();
-    if (res <= 0)
-        return cudaErrorInvalidValue;
-    const int64_t gx = (nx + kSeg - 1) / kSeg, gy = (ny + kWaveTY - 1) / kWaveTY;
-    const int64_t chunk = choose_chunk(gx * gy, nz, 16, 9, res);
-    const int64_t gz = (nz + chunk - 1) / chunk;
-    if (gx * gy > 0x7fffffffll || nz > (1ll << 30))
-        return cudaErrorInvalidValue;
-    return launch(false, wave25_kernel<1>, dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWaveTY),
-                      sizeof(WaveSmem), st,
-        p, mu, (float *)nullptr, (const float *)nullptr, (int)nz, 0, Grid3{nx, ny, nz, nx * ny}, 0, nz, chunk, -1, -1, -1, 0.0f, g,
-        WaveSrcTable{}, (float *)nullptr);
+    return run_wave25<1>(false, p, mu, nullptr, nullptr, nz, 0, nx, ny, nz, 0, nz, -1, -1, -1, 0.0f, g,
+                         WaveSrcTable{}, nullptr, nullptr, nullptr, false, st);
 }
 
-cudaError_t launch_wave25_grad32(const float *p, const float *mu, float *gacc, int64_t nx, int64_t ny, int64_t nz,
-                                 cudaStream_t st)
+cudaError_t launch_wave25_lap(const float *p, const float *pprev, float *pnew, const float *kappa, float *lap,
+                              int64_t nx, int64_t ny, int64_t nz, int64_t sx, int64_t sy, int64_t sz, float w,
+                              cudaStream_t st)
 {
-    // set once (thread-safe); 0 if the attribute could not be set
-    static const int res = []() -> int {
-        if (cudaFuncSetAttribute(wave25_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(WaveSmem)) != cudaSuccess)
-            return 0;
-        return resident((const void *)wave25_kernel<2>, kTX * kWaveTY, sizeof(WaveSmem));
-    }();
-    if (res <= 0)
-        return cudaErrorInvalidValue;
-    const int64_t gx = (nx + kSeg - 1) / kSeg, gy = (ny + kWaveTY - 1) / kWaveTY;
-    const int64_t chunk = choose_chunk(gx * gy, nz, 16, 9, res);
-    const int64_t gz = (nz + chunk - 1) / chunk;
-    if (gx * gy > 0x7fffffffll || nz > (1ll << 30))
-        return cudaErrorInvalidValue;
-    return launch(true, wave25_kernel<2>, dim3((unsigned)(gx * gy), (unsigned)gz), dim3(kTX, kWaveTY),
-                      sizeof(WaveSmem), st,
-        p, mu, (float *)nullptr, (const float *)nullptr, (int)nz, 0, Grid3{nx, ny, nz, nx * ny}, 0, nz, chunk, -1, -1, -1, 0.0f, (double *)nullptr,
-        WaveSrcTable{}, gacc);
+    return run_wave25<2>(true, p, pprev, pnew, kappa, nz, 0, nx, ny, nz, 0, nz, sx, sy, sz, w, nullptr,
+                         WaveSrcTable{}, lap, nullptr, nullptr, false, st);
+}
+
+cudaError_t launch_wave25_gacc(const float *p, float *pprev_out, const float *kappa, const float *lap_pprev,
+                               const float *lap_p, float *gacc, bool fresh, int64_t nx, int64_t ny, int64_t nz,
+                               cudaStream_t st)
+{
+    return run_wave25<3>(true, p, pprev_out, pprev_out, kappa, nz, 0, nx, ny, nz, 0, nz, -1, -1, -1, 0.0f, nullptr,
+                         WaveSrcTable{}, const_cast<float *>(lap_pprev), lap_p, gacc, fresh, st);
 }
 
 cudaError_t launch_wave25(ConstRing p, Ring pprev_out, ConstRing kappa, int64_t nx, int64_t ny, int64_t nz,
