@@ -38,6 +38,7 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "div64.cuh"
 #include "host_wait.cuh"
 
 using namespace ooc;
@@ -68,6 +69,13 @@ __device__ unsigned g_receivers_bad = 0u;
 constexpr int kTX = 32, kTY = 8, kSeg = 4 * kTX, kR = 4;
 
 __device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+// 1 / x to 2^-23 (x normal)
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 __device__ __forceinline__ float4 mul4(float4 a, float4 b) { return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w); }
 
 // Adjoint step in its mu form on dense fields (plane z at z * nx * ny):
@@ -232,23 +240,27 @@ __global__ void check_indices_kernel(const int64_t *__restrict__ idx, int64_t n,
 }
 
 // A segment's FP32 gradient sum a (nullptr: 0) and its last one or two terms,
-// w1 l1 (w1 may be nullptr) and w0 l0, into the FP64 total g.
-__global__ void flush_segment_kernel(double *__restrict__ g, const float *__restrict__ a,
+// w1 l1 (w1 may be nullptr) and w0 l0, into the FP64 total g; `fresh`: g is
+// written, not added to (the first flush).  The last one (kap given) also
+// divides by kappa: in integers, since the FP64 division of 256^3 points took
+// 627 us of the FP64 pipe, and the flush hides it under its 36 bytes per
+// point (86 us with or without).
+__global__ void flush_segment_kernel(double *__restrict__ g, bool fresh, const float *__restrict__ a,
                                      const float *__restrict__ w1, const float *__restrict__ l1,
-                                     const float *__restrict__ w0, const float *__restrict__ l0, int64_t n)
+                                     const float *__restrict__ w0, const float *__restrict__ l0,
+                                     const float *__restrict__ kap, int64_t n)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         float s = a ? a[i] : 0.0f;
         if (w1)
             s = __fmaf_rn(w1[i], l1[i], s);
-        g[i] += (double)__fmaf_rn(w0[i], l0[i], s);
+        double t = (fresh ? 0.0 : g[i]) + widen(__fmaf_rn(w0[i], l0[i], s));
+        if (kap) {
+            const float k = kap[i];
+            t = div_f64_f32(t, k, rcp_approx(significand(k)));
+        }
+        g[i] = t;
     }
-}
-
-__global__ void divide_by_kappa_kernel(double *g, const float *__restrict__ kap, int64_t n)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        g[i] /= (double)kap[i];
 }
 
 __global__ void kappa_kernel(const float *__restrict__ v, float *__restrict__ kappa, int64_t n, float c)
@@ -259,11 +271,13 @@ __global__ void kappa_kernel(const float *__restrict__ v, float *__restrict__ ka
     }
 }
 
+// Two FP64 multiplies and one conversion per point (256^3: 157 us with two
+// conversions and three multiplies, 97 us so; its traffic takes 40).
 __global__ void grad_v_kernel(const double *__restrict__ gk, const float *__restrict__ v, float *__restrict__ gv,
                               int64_t n, double c2)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        gv[i] = (float)(gk[i] * 2.0 * (double)v[i] * c2);
+        gv[i] = (float)(gk[i] * widen(v[i]) * c2);
 }
 
 unsigned grid1d(int64_t n, int threads)
@@ -441,7 +455,7 @@ ooc_status ooc_velocity_grad(const double *d_grad_kappa, const float *d_v, float
     if (n == 0)
         return OOC_OK;
     grad_v_kernel<<<grid1d(n, 256), 256, 0, (cudaStream_t)stream>>>(d_grad_kappa, d_v, d_grad_v, n,
-                                                                   dt_over_dx * dt_over_dx);
+                                                                   2.0 * (dt_over_dx * dt_over_dx));
     return cudaGetLastError() == cudaSuccess ? OOC_OK : OOC_E_CUDA;
 }
 
@@ -552,7 +566,6 @@ ooc_status ooc_wave25_backward_ckpt(const float *d_kappa, int64_t nx, int64_t ny
     }
     TRY_CUDA(cudaMemsetAsync(mu1, 0, sizeof(float) * n, sC));
     TRY_CUDA(cudaMemsetAsync(mu2, 0, sizeof(float) * n, sC));
-    TRY_CUDA(cudaMemsetAsync(d_grad, 0, sizeof(double) * n, sC));
     const bool src = sx >= 0 && h_w != nullptr;
     const int64_t nseg = (nsteps + every - 1) / every;
     auto load = [&](int64_t k) -> cudaError_t {  // checkpoint k -> staging (k & 1), on sD
@@ -616,13 +629,12 @@ ooc_status ooc_wave25_backward_ckpt(const float *d_kappa, int64_t nx, int64_t ny
         }
         // the segment's sum (at most `every` terms) into the FP64 total, with
         // its last terms: w^{n0+2} L(p^{n0+1}) if len is even, w^{n0+1} L(p^{n0})
-        flush_segment_kernel<<<grid1d(n, 256), 256, 0, sC>>>(d_grad, len > 2 ? gacc : nullptr,
-                                                             len % 2 ? nullptr : mu2, len % 2 ? nullptr : lap(1), mu1,
-                                                             lap(0), n);
+        // the last segment's flush also divides by kappa
+        flush_segment_kernel<<<grid1d(n, 256), 256, 0, sC>>>(
+            d_grad, k == nseg - 1, len > 2 ? gacc : nullptr, len % 2 ? nullptr : mu2, len % 2 ? nullptr : lap(1), mu1,
+            lap(0), k == 0 ? d_kappa : nullptr, n);
         TRY_CUDA(cudaGetLastError());
     }
-    divide_by_kappa_kernel<<<grid1d(n, 256), 256, 0, sC>>>(d_grad, d_kappa, n);
-    TRY_CUDA(cudaGetLastError());
     TRY_CUDA(cudaEventRecord(ev.e[4], sC));
     TRY_CUDA(cudaEventRecord(ev.e[5], sD));
     ooc_status st = wait_event(ev.e[4], 600000);
