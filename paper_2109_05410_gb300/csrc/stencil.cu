@@ -522,13 +522,21 @@ OOC_PRAGMA(unroll OOC_HEATX2_UNROLL)
 // each side, plus the 4-point groups beyond the own rows' ends) in kWavePS
 // stages, and p_prev / kappa of the own rows in kWaveKS stages.  The copy
 // group of plane g, issued kWaveLead planes before g is the centre, carries
-// the p tile of g and p_prev / kappa of plane g - kWaveLead + 2.  The z-loop
-// runs in rounds of 9 planes, so that the 9-plane z-queue and both stage
-// rings are indexed by constants: the queue rotates by renaming, not by
-// register copies.
+// the p tile of g and p_prev / kappa of plane g - kWaveLead + kWaveKS - 1:
+// at the time of a plane's barrier, p is in flight for 4 planes beyond the
+// queue's last and p_prev / kappa for 3.  The z-loop runs in rounds of 9
+// planes, so that the 9-plane z-queue and the p stages are indexed by
+// constants: the queue rotates by renaming, not by register copies.
+// What bounds it: with p_prev / kappa only 2 planes ahead the latency of
+// those copies did (512^3 360 us per step); 3 ahead in a fourth stage, two
+// CTAs still fitting an SM, it is 331 us, 6.5 TB/s (256^3 52.1 -> 49.9, 60 x
+// 512^2 49.0 -> 47.2, where 256 CTAs fill 304 places once and instructions
+// and shared memory bind).  Also measured: p 3 and p_prev / kappa 4 planes
+// ahead, or all stages indexed at run time, 342; p_prev / kappa straight into
+// registers one plane ahead 484; rounds of 8 planes 342.
 constexpr int kWaveR = 4;
 constexpr int kWavePS = 9;
-constexpr int kWaveKS = 3;
+constexpr int kWaveKS = 4;
 constexpr int kWaveLead = 8;
 struct WaveSmem {
     float4 p[kWavePS][kWaveTY + 2 * kWaveR][kTX];
@@ -560,7 +568,8 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
                   const float *__restrict__ lap2, float *__restrict__ gacc, bool fresh)
 {
     constexpr int R = kWaveR;
-    static_assert(kWavePS == 2 * R + 1 && kWavePS % kWaveKS == 0 && kWaveLead == kWavePS - 1, "stage geometry");
+    static_assert(kWavePS == 2 * R + 1 && kWaveLead == kWavePS - 1 && (kWaveKS & (kWaveKS - 1)) == 0 &&
+                      kWaveKS - 2 <= kWaveLead - R - 1, "stage geometry");
     extern __shared__ __align__(16) unsigned char wave_smem[];
     WaveSmem &sm = *reinterpret_cast<WaveSmem *>(wave_smem);
     pdl_begin();
@@ -594,16 +603,18 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
     const bool step_on = MODE != 2 || pout != nullptr;
     const float4 z4 = zero4();
 
-    // Copy group of plane gz into p stage ST and, with K, p_prev / kappa of
-    // plane gz - kWaveLead + 2 into stage KST.  Copies past the chunk's last
-    // use are skipped (the group stays, empty, so that the counts hold).
+    // Copy group of plane za + gi into p stage ST and, with_k, p_prev / kappa
+    // of plane za + gi - kWaveLead + kWaveKS - 1.  Copies past the chunk's
+    // last use are skipped (the group stays, empty, so that the counts hold).
     // The p slot advances with every group, the p_prev / kappa slot with
     // every group that carries them.
     int ps = (int)ring_slot(za, zbase, nslot), ks = ps, os = ps;
-    auto issue = [&](auto st_c, auto kst_c, int64_t gz, bool with_k) {
-        constexpr int ST = decltype(st_c)::value, KST = decltype(kst_c)::value;
-        if (gz < zend + R) {
-            const bool vz = gz < nz;
+    const int nzr = (int)min(nz - za, (int64_t)1 << 30);  // planes from za to the grid's end
+    int kst = 0, kld = 0;  // K stage of the next copy and of plane z
+    auto issue = [&](auto st_c, int gi, bool with_k) {
+        constexpr int ST = decltype(st_c)::value;
+        if (gi < cnt + R) {
+            const bool vz = gi < nzr;
             const float *pl = pin + (int64_t)ps * plane;
             cp_async16(&sm.p[ST][ty][lane], pl + offa, vz && va);
             if (has_b)
@@ -613,13 +624,14 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
         }
         ps = wrap_add(ps, 1, nslot);
         if (with_k) {
-            if (gz - kWaveLead + 2 < zend) {
+            if (gi - (kWaveLead - kWaveKS + 1) < cnt) {
                 const int64_t kb = (int64_t)ks * plane;
-                cp_async16(&sm.pp[KST][ty][lane], pprev + kb + off, inside && step_on);
+                cp_async16(&sm.pp[kst][ty][lane], pprev + kb + off, inside && step_on);
                 if (MODE != 1)
-                    cp_async16(&sm.kk[KST][ty][lane], kap + kb + off, inside && step_on);
+                    cp_async16(&sm.kk[kst][ty][lane], kap + kb + off, inside && step_on);
             }
             ks = wrap_add(ks, 1, nslot);
+            kst = (kst + 1) & (kWaveKS - 1);
         }
         cp_async_commit();
     };
@@ -634,24 +646,24 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
         const float *pj = pin + (int64_t)wrap_add(os, nslot - R + j >= nslot ? j - R : nslot - R + j, nslot) * plane;
         q[j] = (inside && zj >= 0 && zj < nz) ? ldg4(pj + off) : z4;
     }
-    issue(IC<0>{}, IC<0>{}, za + 0, false);
-    issue(IC<1>{}, IC<0>{}, za + 1, false);
-    issue(IC<2>{}, IC<0>{}, za + 2, false);
-    issue(IC<3>{}, IC<0>{}, za + 3, false);
-    issue(IC<4>{}, IC<0>{}, za + 4, false);
-    issue(IC<5>{}, IC<0>{}, za + 5, false);
-    issue(IC<6>{}, IC<0>{}, za + 6, true);
-    issue(IC<7>{}, IC<1>{}, za + 7, true);
+    issue(IC<0>{}, 0, false);
+    issue(IC<1>{}, 1, false);
+    issue(IC<2>{}, 2, false);
+    issue(IC<3>{}, 3, false);
+    issue(IC<4>{}, 4, false);
+    issue(IC<5>{}, 5, true);
+    issue(IC<6>{}, 6, true);
+    issue(IC<7>{}, 7, true);
 
-    int64_t z = za;
+    const int isz = src_here && sz >= za && sz < zend ? (int)(sz - za) : -1;
     int base = 0;  // first iteration of the current round
     auto step = [&](auto ph_c) {
         constexpr int PH = decltype(ph_c)::value;  // iteration mod 9: stage of plane z
         if (base + PH >= cnt)
             return;
-        cp_async_wait<1>();  // groups up to plane z + 6 have landed (p tile of z + 4, p_prev / kappa of z)
+        cp_async_wait<kWaveKS - 2>();  // groups up to plane z + 5 have landed (p tile of z + 4, p_prev / kappa of z)
         __syncthreads();     // ... for every thread; the stages of plane z - 1 are free
-        issue(IC<(PH + kWaveLead) % kWavePS>{}, IC<(PH + 2) % kWaveKS>{}, z + kWaveLead, true);
+        issue(IC<(PH + kWaveLead) % kWavePS>{}, base + PH + kWaveLead, true);
         // MODE 3: read here, used after the Laplacian
         const int64_t own = (int64_t)os * plane + off;
         const float4 la = MODE == 3 ? ldg4(lapf + own) : z4;
@@ -672,8 +684,9 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
             lf = sm.xh[PH][ty][0];
         if (lane == kTX - 1)
             rt = sm.xh[PH][ty][1];
-        const float4 ppv = sm.pp[PH % kWaveKS][ty][lane];
-        const float4 kv = MODE != 1 ? sm.kk[PH % kWaveKS][ty][lane] : z4;
+        const float4 ppv = sm.pp[kld][ty][lane];
+        const float4 kv = MODE != 1 ? sm.kk[kld][ty][lane] : z4;
+        kld = (kld + 1) & (kWaveKS - 1);
         const float L[4] = {lf.x, lf.y, lf.z, lf.w};
         const float C[4] = {c.x, c.y, c.z, c.w};
         const float Rt[4] = {rt.x, rt.y, rt.z, rt.w};
@@ -733,7 +746,7 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 o[j] = __fmaf_rn(KV[j], lap[j], __fmaf_rn(2.0f, C[j], -PP[j]));
-            if (src_here && z == sz) {
+            if (base + PH == isz) {
                 float ws = w;
                 if (tab.w) {  // amplitude of step n = plan time + n_off, from the device table
                     const int64_t n = *tab.t + tab.n_off;
@@ -766,7 +779,6 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
             gp[1] = g1;
         }
         os = wrap_add(os, 1, nslot);
-        ++z;
     };
 #pragma unroll 1
     for (; base < cnt; base += kWavePS) {
