@@ -23,7 +23,7 @@
 //
 // The kernels are bound by the integer ALU pipe (78-80 % busy, against 23-27 %
 // of DRAM), which issues half of what the schedulers do.  56 planes of 1024^2,
-// R = 8, 16, 24, us: encode 196, 224, 241 -> 138, 150, 165; decode 196, 236,
+// R = 8, 16, 24, us: encode 196, 224, 241 -> 134, 148, 164; decode 196, 236,
 // 261 -> 142, 166, 179, against a plane loop that wrote its fields by
 // read-modify-write and parsed the new ones segment by segment (22 of 32
 // lanes active).  The transform and the transposes alone take 92 and 80 us.
@@ -31,7 +31,11 @@
 // registers (no shared memory for them, but its code overflows the
 // instruction cache: 230 us; with a plane as a called function 208), all 32
 // masks of a block in shared memory at once (16 warps per SM instead of 24:
-// 216).
+// 216).  For the encoder: a plane's new ones through a 256-entry table in
+// place of insert_ones' loop (148 -> 165: a plane of a smooth field has one or
+// none).  Of the encoder's 4506 instructions per warp 877 load, convert and
+// store (62 us by themselves), 340 transform, 720 transpose and 2570 code the
+// planes.
 //
 // Also here: dense-field kernels for any shape (partial blocks padded with
 // the nearest inside value) and the variable-size fixed-precision and
@@ -400,10 +404,13 @@ __device__ __forceinline__ void clear_tail(uint32_t *dst, int off, int words)
 __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mode, int mparam, uint32_t *dst,
                                             uint32_t *pm)
 {
-    uint32_t mx = 0;
+    // the largest magnitude, three values per instruction (any NaN gives one
+    // with the same exponent)
+    float top = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 64; ++i)
-        mx = max(mx, v[i] & 0x7FFFFFFFu);
+    for (int i = 0; i < 64; i += 2)
+        asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(top) : "f"(__uint_as_float(v[i])), "f"(__uint_as_float(v[i + 1])));
+    const uint32_t mx = __float_as_uint(top);
     const int budget = 32 * words;
     if (mx == 0u) {
         dst[0] = 0u;
@@ -428,14 +435,14 @@ __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mo
 
     transform_fwd(q);
     to_coding_order(v, q, std::make_integer_sequence<int, 64>{});
-    // the leading planes without a one, a group bit 0 each
-    uint32_t any = 0u;
-#pragma unroll
-    for (int i = 0; i < 64; ++i)
-        any |= v[i] ^ kNB;
-    const int skip = min(__clz((int)any), 32 - pmin);
     to_planes32<0>(v);   // v[p]      = bits p of coefficients 0..31
     to_planes32<32>(v);  // v[32 + p] = bits p of coefficients 32..63
+    // the leading planes without a one (up to 8 of them), a group bit 0 each
+    int skip = 8;
+#pragma unroll
+    for (int i = 7; i >= 0; --i)
+        skip = (v[31 - i] | v[63 - i]) != 0u ? i : skip;
+    skip = min(skip, 32 - pmin);
     dst[0] = 1u | ((uint32_t)((emax + 127) & 0xFF) << 1);
     dst[1] = 0u;
     CodePos c{0, 9 + skip};

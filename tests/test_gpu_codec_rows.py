@@ -74,3 +74,23 @@ def test_variable_decoder_rounds(ooc, kind):
     out = ooc.ooc_decompress_var(got, torch.from_numpy(index2.astype(np.int64)).cuda(), f.shape, 1, 32)
     torch.cuda.synchronize()
     assert out.shape == f.shape
+
+
+def test_block_exponents_of_special_values(ooc):
+    # a block's header holds the exponent of its largest bit pattern without
+    # the sign: zeros, subnormals, the largest values, infinities and NaN of
+    # any payload
+    specials = np.array([0x00000000, 0x80000000, 0x00000001, 0x80000001, 0x007fffff, 0x00800000, 0x3f800000,
+                         0xff7fffff, 0x7f800000, 0xff800000, 0x7fc00000, 0xffc00001, 0x7f800001], dtype=np.uint32)
+    rng = np.random.default_rng(8)
+    blocks = np.zeros((2 * specials.size, 64), dtype=np.uint32)
+    for i, v in enumerate(specials):  # alone, and among smaller ones
+        blocks[2 * i, rng.integers(64)] = v
+        m = (int(v) & 0x7fffffff) >> 23
+        blocks[2 * i + 1] = rng.integers(0, max(m, 1) << 23, 64).astype(np.uint32) if m else 0
+        blocks[2 * i + 1, rng.integers(64)] = v
+    mx = (blocks & 0x7fffffff).max(axis=1)
+    want = np.where(mx == 0, 0, 1 | (((mx >> 23) + 1 & 0xff) << 1))
+    f = blocks.reshape(-1, 4, 4, 4).transpose(1, 2, 0, 3).reshape(4, 4, -1).view(np.float32)
+    words = ooc.ooc_compress(torch.from_numpy(np.ascontiguousarray(f)).cuda(), 16).cpu().numpy().view(np.uint32)
+    assert np.array_equal(words.reshape(-1, 32)[:, 0] & 0x1ff, want)
