@@ -23,7 +23,7 @@
 //
 // The kernels are bound by the integer ALU pipe (78-80 % busy, against 23-27 %
 // of DRAM), which issues half of what the schedulers do.  56 planes of 1024^2,
-// R = 8, 16, 24, us: encode 196, 224, 241 -> 134, 148, 164; decode 196, 236,
+// R = 8, 16, 24, us: encode 196, 224, 241 -> 126, 141, 157; decode 196, 236,
 // 261 -> 142, 166, 179, against a plane loop that wrote its fields by
 // read-modify-write and parsed the new ones segment by segment (22 of 32
 // lanes active).  The transform and the transposes alone take 92 and 80 us.
@@ -33,9 +33,12 @@
 // masks of a block in shared memory at once (16 warps per SM instead of 24:
 // 216).  For the encoder: a plane's new ones through a 256-entry table in
 // place of insert_ones' loop (148 -> 165: a plane of a smooth field has one or
-// none).  Of the encoder's 4506 instructions per warp 877 load, convert and
-// store (62 us by themselves), 340 transform, 720 transpose and 2570 code the
-// planes.
+// none); the refinement bits and the new ones of every plane as one field
+// (145).  For the decoder: the first planes apart as the encoder does
+// (code_planes; 142, 166, 179 -> 140, 165, 177, but 138, 167, 188 -> 140, 169,
+// 189 on rougher fields).  Of the encoder's instructions per warp 877 load,
+// convert and store (62 us by themselves), 340 transform, 720 transpose and
+// 2300 code the planes.
 //
 // Also here: dense-field kernels for any shape (partial blocks padded with
 // the nearest inside value) and the variable-size fixed-precision and
@@ -389,6 +392,49 @@ __device__ __forceinline__ CodePos code_plane(uint32_t *dst, uint32_t xl, uint32
     return CodePos{len, off + bits + (open ? 2 : 0)};
 }
 
+__device__ __forceinline__ uint32_t shl32(uint32_t v, int n)  // n >= 0; 0 for n >= 32
+{
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+    return r;
+}
+__device__ __forceinline__ uint32_t shr32(uint32_t v, int n)
+{
+    uint32_t r;
+    asm("shr.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+    return r;
+}
+
+// Planes p .. stop, whose masks are at pb[p] and pb[16 + p].  FIRST (the first
+// 16 planes of a block): the leading ones take few bits, and as long as a
+// plane of every lane's block fits 32 (and the coefficients 32..63 have no one
+// yet), it is written as one field.  On smooth fields these are 10 to 12 of
+// 28 planes: R = 16 148 -> 141 us, 139 -> 138 on rough ones; in the later
+// parts too it gains nothing there and costs 2 %.  The vote only chooses
+// between two ways to the same bits, so it may be taken by any set of lanes.
+template <bool FIRST>
+__device__ __forceinline__ CodePos code_planes(uint32_t *dst, const uint32_t *pb, int &p, int stop, int budget, CodePos c)
+{
+#pragma unroll 1
+    for (; FIRST && p >= stop && c.off < budget; --p) {
+        const uint32_t x = pb[p];
+        const uint32_t s = shr32(x, c.n);  // new ones; 0: tl = -1, bits = -1
+        const int tl = 31 - __clz((int)s), bits = tl + __popc((int)s);
+        const bool fits = pb[16 + p] == 0u && c.n + bits + 2 <= 32;
+        if (__any_sync(__activemask(), !fits))
+            break;
+        const uint32_t v = insert_ones(s, s ^ (1u << (tl & 31)));
+        const uint32_t field = (v << 1) | (s != 0u ? 1u : 0u);
+        put32(dst, c.off, (x & ~shl32(~0u, c.n)) | shl32(field, c.n));
+        c.off += c.n + bits + 2;
+        c.n += tl + 1;
+    }
+#pragma unroll 1
+    for (; p >= stop && c.off < budget; --p)
+        c = code_plane(dst, pb[p], pb[16 + p], c.n, c.off);
+    return c;
+}
+
 // The words behind the coded bits up to the block's `words`.
 __device__ __forceinline__ void clear_tail(uint32_t *dst, int off, int words)
 {
@@ -447,25 +493,24 @@ __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mo
     dst[1] = 0u;
     CodePos c{0, 9 + skip};
     int p = 31 - skip;
-    auto code_half = [&](int base) {  // planes base + 15 .. base
+    auto code_half = [&](auto base_c) {  // planes base + 15 .. base
+        constexpr int base = decltype(base_c)::value;
         const int stop = max(pmin, base);
         const uint32_t *pb = pm - base;
-#pragma unroll 1
-        for (; p >= stop && c.off < budget; --p)
-            c = code_plane(dst, pb[p], pb[16 + p], c.n, c.off);
+        c = code_planes<base != 0>(dst, pb, p, stop, budget, c);
     };
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         pm[i] = v[16 + i];
         pm[16 + i] = v[48 + i];
     }
-    code_half(16);
+    code_half(std::integral_constant<int, 16>{});
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         pm[i] = v[i];
         pm[16 + i] = v[32 + i];
     }
-    code_half(0);
+    code_half(std::integral_constant<int, 0>{});
     if (mode == OOC_FR4_RATE)
         clear_tail(dst, c.off, words);
     return c.off;
@@ -966,7 +1011,8 @@ __device__ __forceinline__ void encode_block64(const uint64_t (&v)[64], int word
     CodePos c{0, 12 + skip};
     int p = 63 - skip;
     // planes base + 15 .. base, whose masks are in a[at ..] and a[at + 32 ..]
-    auto code_part = [&](int base, const uint32_t (&a)[64], auto at_c) {
+    auto code_part = [&](auto base_c, const uint32_t (&a)[64], auto at_c) {
+        constexpr int base = decltype(base_c)::value;
         constexpr int at = decltype(at_c)::value;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
@@ -974,19 +1020,17 @@ __device__ __forceinline__ void encode_block64(const uint64_t (&v)[64], int word
             pm[16 + i] = a[32 + at + i];
         }
         const uint32_t *pb = pm - base;
-#pragma unroll 1
-        for (; p >= base && c.off < 32 * words; --p)
-            c = code_plane(dst, pb[p], pb[16 + p], c.n, c.off);
+        c = code_planes<base == 48>(dst, pb, p, base, 32 * words, c);
     };
     to_planes32<0>(hi);
     to_planes32<32>(hi);
-    code_part(48, hi, std::integral_constant<int, 16>{});
-    code_part(32, hi, std::integral_constant<int, 0>{});
+    code_part(std::integral_constant<int, 48>{}, hi, std::integral_constant<int, 16>{});
+    code_part(std::integral_constant<int, 32>{}, hi, std::integral_constant<int, 0>{});
     if (c.off < 32 * words) {
         to_planes32<0>(lo);
         to_planes32<32>(lo);
-        code_part(16, lo, std::integral_constant<int, 16>{});
-        code_part(0, lo, std::integral_constant<int, 0>{});
+        code_part(std::integral_constant<int, 16>{}, lo, std::integral_constant<int, 16>{});
+        code_part(std::integral_constant<int, 0>{}, lo, std::integral_constant<int, 0>{});
     }
     clear_tail(dst, c.off, words);
 }

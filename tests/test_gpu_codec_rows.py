@@ -94,3 +94,17 @@ def test_block_exponents_of_special_values(ooc):
     f = blocks.reshape(-1, 4, 4, 4).transpose(1, 2, 0, 3).reshape(4, 4, -1).view(np.float32)
     words = ooc.ooc_compress(torch.from_numpy(np.ascontiguousarray(f)).cuda(), 16).cpu().numpy().view(np.uint32)
     assert np.array_equal(words.reshape(-1, 32)[:, 0] & 0x1ff, want)
+
+
+@pytest.mark.parametrize("rate", [1, 3, 9, 16, 40, 64])
+def test_first_planes_of_mixed_warps(ooc, rate):
+    # neighbouring blocks from constant to rough, so that the lanes of a warp
+    # leave the encoder's one-field planes at different ones, or never do
+    rng = np.random.default_rng(rate)
+    f = np.broadcast_to(np.linspace(-1, 1.5, 4 * 67, dtype=np.float32), (8, 4, 4 * 67)).copy()
+    rough = rng.standard_normal(f.shape).astype(np.float32) * np.repeat(np.float32(2.0) ** -rng.integers(0, 40, 67), 4)
+    f += rough.astype(np.float32)
+    f[:, :, 40:44] = 0.25
+    f[4:, :, 96:100] = 0.0
+    ref = oracle.fr4_encode(f, rate)
+    assert np.array_equal(ooc.ooc_compress(on_gpu(f, 0), rate).cpu().numpy().view(np.uint32), ref)
