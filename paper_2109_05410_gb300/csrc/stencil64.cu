@@ -43,8 +43,9 @@
 // against 815).
 //
 // Measured, us per step at 384^3 (G point-steps/s), FP64 instructions against
-// integer sums: wave25 3200 (17.7) and 915 (62); heat7 775 (73) and 317
-// (179).  A wave from rest, whose steep precursors take the FP64 instructions
+// integer sums: wave25 3200 (17.7) and 881 (64); heat7 775 (73) and 288
+// (197; 309 while all-zero stencils had FP64 instructions of their own, which
+// issue on that pipe for every stencil once predicated).  A wave from rest, whose steep precursors take the FP64 instructions
 // in part: 1.07 ms per 256^3 step against 0.30 to 1.08, by phase; neighbours
 // 2^60 apart at random, which nearly all take them: 1.36 against 1.38 ms
 // (heat7 0.315 against 0.403).  Bound now: wave25 by the ALU pipe and
@@ -188,10 +189,15 @@ __global__ void __launch_bounds__(kTX *kTY64, 7)
     Fx2 fc = to_fx(cur);
     double2 nxt = (inside && za + 1 < nz) ? ldg2(p1 + off) : z2;
     double2 hv = hin ? ldg2(p0 + hoff) : z2;
+    // offsets of the planes z and z + 1; planes from za to the grid's end
+    int64_t o0 = (int64_t)s0 * plane, o1 = (int64_t)s1 * plane;
+    const int left = (int)min(nz - za, (int64_t)1 << 30);
+    const double *in_own = in + off, *in_halo = in + hoff;
+    double *out_own = out + off;
 #pragma unroll 2
     for (int i = 0; i < cnt; ++i) {
-        const int64_t z = za + i;
         const int s2 = wrap_add(s1, 1, nslot);
+        const int64_t o2 = s2 == 0 ? 0 : o1 + plane;
         const int b = i & 1;
         tm[b][ty + 1][lane + 1] = make_longlong2(fc.a, fc.b);
         te[b][ty + 1][lane + 1] = fc.e;
@@ -201,8 +207,8 @@ __global__ void __launch_bounds__(kTX *kTY64, 7)
             te[b][hr][hc] = h.e;
         }
         // the next planes' loads, a plane ahead of their use
-        const double2 nn = (inside && z + 2 < nz) ? ldg2(in + (int64_t)s2 * plane + off) : z2;
-        hv = (hin && z + 1 < nz) ? ldg2(in + (int64_t)s1 * plane + hoff) : z2;
+        const double2 nn = (inside && i + 2 < left) ? ldg2(in_own + o2) : z2;
+        hv = (hin && i + 1 < left) ? ldg2(in_halo + o1) : z2;
         const Fx2 fp = to_fx(nxt);
         __syncthreads();
         const longlong2 up = tm[b][ty][lane + 1], dn = tm[b][ty + 2][lane + 1];
@@ -211,12 +217,9 @@ __global__ void __launch_bounds__(kTX *kTY64, 7)
         const uint32_t el = te[b][ty + 1][lane], er = te[b][ty + 1][lane + 2];
         const uint32_t E = max(max(max(fm.e, fc.e), max(fp.e, eu)), max(max(ed, el), er));
         double2 o;
-        bool exact = E >= kELo && E <= kEHi;
-        if (E == 0u) {  // all zeros
-            exact = true;
-            o.x = __fma_rn(r, 0.0, cur.x);
-            o.y = __fma_rn(r, 0.0, cur.y);
-        } else if (exact) {
+        const bool zeros = E == 0u;
+        bool exact = zeros || (E >= kELo && E <= kEHi);
+        if (exact) {
             const uint32_t et = E + 4u;
             const long long ca = sar64(fc.a, et - fc.e), cb = sar64(fc.b, et - fc.e);
             const long long za = sar64(fm.a, et - fm.e), zb = sar64(fm.b, et - fm.e);
@@ -224,27 +227,30 @@ __global__ void __launch_bounds__(kTX *kTY64, 7)
             const long long ua = sar64(up.x, et - eu), ub = sar64(up.y, et - eu);
             const long long da = sar64(dn.x, et - ed), db = sar64(dn.y, et - ed);
             const long long la = sar64(xl, et - el), rb = sar64(xr, et - er);
-            exact = (fx_big(ca) | fx_big(cb) | fx_big(za) | fx_big(wa) | fx_big(ua) | fx_big(da) | fx_big(la)) >
-                        kFxBig &&
-                    (fx_big(ca) | fx_big(cb) | fx_big(zb) | fx_big(wb) | fx_big(ub) | fx_big(db) | fx_big(rb)) >
-                        kFxBig;
+            exact = zeros ||
+                    ((fx_big(ca) | fx_big(cb) | fx_big(za) | fx_big(wa) | fx_big(ua) | fx_big(da) | fx_big(la)) >
+                         kFxBig &&
+                     (fx_big(ca) | fx_big(cb) | fx_big(zb) | fx_big(wb) | fx_big(ub) | fx_big(db) | fx_big(rb)) >
+                         kFxBig);
             const long long sa = (za + wa) + (ua + da) + (la + cb) - 6 * ca;
             const long long sb = (zb + wb) + (ub + db) + (rb + ca) - 6 * cb;
             const int k = (int)E - 1081;
-            o.x = __fma_rn(r, scale_exp(__ll2double_rn(sa), k), cur.x);
-            o.y = __fma_rn(r, scale_exp(__ll2double_rn(sb), k), cur.y);
+            o.x = __fma_rn(r, zeros ? 0.0 : scale_exp(__ll2double_rn(sa), k), cur.x);
+            o.y = __fma_rn(r, zeros ? 0.0 : scale_exp(__ll2double_rn(sb), k), cur.y);
         }
         if (!exact && inside) {
-            o = heat_pair_f64(in, s0, nslot, plane, off, g.nx, g.ny, nz, x2, y, z, r);
+            o = heat_pair_f64(in, s0, nslot, plane, off, g.nx, g.ny, nz, x2, y, za + i, r);
         }
         if (inside)
-            *reinterpret_cast<double2 *>(out + (int64_t)s0 * plane + off) = o;
+            *reinterpret_cast<double2 *>(out_own + o0) = o;
         fm = fc;
         fc = fp;
         cur = nxt;
         nxt = nn;
         s0 = s1;
         s1 = s2;
+        o0 = o1;
+        o1 = o2;
     }
 }
 
@@ -428,9 +434,13 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
     int ph = kWR;  // slot of plane z
     double2 hv = hrow ? ldg2(pin + (int64_t)s0 * plane + hoff) : z2;
     double2 xv = xhalo ? ldg2(pin + (int64_t)s0 * plane + xoff) : z2;
+    // offsets of the planes z, z + 1 and z + 5; planes from za to the grid's
+    // end; the source's plane
+    int64_t o0 = (int64_t)s0 * plane, o1 = (int64_t)s1 * plane, o5 = (int64_t)s5 * plane;
+    const int left = (int)min(nz - za, (int64_t)1 << 30);
+    const int isz = src_here && sz >= za && sz < za + cnt ? (int)(sz - za) : -1;
 #pragma unroll 9
     for (int i = 0; i < cnt; ++i) {
-        const int64_t z = za + i;
         const int b = i & 1;
         const longlong2 cm = sm.qm[ph][ty][lane];
         const uint32_t ce = sm.qe[ph][ty][lane];
@@ -449,10 +459,10 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
         // the next plane's halos and the queue's next plane, and this
         // plane's other operands, which are used last
         const bool more = i + 1 < cnt;
-        const int64_t b0 = (int64_t)s0 * plane + off, b1 = (int64_t)s1 * plane;
-        hv = (hrow && more) ? ldg2(pin + b1 + hoff) : z2;
-        xv = (xhalo && more) ? ldg2(pin + b1 + xoff) : z2;
-        const double2 qn = (inside && more && z + kWR + 1 < nz) ? ldg2(pin + (int64_t)s5 * plane + off) : z2;
+        const int64_t b0 = o0 + off;
+        hv = (hrow && more) ? ldg2(pin + hoff + o1) : z2;
+        xv = (xhalo && more) ? ldg2(pin + xoff + o1) : z2;
+        const double2 qn = (inside && more && i + kWR + 1 < left) ? ldg2(pin + off + o5) : z2;
         const double2 c = inside ? ldg2(pin + b0) : z2;
         const double2 kv = inside ? ldg2(kap + b0) : z2;
         // p_prev is overwritten by this kernel: plain loads, not the read-only path
@@ -539,12 +549,12 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
             exact = (onea > kW1 || sixa > kW6) && (oneb > kW1 || sixb > kW6);
         }
         if (!exact && inside) {
-            lap = wave_lap_pair_f64(pin, s0, nslot, plane, off, g.nx, g.ny, nz, x2, y, z);
+            lap = wave_lap_pair_f64(pin, s0, nslot, plane, off, g.nx, g.ny, nz, x2, y, za + i);
         }
         double2 o;
         o.x = __fma_rn(kv.x, lap.x, __fma_rn(2.0, c.x, -ppv.x));
         o.y = __fma_rn(kv.y, lap.y, __fma_rn(2.0, c.y, -ppv.y));
-        if (src_here && z == sz) {
+        if (i == isz) {
             double ws = w;
             if (tab.w) {  // amplitude of step n = plan time + n_off, from the device table
                 const int64_t n = *tab.t + tab.n_off;
@@ -556,7 +566,7 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
                 o.y = __dadd_rn(o.y, ws);
         }
         if (inside)
-            *reinterpret_cast<double2 *>(pout + (int64_t)s0 * plane + off) = o;
+            *reinterpret_cast<double2 *>(pout + b0) = o;
         // plane z + 5 into the slot of z - 4 (read by this thread alone)
         ++ph;
         put(ph + kWR < kWQ ? ph + kWR : ph + kWR - kWQ, to_fx(qn));
@@ -564,6 +574,9 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
         s0 = s1;
         s1 = s1 + 1 == nslot ? 0 : s1 + 1;
         s5 = s5 + 1 == nslot ? 0 : s5 + 1;
+        o0 = o1;
+        o1 = s1 == 0 ? 0 : o1 + plane;
+        o5 = s5 == 0 ? 0 : o5 + plane;
     }
 }
 
