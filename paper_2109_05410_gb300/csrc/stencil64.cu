@@ -43,12 +43,12 @@
 // against 815).
 //
 // Measured, us per step at 384^3 (G point-steps/s), FP64 instructions against
-// integer sums: wave25 3200 (17.7) and 881 (64); heat7 775 (73) and 288
-// (197; 309 while all-zero stencils had FP64 instructions of their own, which
+// integer sums: wave25 3200 (17.7) and 835 (68); heat7 775 (73) and 286
+// (198; 309 while all-zero stencils had FP64 instructions of their own, which
 // issue on that pipe for every stencil once predicated).  A wave from rest, whose steep precursors take the FP64 instructions
-// in part: 1.07 ms per 256^3 step against 0.30 to 1.08, by phase; neighbours
-// 2^60 apart at random, which nearly all take them: 1.36 against 1.38 ms
-// (heat7 0.315 against 0.403).  Bound now: wave25 by the ALU pipe and
+// in part: 1.07 ms per 256^3 step against 0.32 to 1.07, by phase; neighbours
+// 2^60 apart at random, which nearly all take them: 1.36 against 1.39 ms
+// (heat7 0.315 against 0.388).  Bound now: wave25 by the ALU pipe and
 // shared-memory wavefronts (each 55-63 % busy, about 600 instructions per 64
 // points), heat7 by the FP64 pipe (61 %) and the ALU pipe (55 %) with 28 warps
 // per SM.
@@ -218,8 +218,8 @@ __global__ void __launch_bounds__(kTX *kTY64, 7)
         const uint32_t E = max(max(max(fm.e, fc.e), max(fp.e, eu)), max(max(ed, el), er));
         double2 o;
         const bool zeros = E == 0u;
-        bool exact = zeros || (E >= kELo && E <= kEHi);
-        if (exact) {
+        bool exact = E >= kELo && E <= kEHi;
+        {  // run by every thread (branches around it cost more than they save)
             const uint32_t et = E + 4u;
             const long long ca = sar64(fc.a, et - fc.e), cb = sar64(fc.b, et - fc.e);
             const long long za = sar64(fm.a, et - fm.e), zb = sar64(fm.b, et - fm.e);
@@ -227,11 +227,9 @@ __global__ void __launch_bounds__(kTX *kTY64, 7)
             const long long ua = sar64(up.x, et - eu), ub = sar64(up.y, et - eu);
             const long long da = sar64(dn.x, et - ed), db = sar64(dn.y, et - ed);
             const long long la = sar64(xl, et - el), rb = sar64(xr, et - er);
-            exact = zeros ||
-                    ((fx_big(ca) | fx_big(cb) | fx_big(za) | fx_big(wa) | fx_big(ua) | fx_big(da) | fx_big(la)) >
-                         kFxBig &&
-                     (fx_big(ca) | fx_big(cb) | fx_big(zb) | fx_big(wb) | fx_big(ub) | fx_big(db) | fx_big(rb)) >
-                         kFxBig);
+            const uint32_t biga = fx_big(ca) | fx_big(cb) | fx_big(za) | fx_big(wa) | fx_big(ua) | fx_big(da) | fx_big(la);
+            const uint32_t bigb = fx_big(ca) | fx_big(cb) | fx_big(zb) | fx_big(wb) | fx_big(ub) | fx_big(db) | fx_big(rb);
+            exact = zeros || (exact && biga > kFxBig && bigb > kFxBig);
             const long long sa = (za + wa) + (ua + da) + (la + cb) - 6 * ca;
             const long long sb = (zb + wb) + (ub + db) + (rb + ca) - 6 * cb;
             const int k = (int)E - 1081;
@@ -500,7 +498,11 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
         }
         double2 lap = make_double2(0.0, 0.0);
         bool exact = Z == 0;  // all zeros
-        if (E >= (int)kELo && Z <= (int)kEHi) {
+        {
+            // run by every thread: without a branch the values' loads start
+            // ahead of the exponents' test (384^3 881 -> 835 us; all zeros
+            // 0.37 -> 0.44 ms per 256^3 step)
+            const bool range = E >= (int)kELo && Z <= (int)kEHi;
             const uint32_t et = (uint32_t)E + 3u;
             WaveAcc wa{0, kHalf, 0}, wb{0, kHalf, 0};
             // A row value at distance m of the first point is at m - 1 or
@@ -544,9 +546,9 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
             taps(std::integral_constant<int, 3>{});
             taps(std::integral_constant<int, 2>{});
             taps(std::integral_constant<int, 1>{});
-            lap.x = wave_finish(wa, ca, E);
-            lap.y = wave_finish(wb, cb, E);
-            exact = (onea > kW1 || sixa > kW6) && (oneb > kW1 || sixb > kW6);
+            lap.x = exact ? 0.0 : wave_finish(wa, ca, E);
+            lap.y = exact ? 0.0 : wave_finish(wb, cb, E);
+            exact = exact || (range && (onea > kW1 || sixa > kW6) && (oneb > kW1 || sixb > kW6));
         }
         if (!exact && inside) {
             lap = wave_lap_pair_f64(pin, s0, nslot, plane, off, g.nx, g.ny, nz, x2, y, za + i);
