@@ -23,7 +23,7 @@
 //
 // The kernels are bound by the integer ALU pipe (78-80 % busy, against 23-27 %
 // of DRAM), which issues half of what the schedulers do.  56 planes of 1024^2,
-// R = 8, 16, 24, us: encode 196, 224, 241 -> 126, 141, 157; decode 196, 236,
+// R = 8, 16, 24, us: encode 196, 224, 241 -> 126, 140, 144; decode 196, 236,
 // 261 -> 142, 166, 179, against a plane loop that wrote its fields by
 // read-modify-write and parsed the new ones segment by segment (22 of 32
 // lanes active).  The transform and the transposes alone take 92 and 80 us.
@@ -405,7 +405,7 @@ __device__ __forceinline__ uint32_t shr32(uint32_t v, int n)
     return r;
 }
 
-// Planes p .. stop, whose masks are at pb[p] and pb[16 + p].  FIRST (the first
+// Planes p .. stop, whose masks are at pb[-2 p] and pb[1 - 2 p].  FIRST (the first
 // 16 planes of a block): the leading ones take few bits, and as long as a
 // plane of every lane's block fits 32 (and the coefficients 32..63 have no one
 // yet), it is written as one field.  On smooth fields these are 10 to 12 of
@@ -417,10 +417,10 @@ __device__ __forceinline__ CodePos code_planes(uint32_t *dst, const uint32_t *pb
 {
 #pragma unroll 1
     for (; FIRST && p >= stop && c.off < budget; --p) {
-        const uint32_t x = pb[p];
+        const uint32_t x = pb[-2 * p];
         const uint32_t s = shr32(x, c.n);  // new ones; 0: tl = -1, bits = -1
         const int tl = 31 - __clz((int)s), bits = tl + __popc((int)s);
-        const bool fits = pb[16 + p] == 0u && c.n + bits + 2 <= 32;
+        const bool fits = pb[1 - 2 * p] == 0u && c.n + bits + 2 <= 32;
         if (__any_sync(__activemask(), !fits))
             break;
         const uint32_t v = insert_ones(s, s ^ (1u << (tl & 31)));
@@ -431,7 +431,7 @@ __device__ __forceinline__ CodePos code_planes(uint32_t *dst, const uint32_t *pb
     }
 #pragma unroll 1
     for (; p >= stop && c.off < budget; --p)
-        c = code_plane(dst, pb[p], pb[16 + p], c.n, c.off);
+        c = code_plane(dst, pb[-2 * p], pb[1 - 2 * p], c.n, c.off);
     return c;
 }
 
@@ -445,10 +445,38 @@ __device__ __forceinline__ void clear_tail(uint32_t *dst, int off, int words)
 // Encode one block into dst[0 .. words) (a bit budget of 32 words; words =
 // 2R at a fixed rate) with the plane range of `mode`.  Returns the coded
 // length in bits (exact for the variable-size modes, whose budget never
-// binds).  The planes go through the thread's 32 words at pm, 16 at a time:
-// half the shared memory of all 32 planes, for 24 warps per SM instead of 16.
-__device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mode, int mparam, uint32_t *dst,
-                                            uint32_t *pm)
+// binds).  The planes go through shared memory 16 at a time, in the part of
+// dst that the coded words have not reached yet: half the shared memory of
+// all 32 planes, and none beside the words, for 24 warps per SM at any rate
+// up to 32 and in the variable-size modes (with 33 words of their own per
+// thread it was 16 warps at R = 24, 157 us against 144, and 16 in the
+// variable-size encoder, 512^3 at tolerance 1e-4 530 against 475).
+//
+// Before plane 31 - j at most 73 + 65 j bits are coded (var_block_words), and
+// coding it touches words up to (138 + 65 j) / 32 + 1.  Its own two words are
+// read before; the next plane's are at kPlanes1 + 2 (j + 1) while j < 16, at
+// kPlanes0 + 2 (j - 15) after that, which is further for every j.  A budget of
+// `words` ends the coding within 129 bits of it, so that planes behind words +
+// 5 are out of reach whatever j is (R = 8: 55 words per thread instead of 71,
+// which leaves the loads more of the L1 cache: 130 -> 126 us).  The kernel
+// that reads single values takes kPlanes0 at any budget (!TIGHT): it has no
+// register left for the variable (128 x 253 x 515 at R = 16: 43 against 45).
+constexpr int kPlanes1 = 5, kPlanes0 = 38;  // planes 31 .. 16 and 15 .. 0
+template <bool TIGHT>
+__host__ __device__ constexpr int planes0_at(int words)
+{
+    return TIGHT && words + 6 < kPlanes0 ? words + 6 : kPlanes0;
+}
+constexpr bool planes_clear()
+{
+    for (int j = 0; j < 32; ++j)
+        if ((138 + 65 * j) / 32 + 1 >= (j < 16 ? kPlanes1 + 2 * (j + 1) : kPlanes0 + 2 * (j - 15)))
+            return false;
+    return (73 + 65 * 16) / 32 < kPlanes0;  // the second half's planes behind the first half's words
+}
+static_assert(planes_clear(), "coded words stay below the planes that are yet to be coded");
+template <bool TIGHT>
+__device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mode, int mparam, uint32_t *dst)
 {
     // the largest magnitude, three values per instruction (any NaN gives one
     // with the same exponent)
@@ -496,20 +524,20 @@ __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mo
     auto code_half = [&](auto base_c) {  // planes base + 15 .. base
         constexpr int base = decltype(base_c)::value;
         const int stop = max(pmin, base);
-        const uint32_t *pb = pm - base;
+        const uint32_t *pb = dst + (base != 0 ? kPlanes1 : planes0_at<TIGHT>(words)) + 2 * (15 + base);
         c = code_planes<base != 0>(dst, pb, p, stop, budget, c);
     };
+    auto keep_half = [&](uint32_t *pm, auto at_c) {  // the plane that is coded first comes first
+        constexpr int at = decltype(at_c)::value;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        pm[i] = v[16 + i];
-        pm[16 + i] = v[48 + i];
-    }
+        for (int i = 0; i < 16; ++i) {
+            pm[2 * (15 - i)] = v[at + i];
+            pm[2 * (15 - i) + 1] = v[32 + at + i];
+        }
+    };
+    keep_half(dst + kPlanes1, std::integral_constant<int, 16>{});
     code_half(std::integral_constant<int, 16>{});
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        pm[i] = v[i];
-        pm[16 + i] = v[32 + i];
-    }
+    keep_half(dst + planes0_at<TIGHT>(words), std::integral_constant<int, 0>{});
     code_half(std::integral_constant<int, 0>{});
     if (mode == OOC_FR4_RATE)
         clear_tail(dst, c.off, words);
@@ -736,7 +764,13 @@ __device__ __forceinline__ void stage_blocks(const uint32_t *__restrict__ src, i
 // ---- kernels ------------------------------------------------------------------
 // Words per block in the encoder's shared memory: odd, so that the threads'
 // blocks start in different banks.
-__host__ __device__ constexpr int encode_stride(int words) { return (words + kSlack) | 1; }
+__host__ __device__ constexpr int encode_stride64(int words) { return (words + kSlack) | 1; }
+template <bool TIGHT>
+__host__ __device__ constexpr int encode_stride(int words)  // with room for the planes in them
+{
+    const int p = planes0_at<TIGHT>(words) + 32;
+    return words + kSlack > p ? (words + kSlack) | 1 : p | 1;
+}
 
 // A warp's `nv` consecutive blocks of `words` words from its part of shared
 // memory to the stream at `dst`.
@@ -777,8 +811,8 @@ __device__ __forceinline__ void store_blocks(uint32_t *dst, int nv, int words, i
 __global__ void __launch_bounds__(kThreads, 6) fr4_encode_kernel(ConstRing in, int64_t nx, int64_t ny, int64_t z0,
                                                                  int64_t nblk, int rate, uint32_t *__restrict__ out)
 {
-    extern __shared__ uint32_t smem[];  // each thread's block, then each thread's planes
-    const int words = 2 * rate, stride = encode_stride(words);
+    extern __shared__ uint32_t smem[];  // each thread's block
+    const int words = 2 * rate, stride = encode_stride<true>(words);
     const int64_t b = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     const int64_t first = b - (threadIdx.x & 31);
     if (first >= nblk)
@@ -800,7 +834,7 @@ __global__ void __launch_bounds__(kThreads, 6) fr4_encode_kernel(ConstRing in, i
                 v[16 * k + 4 * j + 2] = __float_as_uint(f.z);
                 v[16 * k + 4 * j + 3] = __float_as_uint(f.w);
             }
-        encode_block(v, words, OOC_FR4_RATE, 0, mine, smem + kThreads * stride + threadIdx.x * kHalfStride);
+        encode_block<true>(v, words, OOC_FR4_RATE, 0, mine);
     }
     store_blocks(out + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
                  mine - (threadIdx.x & 31) * stride);
@@ -1016,10 +1050,10 @@ __device__ __forceinline__ void encode_block64(const uint64_t (&v)[64], int word
         constexpr int at = decltype(at_c)::value;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            pm[i] = a[at + i];
-            pm[16 + i] = a[32 + at + i];
+            pm[2 * (15 - i)] = a[at + i];
+            pm[2 * (15 - i) + 1] = a[32 + at + i];
         }
-        const uint32_t *pb = pm - base;
+        const uint32_t *pb = pm + 2 * (15 + base);
         c = code_planes<base == 48>(dst, pb, p, base, 32 * words, c);
     };
     to_planes32<0>(hi);
@@ -1117,7 +1151,7 @@ __global__ void __launch_bounds__(kThreads64, 6) fr4d_encode_kernel(DConstRing i
                                                                  int64_t nblk, int rate, uint32_t *__restrict__ out)
 {
     extern __shared__ uint32_t smem[];  // each thread's block, then each thread's planes
-    const int words = 2 * rate, stride = encode_stride(words);
+    const int words = 2 * rate, stride = encode_stride64(words);
     const int64_t b = (int64_t)blockIdx.x * kThreads64 + threadIdx.x;
     const int64_t first = b - (threadIdx.x & 31);
     if (first >= nblk)
@@ -1181,7 +1215,7 @@ size_t smem_bytes64(int rate, bool encoder)
 {
     if (!encoder)
         return (size_t)kThreads64 * (decode_stride(2 * rate) + kHalfStride) * sizeof(uint32_t);
-    return (size_t)kThreads64 * (encode_stride(2 * rate) + kHalfStride) * sizeof(uint32_t);
+    return (size_t)kThreads64 * (encode_stride64(2 * rate) + kHalfStride) * sizeof(uint32_t);
 }
 
 cudaError_t ensure_smem_attr64()
@@ -1271,7 +1305,7 @@ __global__ void __launch_bounds__(kThreads, 6)
                             uint32_t *__restrict__ out)
 {
     extern __shared__ uint32_t smem[];
-    const int stride = encode_stride(words);
+    const int stride = encode_stride<VEC>(words);
     const int64_t b = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     const int64_t first = b - (threadIdx.x & 31);
     if (first >= nblk)
@@ -1282,7 +1316,7 @@ __global__ void __launch_bounds__(kThreads, 6)
         const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
         uint32_t v[64];
         gather_clamped<VEC>(in, nx, ny, nz, bx, by, bz, v);
-        encode_block(v, words, OOC_FR4_RATE, 0, mine, smem + kThreads * stride + threadIdx.x * kHalfStride);
+        encode_block<VEC>(v, words, OOC_FR4_RATE, 0, mine);
     }
     store_blocks(out + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
                  mine - (threadIdx.x & 31) * stride);
@@ -1397,7 +1431,7 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned l
 // one status word per tile, all zero at launch.  `cap`: words of shared
 // memory for a block (var_block_words of the lowest plane).
 template <bool VEC>
-__global__ void __launch_bounds__(kThreads, 5)
+__global__ void __launch_bounds__(kThreads, 6)
     fr4_encode_var_kernel(const float *__restrict__ in, int64_t nx, int64_t ny, int64_t nz, int64_t nblk, int mode,
                           int mparam, int cap, uint32_t *__restrict__ out, uint64_t out_words,
                           uint64_t *__restrict__ index, unsigned long long *scratch)
@@ -1414,7 +1448,7 @@ __global__ void __launch_bounds__(kThreads, 5)
     }
     __syncthreads();
     const int64_t tile = s_tile;
-    const int stride = encode_stride(cap);
+    const int stride = encode_stride<true>(cap);
     const int64_t b = tile * kThreads + threadIdx.x;
     uint32_t *mine = smem + threadIdx.x * stride;
     uint64_t nw = 0;
@@ -1423,8 +1457,7 @@ __global__ void __launch_bounds__(kThreads, 5)
         const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
         uint32_t v[64];
         gather_clamped<VEC>(in, nx, ny, nz, bx, by, bz, v);
-        const int bits = encode_block(v, cap, mode, mparam, mine,
-                                      smem + kThreads * stride + threadIdx.x * kHalfStride);
+        const int bits = encode_block<true>(v, cap, mode, mparam, mine);
         nw = (uint64_t)((bits + 31) >> 5);
     }
     // exclusive scan of the word counts over the CTA
@@ -1501,15 +1534,15 @@ __global__ void __launch_bounds__(kThreads, 5)
             out[off + i] = mine[i];
 }
 
-size_t dense_smem_bytes(int words, bool encoder)
+size_t dense_smem_bytes(int words, bool encoder, bool vec)
 {
     if (!encoder)
         return (size_t)kThreads * (decode_stride(words) + kHalfStride) * sizeof(uint32_t);
-    return (size_t)kThreads * (encode_stride(words) + kHalfStride) * sizeof(uint32_t);
+    return (size_t)kThreads * (vec ? encode_stride<true>(words) : encode_stride<false>(words)) * sizeof(uint32_t);
 }
 
 // Shared memory of the variable-size kernels.
-size_t var_encode_smem(int cap) { return dense_smem_bytes(cap, true); }
+size_t var_encode_smem(int cap) { return dense_smem_bytes(cap, true, true); }
 constexpr size_t kVarDecodeSmem = (size_t)((kThreads / 32) * kVarBuf + kThreads * kHalfStride) * sizeof(uint32_t);
 
 cudaError_t ensure_dense_smem_attr()
@@ -1519,10 +1552,10 @@ cudaError_t ensure_dense_smem_attr()
         struct {
             const void *fn;
             size_t bytes;
-        } const a[] = {{(const void *)fr4_encode_dense_kernel<false>, dense_smem_bytes(128, true)},
-                       {(const void *)fr4_encode_dense_kernel<true>, dense_smem_bytes(128, true)},
-                       {(const void *)fr4_decode_dense_kernel<false>, dense_smem_bytes(128, false)},
-                       {(const void *)fr4_decode_dense_kernel<true>, dense_smem_bytes(128, false)},
+        } const a[] = {{(const void *)fr4_encode_dense_kernel<false>, dense_smem_bytes(128, true, false)},
+                       {(const void *)fr4_encode_dense_kernel<true>, dense_smem_bytes(128, true, false)},
+                       {(const void *)fr4_decode_dense_kernel<false>, dense_smem_bytes(128, false, false)},
+                       {(const void *)fr4_decode_dense_kernel<true>, dense_smem_bytes(128, false, false)},
                        {(const void *)fr4_encode_var_kernel<false>, var_encode_smem(var_block_words(0))},
                        {(const void *)fr4_encode_var_kernel<true>, var_encode_smem(var_block_words(0))},
                        {(const void *)fr4_decode_var_kernel<false>, kVarDecodeSmem},
@@ -1537,15 +1570,13 @@ cudaError_t ensure_dense_smem_attr()
     return once;
 }
 
-// Shared memory per CTA (encoder): each thread's compressed words plus
-// kSlack words of slack (stride 2R + kSlack + 1, odd, so that the threads'
-// slots start in different banks), then each thread's 64 plane masks
-// (stride 65).  The decoder keeps only the plane masks.
+// Shared memory per CTA: the encoder's blocks with the planes in them, or the
+// decoder's blocks and then each thread's planes.
 size_t smem_bytes(int rate, bool encoder)
 {
     if (!encoder)
         return (size_t)kThreads * (decode_stride(2 * rate) + kHalfStride) * sizeof(uint32_t);
-    return (size_t)kThreads * (encode_stride(2 * rate) + kHalfStride) * sizeof(uint32_t);
+    return (size_t)kThreads * encode_stride<true>(2 * rate) * sizeof(uint32_t);
 }
 
 cudaError_t ensure_smem_attr()
@@ -1645,7 +1676,7 @@ cudaError_t launch_fr4_encode_dense(const float *in, int64_t nx, int64_t ny, int
         return e;
     const int64_t grid = (nblk + kThreads - 1) / kThreads;
     const auto kernel = vec_rows(in, nx) ? fr4_encode_dense_kernel<true> : fr4_encode_dense_kernel<false>;
-    kernel<<<(unsigned)grid, kThreads, dense_smem_bytes(words, true), st>>>(in, nx, ny, nz, nblk, words, out);
+    kernel<<<(unsigned)grid, kThreads, dense_smem_bytes(words, true, vec_rows(in, nx)), st>>>(in, nx, ny, nz, nblk, words, out);
     return cudaGetLastError();
 }
 
@@ -1696,7 +1727,7 @@ cudaError_t launch_fr4_decode_dense(const uint32_t *in, int64_t in_words, const 
         if (words < 1 || words > 128)
             return cudaErrorInvalidValue;
         const auto kernel = vec_rows(out, nx) ? fr4_decode_dense_kernel<true> : fr4_decode_dense_kernel<false>;
-        kernel<<<(unsigned)grid, kThreads, dense_smem_bytes(words, false), st>>>(in, nx, ny, nz, nblk, words, out);
+        kernel<<<(unsigned)grid, kThreads, dense_smem_bytes(words, false, false), st>>>(in, nx, ny, nz, nblk, words, out);
     } else {
         const auto kernel = vec_rows(out, nx) ? fr4_decode_var_kernel<true> : fr4_decode_var_kernel<false>;
         kernel<<<(unsigned)grid, kThreads, kVarDecodeSmem, st>>>(in, in_words, index, nx, ny, nz, nblk, mode, mparam,
