@@ -396,10 +396,7 @@ cudaError_t take_stencil_fault(unsigned *fault)
         const unsigned zero = 0u;
         e = cudaMemcpyToSymbol(g_stencil_fault, &zero, sizeof(zero));
     }
-    unsigned vw = 0u;
-    if (e == cudaSuccess)
-        e = take_wave_fault(&vw);
-    *fault = v | vw;
+    *fault = v;
     return e;
 }
 

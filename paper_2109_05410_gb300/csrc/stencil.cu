@@ -517,7 +517,6 @@ OOC_PRAGMA(unroll OOC_HEATX2_UNROLL)
     }
 }
 
-#if !OOC_WAVE_TMA
 // wave25 staging: the p tile of every plane (8 own rows and 4 halo rows on
 // each side, plus the 4-point groups beyond the own rows' ends) in kWavePS
 // stages, and p_prev / kappa of the own rows in kWaveKS stages.  The copy
@@ -795,8 +794,6 @@ __global__ void __launch_bounds__(kTX *kWaveTY, kWaveTY <= 8 ? 2 : 1)
     cp_async_wait<0>();  // no copy may outlive the CTA's shared memory
 }
 
-#endif
-
 __global__ void add_time_kernel(int64_t *t, int64_t n) { *t += n; }
 
 __global__ void swap_kernel(float *a, float *b, int64_t n)
@@ -873,7 +870,6 @@ cudaError_t launch_heat7x2_regs(ConstRing in, Ring out, int64_t nx, int64_t ny, 
 }
 
 
-#if !OOC_WAVE_TMA
 namespace {
 // One launch of a wave25_kernel mode over planes [z0, z1) of rings that share
 // nslot and zbase.
@@ -946,8 +942,6 @@ cudaError_t launch_wave25(ConstRing p, Ring pprev_out, ConstRing kappa, int64_t 
     return launch_wave25_to(p, ConstRing{pprev_out.base, pprev_out.nslot, pprev_out.zbase}, pprev_out, kappa, nx, ny,
                             nz, z0, z1, sx, sy, sz, w, st, tab, pdl);
 }
-
-#endif
 
 cudaError_t launch_add_time(int64_t *t, int64_t n, cudaStream_t st)
 {

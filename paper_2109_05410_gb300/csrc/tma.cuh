@@ -1,6 +1,6 @@
 // tma.cuh -- TMA tensor copies into shared memory with mbarrier completion,
-// and bounded mbarrier waits, shared by the TMA-staged stencil kernels
-// (heat_tma.cu, wave_tma.cu).
+// and bounded mbarrier waits, for the TMA-staged stencil kernel
+// (heat_tma.cu).
 #pragma once
 #include <cuda.h>
 
@@ -24,11 +24,6 @@ __device__ __forceinline__ void mbar_arrive_tx(uint64_t *bar, unsigned bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // true once the phase with parity `parity` has completed; false after
@@ -71,7 +66,5 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
 // base 16-byte aligned.
 cudaError_t ring_tensor_map(const float *base, int64_t nx, int64_t ny, int64_t nslot, int box_x, int box_y,
                             CUtensorMap *out);
-// Reads and clears the device fault word of the TMA-staged wave kernel.
-cudaError_t take_wave_fault(unsigned *fault);
 
 }  // namespace ooc
