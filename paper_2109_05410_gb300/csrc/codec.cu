@@ -1408,8 +1408,11 @@ __global__ void __launch_bounds__(kThreads, 6)
 // running and never waits on a later one.  status[t] holds the tile's state
 // in bits 62-63 and a word count in bits 0-61: kTileAgg its own words,
 // kTilePrefix the words of tiles 0 .. t, kTileFailed a look-back that gave up.
-// Each published value carries everything its reader needs, so relaxed
-// 64-bit loads and stores suffice.
+// Each published value carries everything its reader needs, so relaxed 64-bit
+// accesses suffice.  The states are in rising order and are published by
+// atomicMax: a tile that gave up also marks the last tile failed, whose word
+// the host reads, and that mark stays whatever the last tile publishes later
+// (a later tile may have counted the failed one's words before it gave up).
 constexpr uint64_t kTileAgg = 1ull << 62, kTilePrefix = 2ull << 62, kTileFailed = 3ull << 62;
 constexpr uint64_t kTileValue = (1ull << 62) - 1;
 constexpr int kLookbackSpins = 1 << 24;  // about a second of 64 ns sleeps per tile waited on
@@ -1419,11 +1422,6 @@ __device__ __forceinline__ uint64_t ld_relaxed_u64(const unsigned long long *p)
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
-}
-
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned long long v)
-{
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 // Block b's words at out + index[b]; index[nblk] = total words.  A block is
@@ -1484,7 +1482,7 @@ __global__ void __launch_bounds__(kThreads, 6)
         uint64_t prefix = 0;
         bool failed = false;
         if (lane == 0)
-            st_relaxed_u64(&status[tile], (tile == 0 ? kTilePrefix : kTileAgg) | total);
+            atomicMax(&status[tile], (tile == 0 ? kTilePrefix : kTileAgg) | total);
         for (int64_t j = tile - 1 - lane; tile > 0; j -= 32) {
             uint64_t v = kTilePrefix;  // before tile 0: nothing
             if (j >= 0) {
@@ -1513,11 +1511,12 @@ __global__ void __launch_bounds__(kThreads, 6)
         }
         if (lane == 0) {
             if (failed) {
-                st_relaxed_u64(&status[tile], kTileFailed);  // later tiles stop at once
+                atomicMax(&status[tile], kTileFailed);  // later tiles stop at once
+                atomicMax(&status[gridDim.x - 1], kTileFailed);
                 atomicOr(&g_codec_fault, 1u);
                 s_fail = 1;
             } else if (tile > 0) {
-                st_relaxed_u64(&status[tile], kTilePrefix | (prefix + total));
+                atomicMax(&status[tile], kTilePrefix | (prefix + total));
             }
             s_prefix = prefix;
         }
