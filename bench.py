@@ -64,10 +64,10 @@ COMPARE = [("fp32", 0), ("bf16", 0), ("fr4", 8), ("fr4", 12), ("fr4", 24)]
 # lines, and a changed file gives null.
 NCU_UNITS = 56 * 1024 * 1024
 NCU_COUNTERS = {
-    "heat7_stencil": {"src": ["heat_tma.cu", "tma.cuh", "stencil_common.cuh", "f32x2.cuh"], "sha": "0d363f8834289584",
-                      "dram_bytes": 428.6e6, "warp_inst": 83.74e6},
-    "fr4_encode": {"src": "codec.cu", "sha": "3d031d5fc8adc782", "dram_bytes": 320.7e6, "warp_inst": 180.37e6},
-    "fr4_decode": {"src": "codec.cu", "sha": "3d031d5fc8adc782", "dram_bytes": 296.2e6, "warp_inst": 180.98e6},
+    "heat7_stencil": {"src": ["heat_tma.cu", "tma.cuh", "stencil_common.cuh", "f32x2.cuh"], "sha": "71ba1f15c6a3e79f",
+                      "dram_bytes": 428.5e6, "warp_inst": 76.58e6},
+    "fr4_encode": {"src": "codec.cu", "sha": "693514c532d3f048", "dram_bytes": 317.1e6, "warp_inst": 120.29e6},
+    "fr4_decode": {"src": "codec.cu", "sha": "693514c532d3f048", "dram_bytes": 293.1e6, "warp_inst": 143.52e6},
 }
 # issue peak: 152 SMs x 4 schedulers x one warp instruction per clock at the
 # maximum SM clock of 2070 MHz
