@@ -17,8 +17,8 @@
 // exponent; a thread shifts the values of its two points' stencils to the
 // largest exponent among them, with 6 (heat7) or 7 (wave25) bits below that
 // value's last place, and adds them without rounding.  The wave's weights are
-// the integers 5040 c_m.  One conversion and one (heat7) or two (wave25)
-// FMAs in FP64 finish the point.
+// the integers 5040 c_m.  One conversion and two FMAs in FP64 finish the
+// point.
 // Against the FP64 sequence the sum carries no rounding but the shifts'
 // (below 2^-58 of the stencil's largest value each), so the result is nearer
 // the exact one: over random smooth and rough fields the error against exact
@@ -230,11 +230,18 @@ __global__ void __launch_bounds__(kTX *kTY64, 7)
             const uint32_t biga = fx_big(ca) | fx_big(cb) | fx_big(za) | fx_big(wa) | fx_big(ua) | fx_big(da) | fx_big(la);
             const uint32_t bigb = fx_big(ca) | fx_big(cb) | fx_big(zb) | fx_big(wb) | fx_big(ub) | fx_big(db) | fx_big(rb);
             exact = zeros || (exact && biga > kFxBig && bigb > kFxBig);
-            const long long sa = (za + wa) + (ua + da) + (la + cb) - 6 * ca;
-            const long long sb = (zb + wb) + (ub + db) + (rb + ca) - 6 * cb;
+            const long long sa = (za + wa) + (ua + da) + (la + cb);
+            const long long sb = (zb + wb) + (ub + db) + (rb + ca);
             const int k = (int)E - 1081;
-            o.x = __fma_rn(r, zeros ? 0.0 : scale_exp(__ll2double_rn(sa), k), cur.x);
-            o.y = __fma_rn(r, zeros ? 0.0 : scale_exp(__ll2double_rn(sb), k), cur.y);
+            // The sum is rounded before 6 c comes off: kept whole, sum - 6 c is
+            // any multiple n of c's last bit, and with r = RN(1/6) < 1/6 an
+            // n = 3 (mod 6), just short of a tie, always rounds towards c, a
+            // bias that adds up (error of 8 steps 1.03e-16, of 32 3.5e-16; so 7.7e-17 and
+            // 8.1e-17, in FP64 instructions 1.0e-16 and 1.05e-16).
+            const double ta = zeros ? 0.0 : scale_exp(__ll2double_rn(sa), k);
+            const double tb = zeros ? 0.0 : scale_exp(__ll2double_rn(sb), k);
+            o.x = __fma_rn(r, __fma_rn(-6.0, cur.x, ta), cur.x);
+            o.y = __fma_rn(r, __fma_rn(-6.0, cur.y, tb), cur.y);
         }
         if (!exact && inside) {
             o = heat_pair_f64(in, s0, nslot, plane, off, g.nx, g.ny, nz, x2, y, za + i, r);
