@@ -44,13 +44,13 @@
 //
 // Measured, us per step at 384^3 (G point-steps/s), FP64 instructions against
 // integer sums: wave25 3200 (17.7) and 835 (68); heat7 775 (73) and 286
-// (198; 309 while all-zero stencils had FP64 instructions of their own, which
+// (198; 166 G since the sum is rounded before 6 c comes off; 309 while all-zero stencils had FP64 instructions of their own, which
 // issue on that pipe for every stencil once predicated).  A wave from rest, whose steep precursors take the FP64 instructions
 // in part: 1.07 ms per 256^3 step against 0.32 to 1.07, by phase; neighbours
 // 2^60 apart at random, which nearly all take them: 1.36 against 1.39 ms
 // (heat7 0.315 against 0.388).  Bound now: wave25 by the ALU pipe and
 // shared-memory wavefronts (each 55-63 % busy, about 600 instructions per 64
-// points), heat7 by the FP64 pipe (61 %) and the ALU pipe (55 %) with 28 warps
+// points), heat7 by the FP64 pipe (61 %, one FMA more since) and the ALU pipe (55 %) with 28 warps
 // per SM.
 #include <type_traits>
 
