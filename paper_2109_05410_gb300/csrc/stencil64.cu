@@ -12,25 +12,27 @@
 // (measured: 0.06 against 2 warp instructions per clock and SM), so a stencil
 // in FP64 instructions (7 per heat7 point, 27 per wave25 point) takes 112 and
 // 432 SM clocks per warp whatever the memory does.  The neighbour sums
-// therefore run in exact 64-bit integer arithmetic: each value is kept as its
-// signed 53-bit significand (left-justified in 64 bits) and its biased
-// exponent; a thread shifts the values of its two points' stencils to the
-// largest exponent among them, with 6 (heat7) or 7 (wave25) bits below that
-// value's last place, and adds them without rounding.  The wave's weights are
-// the integers 5040 c_m.  One conversion and two FMAs in FP64 finish the
+// therefore run in 64-bit integer arithmetic: each value is kept as its
+// 53-bit significand (left-justified in 64 bits) and its biased exponent; a
+// thread shifts the values of its two points' stencils to the largest exponent
+// among them, with 5 (heat7) or 6 (wave25) bits below that value's last place
+// and rounded to nearest, and adds them without rounding.  The wave's weights
+// are the integers 5040 c_m.  One conversion and two FMAs in FP64 finish the
 // point.
 // Against the FP64 sequence the sum carries no rounding but the shifts'
-// (below 2^-58 of the stencil's largest value each), so the result is nearer
+// (at most 2^-59 of the stencil's largest value each), so the result is nearer
 // the exact one: over random smooth and rough fields the error against exact
-// arithmetic is below the FP64 instructions' (see the GPU tests).
+// arithmetic is below the FP64 instructions' after one step, and heat7's over
+// many steps (see the GPU tests).
 //
 // Stencils that the integer form does not hold as exactly as FP64 would take
 // the FP64 instructions instead, per thread: infinities, NaN, a largest
 // exponent outside [kELo, kEHi] (results near overflow or below 1e-270), and
-// values so far apart that the sum's last bit exceeds 2^-54 of every value of
-// the point's own stencil (wave25: of their shares of the sum).  A
-// result depends only on the values of its thread's two stencils, so windows
-// of a slab and whole fields give the same bits.
+// values so far apart that the sum's last bit exceeds 2^-54 of every value that
+// the point sums (wave25: of their shares of the sum).  A result depends only
+// on the values of its thread's two stencils (and the exponents of the pairs
+// beside them, which hold one value more), so windows of a slab and whole
+// fields give the same bits.
 //
 // A warp owns a 64-point row segment, two points per thread (16-byte double2
 // accesses); each value is converted once by the thread that loads it (halo
@@ -80,10 +82,19 @@ __device__ __forceinline__ double heat_pt64(double c, double xl, double xr, doub
 
 __device__ __forceinline__ double2 ldg2(const double *p) { return __ldg(reinterpret_cast<const double2 *>(p)); }
 
-// A pair of doubles as signed significands at the pair's exponent (the
-// larger of the two biased exponents): x = m * 2^(e - 1085), |m| < 2^63.  A
-// zero takes the implicit one too: its exponent shifts it out.  e is 0 only
-// where both values are zero.
+// A pair of doubles as significands at the pair's exponent (the larger of the
+// two biased exponents): |x| = m * 2^(e - 1085), 0 <= m < 2^63, held as m and,
+// for a negative x, as ~m.  A zero takes the implicit one too: its exponent
+// shifts it out.  e is 0 only where both values are zero.
+//
+// The ones' complement makes the shifts odd functions of x.  An arithmetic
+// shift of ~m is the complement of that of m, and y + (y & 1) takes y and ~y to
+// opposite even numbers, |x| rounded to the nearest (a tie away from zero).  A
+// shift of -m would be cut off towards minus infinity, an error of one sign
+// that adds up over the steps: on a point release at r = 1/6, heat7's error
+// was 1.9 times the FP64 instructions' after 200 steps and 2.5 times after 800
+// (1.0 so), and f(-u) differed from -f(u) (CPU emulation of the kernel's
+// integers against 113 bits, 24 x 20 x 20).
 struct Fx2 {
     long long a, b;
     uint32_t e;
@@ -100,9 +111,12 @@ __device__ __forceinline__ long long fx_mant(uint32_t hi, uint32_t lo, uint32_t 
 {
     unsigned long long m = (((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo) << 10;
     asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(d));  // shifts past 63 give 0
-    const long long s = (long long)((int)hi >> 31);
-    return ((long long)m ^ s) - s;
+    return (long long)m ^ (long long)((int)hi >> 31);
 }
+
+__device__ __forceinline__ int fx_odd(long long y) { return (int)((uint32_t)y & 1u); }
+// the even number that y stands for
+__device__ __forceinline__ long long fx_even(long long y) { return y + fx_odd(y); }
 
 __device__ __forceinline__ Fx2 to_fx(double2 v)
 {
@@ -227,11 +241,16 @@ __global__ void __launch_bounds__(kTX *kTY64, 7)
             const long long ua = sar64(up.x, et - eu), ub = sar64(up.y, et - eu);
             const long long da = sar64(dn.x, et - ed), db = sar64(dn.y, et - ed);
             const long long la = sar64(xl, et - el), rb = sar64(xr, et - er);
-            const uint32_t biga = fx_big(ca) | fx_big(cb) | fx_big(za) | fx_big(wa) | fx_big(ua) | fx_big(da) | fx_big(la);
-            const uint32_t bigb = fx_big(ca) | fx_big(cb) | fx_big(zb) | fx_big(wb) | fx_big(ub) | fx_big(db) | fx_big(rb);
+            // the six that are summed: the FP64 sequence rounds at their size,
+            // not at c's, and a large c among tiny neighbours is what a point
+            // release at r = 1/6 consists of
+            const uint32_t biga = fx_big(cb) | fx_big(za) | fx_big(wa) | fx_big(ua) | fx_big(da) | fx_big(la);
+            const uint32_t bigb = fx_big(ca) | fx_big(zb) | fx_big(wb) | fx_big(ub) | fx_big(db) | fx_big(rb);
             exact = zeros || (exact && biga > kFxBig && bigb > kFxBig);
-            const long long sa = (za + wa) + (ua + da) + (la + cb);
-            const long long sb = (zb + wb) + (ub + db) + (rb + ca);
+            const int na = (fx_odd(za) + fx_odd(wa) + fx_odd(ua)) + (fx_odd(da) + fx_odd(la) + fx_odd(cb));
+            const int nb = (fx_odd(zb) + fx_odd(wb) + fx_odd(ub)) + (fx_odd(db) + fx_odd(rb) + fx_odd(ca));
+            const long long sa = (za + wa) + (ua + da) + (la + cb) + na;
+            const long long sb = (zb + wb) + (ub + db) + (rb + ca) + nb;
             const int k = (int)E - 1081;
             // The sum is rounded before 6 c comes off: kept whole, sum - 6 c is
             // any multiple n of c's last bit, and with r = RN(1/6) < 1/6 an
@@ -519,14 +538,15 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
             const longlong2 r1 = sm.tm[b][ty + kWR][e + 1], r2 = sm.tm[b][ty + kWR][e + 2];
             auto at = [&](long long v, uint32_t ev, int m) { return sar64(v, et + (uint32_t)kU(m) - ev); };
             const long long ca = at(cm.x, ce, 0), cb = at(cm.y, ce, 0);
-            const long long xa[kWR] = {at(l1.y, exn[1], 1) + cb, at(l1.x, exn[1], 2) + at(r1.x, exn[2], 2),
-                                       at(l2.y, exn[0], 3) + at(r1.y, exn[2], 3),
-                                       at(l2.x, exn[0], 4) + at(r2.x, exn[3], 4)};
-            const long long xb[kWR] = {ca + at(r1.x, exn[2], 1), at(l1.y, exn[1], 2) + at(r1.y, exn[2], 2),
-                                       at(l1.x, exn[1], 3) + at(r2.x, exn[3], 3),
-                                       at(l2.y, exn[0], 4) + at(r2.y, exn[3], 4)};
-            wave_add<false>(wa, kN0, ca);
-            wave_add<false>(wb, kN0, cb);
+            auto two = [&](long long v, long long q) { return v + q + (fx_odd(v) + fx_odd(q)); };
+            const long long xa[kWR] = {two(at(l1.y, exn[1], 1), cb), two(at(l1.x, exn[1], 2), at(r1.x, exn[2], 2)),
+                                       two(at(l2.y, exn[0], 3), at(r1.y, exn[2], 3)),
+                                       two(at(l2.x, exn[0], 4), at(r2.x, exn[3], 4))};
+            const long long xb[kWR] = {two(ca, at(r1.x, exn[2], 1)), two(at(l1.y, exn[1], 2), at(r1.y, exn[2], 2)),
+                                       two(at(l1.x, exn[1], 3), at(r2.x, exn[3], 3)),
+                                       two(at(l2.y, exn[0], 4), at(r2.y, exn[3], 4))};
+            wave_add<false>(wa, kN0, fx_even(ca));
+            wave_add<false>(wb, kN0, fx_even(cb));
             // is the sums' last bit small against the values of each point's
             // own stencil (one1: beside it, six: sums further out)?
             const uint32_t own = w_one(ca) | w_one(cb);
@@ -539,15 +559,18 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
                 const uint32_t em = ey[m - 1], ep = ey[kWR + m - 1], fm = ez[m - 1], fp = ez[kWR + m - 1];
                 const long long ya = at(um.x, em, m), va = at(up.x, ep, m), za = at(zm.x, fm, m), qa = at(zp.x, fp, m);
                 const long long yb = at(um.y, em, m), vb = at(up.y, ep, m), zb = at(zm.y, fm, m), qb = at(zp.y, fp, m);
-                const long long sa = xa[m - 1] + (ya + va) + (za + qa), sb = xb[m - 1] + (yb + vb) + (zb + qb);
+                // the sums before their last value is rounded are complements
+                // of each other for u and -u too, as the test below needs
+                const long long ga = xa[m - 1] + (ya + va) + (za + qa) + (fx_odd(ya) + fx_odd(va) + fx_odd(za));
+                const long long gb = xb[m - 1] + (yb + vb) + (zb + qb) + (fx_odd(yb) + fx_odd(vb) + fx_odd(zb));
                 if (m == 1) {
                     onea |= w_one(ya) | w_one(va) | w_one(za) | w_one(qa);
                     oneb |= w_one(yb) | w_one(vb) | w_one(zb) | w_one(qb);
                 }
-                sixa |= w_six(sa);
-                sixb |= w_six(sb);
-                wave_add<(m & 1) != 0>(wa, k, sa);
-                wave_add<(m & 1) != 0>(wb, k, sb);
+                sixa |= w_six(ga);
+                sixb |= w_six(gb);
+                wave_add<(m & 1) != 0>(wa, k, ga + fx_odd(qa));
+                wave_add<(m & 1) != 0>(wb, k, gb + fx_odd(qb));
             };
             taps(std::integral_constant<int, 4>{});
             taps(std::integral_constant<int, 3>{});
