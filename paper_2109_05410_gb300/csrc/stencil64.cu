@@ -17,19 +17,20 @@
 // thread shifts the values of its two points' stencils to the largest exponent
 // among them, with 5 (heat7) or 6 (wave25) bits below that value's last place
 // and rounded to nearest, and adds them without rounding.  The wave's weights
-// are the integers 5040 c_m.  One conversion and two FMAs in FP64 finish the
-// point.
-// Against the FP64 sequence the sum carries no rounding but the shifts'
-// (at most 2^-59 of the stencil's largest value each), so the result is nearer
-// the exact one: over random smooth and rough fields the error against exact
-// arithmetic is below the FP64 instructions' after one step, and heat7's over
-// many steps (see the GPU tests).
+// are its FP64 coefficients as 53-bit integers.  One conversion and two FMAs in
+// FP64 finish the point.
+// Against the FP64 sequence the sum carries no rounding but the shifts' (each
+// at most 2^-58 of the stencil's largest value, wave25 2^-59 in its unit) and
+// one at its end.  By CPU emulation against 113 bits the error is 0.6 to 0.8 of
+// the FP64 instructions' for wave25 from 8 to 12800 steps, 0.8 to 1.0 for heat7
+// (whose two FMAs set it) from 8 to 800, on smooth, rough, positive, steep and
+// isolated fields; f(-u) = -f(u) as in FP64 instructions (see the GPU tests).
 //
 // Stencils that the integer form does not hold as exactly as FP64 would take
 // the FP64 instructions instead, per thread: infinities, NaN, a largest
 // exponent outside [kELo, kEHi] (results near overflow or below 1e-270), and
-// values so far apart that the sum's last bit exceeds 2^-54 of every value that
-// the point sums (wave25: of their shares of the sum).  A result depends only
+// values so far apart that the sum's unit exceeds 2^-53 of every value that the
+// point sums (wave25: of their shares of the sum).  A result depends only
 // on the values of its thread's two stencils (and the exponents of the pairs
 // beside them, which hold one value more), so windows of a slab and whole
 // fields give the same bits.
@@ -40,20 +41,17 @@
 // memory (double buffered, one barrier per plane), each load issued one plane
 // ahead of its use.  heat7 keeps its z-neighbours in registers; wave25 keeps
 // its nine planes' own values in shared memory, which leaves 80 registers and
-// 24 warps per SM (in registers, before the unit and the exactness check were
-// added: 964 us per 384^3 step with 16 warps and spills, 886 with 8 warps,
-// against 815).
+// 24 warps per SM.
 //
 // Measured, us per step at 384^3 (G point-steps/s), FP64 instructions against
-// integer sums: wave25 3200 (17.7) and 835 (68); heat7 775 (73) and 286
-// (198; 166 G since the sum is rounded before 6 c comes off; 309 while all-zero stencils had FP64 instructions of their own, which
-// issue on that pipe for every stencil once predicated).  A wave from rest, whose steep precursors take the FP64 instructions
-// in part: 1.07 ms per 256^3 step against 0.32 to 1.07, by phase; neighbours
-// 2^60 apart at random, which nearly all take them: 1.36 against 1.39 ms
-// (heat7 0.315 against 0.388).  Bound now: wave25 by the ALU pipe and
-// shared-memory wavefronts (each 55-63 % busy, about 600 instructions per 64
-// points), heat7 by the FP64 pipe (61 %, one FMA more since) and the ALU pipe (55 %) with 28 warps
-// per SM.
+// integer sums: wave25 3200 (17.7) and 1066 (53); heat7 775 (73) and 344
+// (165).  wave25 took 839 with shifts cut off and 16-bit rational weights: a
+// tenth more instructions for the rounding, twice the multiplies for the
+// weights.  White noise: wave25 1067, heat7 478, where some lane of nearly every
+// warp takes the FP64 instructions.  A wave from rest, whose steep precursors
+// take them in part: 0.85 ms per 256^3 step over its first 100.  Bound now:
+// wave25 by the ALU pipe and shared-memory wavefronts, heat7 by the FP64 pipe
+// (61 %) and the ALU pipe with 28 warps per SM.
 #include <type_traits>
 
 #include "stencil_common.cuh"
@@ -130,7 +128,7 @@ __device__ __forceinline__ Fx2 to_fx(double2 v)
 }
 
 // Above kFxBig when |v| >= 2^54 (also of several of these ORed together: when
-// one of their values is).  Then v's last bit is at most 2^-54 of its value.
+// one of their values is).  Then a rounded shift is off by at most 2^-54 of v.
 constexpr uint32_t kFxBig = (1u << 23) - 1;
 __device__ __forceinline__ uint32_t fx_big(long long v) { return (uint32_t)(v >> 32) + (1u << 22); }
 
@@ -140,6 +138,9 @@ __device__ __forceinline__ double scale_exp(double v, int k)
     const int hi = __double2hiint(v), lo = __double2loint(v);
     return (hi | lo) == 0 ? v : __hiloint2double(hi + (k << 20), lo);
 }
+
+template <int V>
+using IC = std::integral_constant<int, V>;
 
 // Slots of consecutive planes: the slot of plane z + d from the slot of z.
 __device__ __forceinline__ int slot_at(int s, int d, int nslot)
@@ -328,18 +329,55 @@ __device__ __noinline__ double2 wave_lap_pair_f64(const double *in, int s, int n
     return make_double2(l[0], l[1]);
 }
 
-// The weights are 5040 times the coefficients, 5040 (3 c0, c1 .. c4), signs
-// -, +, -, +, -.  The values at distance m are held in units of 2^kU(m) last
-// bits (0, 2, 5 and 9, about the inverse of their coefficient), so that where
-// a field rises steeply (ahead of a wave front a value four cells away is
-// many orders larger) the large far values, which weigh little, don't push
-// the near ones out; the weights take the units up.  The high and low words
-// of the 64-bit sums are weighted apart, each exactly in 64 bits: h and l - n.
+// The weights are the FP64 coefficients 3 c0, c1 .. c4 themselves, as integers
+// (53 bits each), so that the sum carries the operator that FP64 instructions
+// carry.  (The rational coefficients, 5040 c_m in 16 bits, differ from it by
+// some 1e-16 in the same way at every step: the error of 200 steps on rough
+// fields was 2.8 times the FP64 instructions', of 800 steps 5.2 times; 0.75 and
+// 0.77 with these weights, by CPU emulation against 113 bits.)  The values at
+// distance m are held in units of 2^kU(m) last bits (0, 2, 5 and 9, about the
+// inverse of their coefficient), so that where a field rises steeply (ahead of
+// a wave front a value four cells away is many orders larger) the large far
+// values, which weigh little, don't push the near ones out; the weights take
+// the units up.
+//
+// A weight is kWE bits left-justified and split as hi 2^31 + lo, lo in
+// [-2^30, 2^30); a sum S is even and split as hi 2^32 + 2 lo, so that all four
+// partial products are of signed words.
 __host__ __device__ constexpr int kU(int m) { return m == 4 ? 9 : (m == 3 ? 5 : (m == 2 ? 2 : 0)); }
-constexpr uint32_t kN0 = 43050, kN1 = 8064, kN2 = 1008u << kU(2), kN3 = 128u << kU(3), kN4 = 9u << kU(4);
+constexpr int kWE = 57;  // weight of 1.0: 2^57
+__host__ __device__ constexpr long long wave_weight(int m)
+{
+    const double c = m == 0 ? 3.0 * kD0 : (m == 1 ? kD1 : (m == 2 ? kD2 : (m == 3 ? kD3 : kD4)));
+    return (long long)(c * (double)(1ll << kU(m)) * (double)(1ll << kWE));
+}
+__host__ __device__ constexpr int wave_wlo(int m)
+{
+    return (int)(((wave_weight(m) + (1ll << 30)) & 0x7FFFFFFFll) - (1ll << 30));
+}
+__host__ __device__ constexpr int wave_whi(int m) { return (int)((wave_weight(m) - wave_wlo(m)) / (1ll << 31)); }
+// Exact, and the accumulators below hold any sums: |S| <= 2^60 for the centre
+// and 6 2^60 at a distance.
+constexpr bool wave_weights_fit()
+{
+    double pos = 0.0, neg = 0.0, lpos = 0.0, lneg = 0.0, mid = 0.0;
+    for (int m = 0; m <= 4; ++m) {
+        const double c = m == 0 ? 3.0 * kD0 : (m == 1 ? kD1 : (m == 2 ? kD2 : (m == 3 ? kD3 : kD4)));
+        if ((double)wave_weight(m) != c * (double)(1ll << kU(m)) * (double)(1ll << kWE) ||
+            (long long)wave_whi(m) * (1ll << 31) + wave_wlo(m) != wave_weight(m))
+            return false;
+        const double h = wave_whi(m), l = wave_wlo(m), al = l < 0.0 ? -l : l;
+        (h < 0.0 ? neg : pos) += h < 0.0 ? -h : h;
+        (l < 0.0 ? lneg : lpos) += al;
+        mid += (m == 0 ? 1.0 : 6.0) * al;
+    }
+    const double two31 = 2147483648.0, top = 9.2e18;
+    return (pos > neg ? pos : neg) * two31 + mid * (two31 / 8.0) + 2.0 * two31 < top && lpos * two31 < top &&
+           lneg * two31 < top;
+}
+static_assert(wave_weights_fit(), "weights");
 struct WaveAcc {
-    long long h;
-    unsigned long long l, n;  // low words of the positive and the negative weights
+    long long h, x, l;  // products of the high words, mixed, of the low words
 };
 
 __device__ __forceinline__ long long mad_wide_s(int a, int b, long long c)
@@ -348,51 +386,38 @@ __device__ __forceinline__ long long mad_wide_s(int a, int b, long long c)
     return c;
 }
 
-__device__ __forceinline__ unsigned long long mad_wide_u(uint32_t a, uint32_t b, unsigned long long c)
+template <int M>
+__device__ __forceinline__ void wave_add(WaveAcc &w, long long s)
 {
-    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
-    return c;
+    constexpr int wh = wave_whi(M), wl = wave_wlo(M);
+    const int hi = (int)(s >> 32), lo = (int)((uint32_t)s >> 1);
+    w.h = mad_wide_s(hi, wh, w.h);
+    w.x = mad_wide_s(lo, wh, w.x);
+    w.x = mad_wide_s(hi, wl, w.x);
+    w.l = mad_wide_s(lo, wl, w.l);
 }
 
-template <bool POS>
-__device__ __forceinline__ void wave_add(WaveAcc &w, uint32_t k, long long s)
+// L in FP64: the sum h 2^62 + x 2^31 + l, cut below 2^59 with the last bit set
+// if anything was cut off (which makes the cut an odd function and lets the
+// conversion round correctly), is an integer of 2^(E - 1079), below 2^62.1:
+// 2^-57 of the stencil's largest value.
+__device__ __forceinline__ double wave_finish(const WaveAcc &w, int E)
 {
-    const int hi = (int)(s >> 32);
-    const uint32_t lo = (uint32_t)s;
-    w.h = mad_wide_s(hi, POS ? (int)k : -(int)k, w.h);
-    if (POS)
-        w.l = mad_wide_u(lo, k, w.l);
-    else
-        w.n = mad_wide_u(lo, k, w.n);
+    const long long g = w.x + (w.l >> 31);
+    const long long v = (w.h << 3) + (g >> 28);
+    const uint32_t rest = ((uint32_t)g & 0x0FFFFFFFu) | ((uint32_t)w.l & 0x7FFFFFFFu);
+    return scale_exp(__ll2double_rn(rest != 0u ? v | 1 : v), E - 1079);
 }
 
-// The doubles of the coefficients do not add up to 0 as the coefficients do:
-// 3 kD0 + 6 (kD1 + .. + kD4) = -7.18e-16.  On smooth fields that sum times p
-// is the largest part of what the rounded coefficients change, and it is the
-// same at every step, so it is added here for agreement with the operator of
-// the rounded coefficients.
-constexpr int kSumErr = -4170600;                               // 5040 * 2^60 * (that sum)
-constexpr unsigned long long kInv5040 = 0xD00D00D00D00D00Dull;  // 2^76 / 5040
-constexpr unsigned long long kHalf = 52932;                     // centres the three truncations below
-
-// L in FP64: V = (h 2^32 + l - n) / 2^15 + c kSumErr / 2^75 < 2^62.4, then
-// V 2^12 / 5040 by its 64-bit reciprocal, as an integer of 2^(E - 1079)
-// (2^-57 of the stencil's largest value).
-__device__ __forceinline__ double wave_finish(const WaveAcc &w, long long c, int E)
-{
-    const long long corr = mad_wide_s((int)(c >> 32), kSumErr, 0) >> 43;
-    const long long v = (w.h << 17) + ((long long)(w.l - w.n) >> 15) + corr;
-    return scale_exp(__ll2double_rn(__mul64hi(v, (long long)kInv5040) + v), E - 1079);
-}
-
-// Above kW1 when one of the ORed values is at least 2^54 in magnitude; above
-// kW6 when one of the ORed sums of six reaches 2^57, so that a value in it
-// does.  A value of 2^54 in its unit weighs 0.8 x 2^54 last bits or more.  At
-// 2^54 the rms error stays below the FP64 instructions' on all tested fields
-// (heat7 at 2^53 does not).
+// Above kW1 when one of the ORed values (held as to_fx holds them) is at least
+// 2^54 in magnitude; above kW6 when one of the ORed sums of six (even numbers;
+// v + its sign tells s and -s alike) reaches 2^57, so that a value in it
+// reaches 2^54.  A value of 2^54 in its unit weighs 0.8 x 2^53 units of the
+// sum or more.  At 2^54 the rms error stays below the FP64 instructions' on all
+// tested fields (heat7 at 2^53 does not).
 constexpr uint32_t kW1 = (1u << 23) - 1, kW6 = (1u << 26) - 1;
 __device__ __forceinline__ uint32_t w_one(long long v) { return (uint32_t)(v >> 32) + (1u << 22); }
-__device__ __forceinline__ uint32_t w_six(long long v) { return (uint32_t)(v >> 32) + (1u << 25); }
+__device__ __forceinline__ uint32_t w_six(long long v) { return (uint32_t)((v + (v >> 63)) >> 32) + (1u << 25); }
 
 // Shared memory of a wave25 CTA: the row tile of the centre plane (double
 // buffered: 4 + TY + 4 rows of 2 + 32 + 2 pairs, the 4 x-neighbours beyond
@@ -480,17 +505,13 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
             sm.tm[b][xr][xc] = make_longlong2(h.a, h.b);
             sm.te[b][xr][xc] = h.e;
         }
-        // the next plane's halos and the queue's next plane, and this
-        // plane's other operands, which are used last
+        // the next plane's halos and the queue's next plane
         const bool more = i + 1 < cnt;
         const int64_t b0 = o0 + off;
         hv = (hrow && more) ? ldg2(pin + hoff + o1) : z2;
         xv = (xhalo && more) ? ldg2(pin + xoff + o1) : z2;
         const double2 qn = (inside && more && i + kWR + 1 < left) ? ldg2(pin + off + o5) : z2;
-        const double2 c = inside ? ldg2(pin + b0) : z2;
-        const double2 kv = inside ? ldg2(kap + b0) : z2;
         // p_prev is overwritten by this kernel: plain loads, not the read-only path
-        const double2 ppv = inside ? *reinterpret_cast<const double2 *>(pout + b0) : z2;
         __syncthreads();
         const int e = lane + 2;  // this thread's pair in the row
         uint32_t ey[2 * kWR], exn[4];
@@ -526,11 +547,10 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
         bool exact = Z == 0;  // all zeros
         {
             // run by every thread: without a branch the values' loads start
-            // ahead of the exponents' test (384^3 881 -> 835 us; all zeros
-            // 0.37 -> 0.44 ms per 256^3 step)
+            // ahead of the exponents' test
             const bool range = E >= (int)kELo && Z <= (int)kEHi;
             const uint32_t et = (uint32_t)E + 3u;
-            WaveAcc wa{0, kHalf, 0}, wb{0, kHalf, 0};
+            WaveAcc wa{0, 0, 0}, wb{0, 0, 0};
             // A row value at distance m of the first point is at m - 1 or
             // m + 1 of the second.  xa[j], xb[j]: at distance j + 1 left and
             // right of the first and of the second point, in that unit.
@@ -545,44 +565,50 @@ __global__ void __launch_bounds__(kTX *kWTY64, 3)
             const long long xb[kWR] = {two(ca, at(r1.x, exn[2], 1)), two(at(l1.y, exn[1], 2), at(r1.y, exn[2], 2)),
                                        two(at(l1.x, exn[1], 3), at(r2.x, exn[3], 3)),
                                        two(at(l2.y, exn[0], 4), at(r2.y, exn[3], 4))};
-            wave_add<false>(wa, kN0, fx_even(ca));
-            wave_add<false>(wb, kN0, fx_even(cb));
-            // is the sums' last bit small against the values of each point's
-            // own stencil (one1: beside it, six: sums further out)?
+            wave_add<0>(wa, fx_even(ca));
+            wave_add<0>(wb, fx_even(cb));
+            // is the sums' unit small against the values of each point's own
+            // stencil (one: beside it, six: sums further out)?
             const uint32_t own = w_one(ca) | w_one(cb);
             uint32_t onea = own, oneb = own, sixa = 1u << 25, sixb = 1u << 25;
             auto taps = [&](auto m_c) {
                 constexpr int m = decltype(m_c)::value;
-                constexpr uint32_t k = m == 1 ? kN1 : (m == 2 ? kN2 : (m == 3 ? kN3 : kN4));
                 const longlong2 um = sm.tm[b][ty + kWR - m][e], up = sm.tm[b][ty + kWR + m][e];
                 const longlong2 zm = *zq[m - 1], zp = *zq[kWR + m - 1];
                 const uint32_t em = ey[m - 1], ep = ey[kWR + m - 1], fm = ez[m - 1], fp = ez[kWR + m - 1];
                 const long long ya = at(um.x, em, m), va = at(up.x, ep, m), za = at(zm.x, fm, m), qa = at(zp.x, fp, m);
                 const long long yb = at(um.y, em, m), vb = at(up.y, ep, m), zb = at(zm.y, fm, m), qb = at(zp.y, fp, m);
-                // the sums before their last value is rounded are complements
-                // of each other for u and -u too, as the test below needs
-                const long long ga = xa[m - 1] + (ya + va) + (za + qa) + (fx_odd(ya) + fx_odd(va) + fx_odd(za));
-                const long long gb = xb[m - 1] + (yb + vb) + (zb + qb) + (fx_odd(yb) + fx_odd(vb) + fx_odd(zb));
+                const int na = (fx_odd(ya) + fx_odd(va)) + (fx_odd(za) + fx_odd(qa));
+                const int nb = (fx_odd(yb) + fx_odd(vb)) + (fx_odd(zb) + fx_odd(qb));
+                const long long sa = xa[m - 1] + (ya + va) + (za + qa) + na, sb = xb[m - 1] + (yb + vb) + (zb + qb) + nb;
                 if (m == 1) {
                     onea |= w_one(ya) | w_one(va) | w_one(za) | w_one(qa);
                     oneb |= w_one(yb) | w_one(vb) | w_one(zb) | w_one(qb);
                 }
-                sixa |= w_six(ga);
-                sixb |= w_six(gb);
-                wave_add<(m & 1) != 0>(wa, k, ga + fx_odd(qa));
-                wave_add<(m & 1) != 0>(wb, k, gb + fx_odd(qb));
+                sixa |= w_six(sa);
+                sixb |= w_six(sb);
+                wave_add<m>(wa, sa);
+                wave_add<m>(wb, sb);
             };
-            taps(std::integral_constant<int, 4>{});
-            taps(std::integral_constant<int, 3>{});
-            taps(std::integral_constant<int, 2>{});
-            taps(std::integral_constant<int, 1>{});
-            lap.x = exact ? 0.0 : wave_finish(wa, ca, E);
-            lap.y = exact ? 0.0 : wave_finish(wb, cb, E);
+            taps(IC<4>{});
+            taps(IC<3>{});
+            taps(IC<2>{});
+            taps(IC<1>{});
+            lap.x = exact ? 0.0 : wave_finish(wa, E);
+            lap.y = exact ? 0.0 : wave_finish(wb, E);
             exact = exact || (range && (onea > kW1 || sixa > kW6) && (oneb > kW1 || sixb > kW6));
         }
         if (!exact && inside) {
             lap = wave_lap_pair_f64(pin, s0, nslot, plane, off, g.nx, g.ny, nz, x2, y, za + i);
         }
+        // This plane's other operands, read where they are used (the barrier
+        // keeps them here): 12 registers that, held across the sums, spill
+        // (384^3 1262 us per step loaded before the sums, 1066 here; with L2
+        // prefetches in their old place 1145).
+        asm volatile("" ::: "memory");
+        const double2 c = inside ? ldg2(pin + b0) : z2;
+        const double2 kv = inside ? ldg2(kap + b0) : z2;
+        const double2 ppv = inside ? *reinterpret_cast<const double2 *>(pout + b0) : z2;
         double2 o;
         o.x = __fma_rn(kv.x, lap.x, __fma_rn(2.0, c.x, -ppv.x));
         o.y = __fma_rn(kv.y, lap.y, __fma_rn(2.0, c.y, -ppv.y));

@@ -10,7 +10,9 @@ Bounds.  A CPU emulation of the kernels' integers over 12 random fields each
 heat7 at r = 1/6, point release and half-empty checkerboard, 200 steps, 1.00
 (2.04 and 1.85 with shifts that cut off towards minus infinity); smooth, 32
 steps, 0.81, at most 0.87 (about 3 if 6 c comes off before the sum is
-rounded).  The bounds lie between."""
+rounded); wave25, 100 steps, rough 0.76, smooth 0.66, point release 0.76, at
+most 0.93 (2.09, 0.87 and 2.00 with rational weights).  The bounds lie
+between."""
 import numpy as np
 import pytest
 
@@ -18,6 +20,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 SHAPE = (12, 16, 72)
+C = [-205.0 / 72.0, 8.0 / 5.0, -1.0 / 5.0, 8.0 / 315.0, -1.0 / 560.0]
 KINDS = ["normal", "wide", "steep", "steps", "sparse", "tiny", "huge"]
 
 
@@ -114,3 +117,51 @@ def test_heat7_keeps_a_node_plane(ooc, kind):
     got = heat_gpu(ooc, u, 6)
     assert not np.any(got[5])
     assert np.array_equal(got[4], -got[6]) and np.any(got[4])
+
+
+def wave_gpu(ooc, p, pm, kap, n):
+    dp, dpm = torch.from_numpy(p.copy()).cuda(), torch.from_numpy(pm.copy()).cuda()
+    ooc.ooc_wave25_steps_f64(dp, dpm, torch.from_numpy(kap).cuda(), n)
+    return dp.cpu().numpy()
+
+
+def layers(shape):
+    z = np.indices(shape)[0]
+    return 0.07 * (1.0 + 0.02 * z / shape[0])
+
+
+@pytest.mark.parametrize("kind", ["normal", "smooth", "point"])
+def test_wave25_error_does_not_add_up(ooc, kind):
+    steps, err, kap = 100, np.zeros(2), layers(SHAPE)
+    for seed in range(2):
+        p = field(kind, SHAPE, 40 + seed)
+        got = wave_gpu(ooc, p, 0.95 * p, kap, steps)
+        q, qm, s, sm = p.astype(np.longdouble), (0.95 * p).astype(np.longdouble), p, 0.95 * p
+        for _ in range(steps):
+            lap = np.longdouble(3.0 * C[0]) * q
+            seq = (3.0 * C[0]) * s
+            for m in range(1, 5):
+                lap = lap + np.longdouble(C[m]) * six(q, m)
+                seq = fma(C[m], six(s, m), seq)
+            q, qm = kap * lap + 2 * q - qm, q
+            s, sm = fma(kap, seq, fma(2.0, s, -sm)), s
+        norm = np.sqrt(np.mean(q * q))
+        err += [float(np.mean(((v - q) / norm) ** 2)) for v in (got, s)]
+    assert err[0] <= err[1], np.sqrt(err / 2)
+
+
+@pytest.mark.parametrize("kind", KINDS + ["point", "checker", "smooth"])
+def test_wave25_is_odd(ooc, kind):
+    p, pm, kap = field(kind, SHAPE, 50), 0.9 * field(kind, SHAPE, 50), layers(SHAPE)
+    assert np.array_equal(wave_gpu(ooc, -p, -pm, kap, 4), -wave_gpu(ooc, p, pm, kap, 4))
+
+
+@pytest.mark.parametrize("kind", ["normal", "steps", "wide", "sparse"])
+def test_wave25_keeps_a_node_plane(ooc, kind):
+    shape = (36, 16, 72)
+    u = np.zeros(shape)
+    u[18:20] = field(kind, shape, 51)[18:20]
+    u[15:17] = -u[19:17:-1]
+    got = wave_gpu(ooc, u, 0.9 * u, np.full(shape, 0.1), 6)
+    assert not np.any(got[17])
+    assert np.array_equal(got[16], -got[18]) and np.any(got[16])
