@@ -410,24 +410,33 @@ __device__ __forceinline__ uint32_t shr32(uint32_t v, int n)
 // plane of every lane's block fits 32 (and the coefficients 32..63 have no one
 // yet), it is written as one field.  On smooth fields these are 10 to 12 of
 // 28 planes: R = 16 148 -> 141 us, 139 -> 138 on rough ones; in the later
-// parts too it gains nothing there and costs 2 %.  The vote only chooses
-// between two ways to the same bits, so it may be taken by any set of lanes.
+// parts too it gains nothing there and costs 2 %.  All 32 lanes of the warp
+// come here and take the same turns of the first loop, so the vote is one of
+// the whole warp; a lane without planes (p < stop) or budget left votes for
+// going on.  (56 planes of 1024^2, us, against votes of whatever lanes were
+// together: R = 16 148 and 151, R = 24 153 and 157, rough 138 and 139; FP64, 24
+// of 64 bits, encoded and decoded 848 and 809.)
 template <bool FIRST>
 __device__ __forceinline__ CodePos code_planes(uint32_t *dst, const uint32_t *pb, int &p, int stop, int budget, CodePos c)
 {
 #pragma unroll 1
-    for (; FIRST && p >= stop && c.off < budget; --p) {
-        const uint32_t x = pb[-2 * p];
+    for (int turns = FIRST ? __reduce_max_sync(0xffffffffu, p - stop + 1) : 0; turns > 0; --turns) {
+        const bool more = p >= stop && c.off < budget;
+        const uint32_t *pm = pb - 2 * max(p, stop);
+        const uint32_t x = pm[0];
         const uint32_t s = shr32(x, c.n);  // new ones; 0: tl = -1, bits = -1
         const int tl = 31 - __clz((int)s), bits = tl + __popc((int)s);
-        const bool fits = pb[1 - 2 * p] == 0u && c.n + bits + 2 <= 32;
-        if (__any_sync(__activemask(), !fits))
+        const bool fits = pm[1] == 0u && c.n + bits + 2 <= 32;
+        if (__any_sync(0xffffffffu, more && !fits))
             break;
-        const uint32_t v = insert_ones(s, s ^ (1u << (tl & 31)));
-        const uint32_t field = (v << 1) | (s != 0u ? 1u : 0u);
-        put32(dst, c.off, (x & ~shl32(~0u, c.n)) | shl32(field, c.n));
-        c.off += c.n + bits + 2;
-        c.n += tl + 1;
+        if (more) {
+            const uint32_t v = insert_ones(s, s ^ (1u << (tl & 31)));
+            const uint32_t field = (v << 1) | (s != 0u ? 1u : 0u);
+            put32(dst, c.off, (x & ~shl32(~0u, c.n)) | shl32(field, c.n));
+            c.off += c.n + bits + 2;
+            c.n += tl + 1;
+            --p;
+        }
     }
 #pragma unroll 1
     for (; p >= stop && c.off < budget; --p)
@@ -443,14 +452,14 @@ __device__ __forceinline__ void clear_tail(uint32_t *dst, int off, int words)
 }
 
 // Encode one block into dst[0 .. words) (a bit budget of 32 words; words =
-// 2R at a fixed rate) with the plane range of `mode`.  Returns the coded
-// length in bits (exact for the variable-size modes, whose budget never
-// binds).  The planes go through shared memory 16 at a time, in the part of
-// dst that the coded words have not reached yet: half the shared memory of
-// all 32 planes, and none beside the words, for 24 warps per SM at any rate
-// up to 32 and in the variable-size modes (with 33 words of their own per
-// thread it was 16 warps at R = 24, 157 us against 144, and 16 in the
-// variable-size encoder, 512^3 at tolerance 1e-4 530 against 475).
+// 2R at a fixed rate) with the plane range of `mode`.  Called by whole
+// warps.  Returns the coded length in bits (exact for the variable-size modes,
+// whose budget never binds).  The planes go through shared memory 16 at a time,
+// in the part of dst that the coded words have not reached yet: half the shared
+// memory of all 32 planes, and none beside the words, for 24 warps per SM at
+// any rate up to 32 and in the variable-size modes (with 33 words of their own per thread it was 16 warps
+// at R = 24, 157 us against 144, and 16 in the variable-size encoder, 512^3 at
+// tolerance 1e-4 530 against 475).
 //
 // Before plane 31 - j at most 73 + 65 j bits are coded (var_block_words), and
 // coding it touches words up to (138 + 65 j) / 32 + 1.  Its own two words are
@@ -486,12 +495,14 @@ __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mo
         asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(top) : "f"(__uint_as_float(v[i])), "f"(__uint_as_float(v[i + 1])));
     const uint32_t mx = __float_as_uint(top);
     const int budget = 32 * words;
-    if (mx == 0u) {
+    auto zeros = [&] {
         dst[0] = 0u;
         if (mode == OOC_FR4_RATE)
             clear_tail(dst, 0, words);
         return 1;
-    }
+    };
+    if (!__any_sync(0xffffffffu, mx != 0u))
+        return zeros();
     const int emax = (int)(mx >> 23) - 126;  // largest frexp exponent, >= -126
     const int pmin = plane_floor(mode, mparam, emax);
 
@@ -520,7 +531,7 @@ __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mo
     dst[0] = 1u | ((uint32_t)((emax + 127) & 0xFF) << 1);
     dst[1] = 0u;
     CodePos c{0, 9 + skip};
-    int p = 31 - skip;
+    int p = mx != 0u ? 31 - skip : -1;  // a block of zeros has no planes
     auto code_half = [&](auto base_c) {  // planes base + 15 .. base
         constexpr int base = decltype(base_c)::value;
         const int stop = max(pmin, base);
@@ -539,6 +550,8 @@ __device__ __forceinline__ int encode_block(uint32_t (&v)[64], int words, int mo
     code_half(std::integral_constant<int, 16>{});
     keep_half(dst + planes0_at<TIGHT>(words), std::integral_constant<int, 0>{});
     code_half(std::integral_constant<int, 0>{});
+    if (mx == 0u)
+        return zeros();
     if (mode == OOC_FR4_RATE)
         clear_tail(dst, c.off, words);
     return c.off;
@@ -817,25 +830,24 @@ __global__ void __launch_bounds__(kThreads, 6) fr4_encode_kernel(ConstRing in, i
     const int64_t first = b - (threadIdx.x & 31);
     if (first >= nblk)
         return;
+    const int64_t own = min(b, nblk - 1);  // lanes past the end code the last block too
     uint32_t *mine = smem + threadIdx.x * stride;
-    if (b < nblk) {
-        const int64_t nbx = nx >> 2, nby = ny >> 2;
-        const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
-        const int64_t slot = ring_slot(z0 + 4 * bz, in.zbase, in.nslot);
-        const float *p = in.base + (slot * ny + 4 * by) * nx + 4 * bx;
-        uint32_t v[64];
+    uint32_t v[64];
+    const int64_t nbx = nx >> 2, nby = ny >> 2;
+    const int64_t bx = own % nbx, t2 = own / nbx, by = t2 % nby, bz = t2 / nby;
+    const int64_t slot = ring_slot(z0 + 4 * bz, in.zbase, in.nslot);
+    const float *p = in.base + (slot * ny + 4 * by) * nx + 4 * bx;
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < 4; ++k)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float4 f = __ldg(reinterpret_cast<const float4 *>(p + ((int64_t)k * ny + j) * nx));
-                v[16 * k + 4 * j + 0] = __float_as_uint(f.x);
-                v[16 * k + 4 * j + 1] = __float_as_uint(f.y);
-                v[16 * k + 4 * j + 2] = __float_as_uint(f.z);
-                v[16 * k + 4 * j + 3] = __float_as_uint(f.w);
-            }
-        encode_block<true>(v, words, OOC_FR4_RATE, 0, mine);
-    }
+        for (int j = 0; j < 4; ++j) {
+            const float4 f = __ldg(reinterpret_cast<const float4 *>(p + ((int64_t)k * ny + j) * nx));
+            v[16 * k + 4 * j + 0] = __float_as_uint(f.x);
+            v[16 * k + 4 * j + 1] = __float_as_uint(f.y);
+            v[16 * k + 4 * j + 2] = __float_as_uint(f.z);
+            v[16 * k + 4 * j + 3] = __float_as_uint(f.w);
+        }
+    encode_block<true>(v, words, OOC_FR4_RATE, 0, mine);
     store_blocks(out + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
                  mine - (threadIdx.x & 31) * stride);
 }
@@ -1002,14 +1014,14 @@ __device__ __forceinline__ double pow2d(int k)  // k in [-1022, 1023]
 }
 
 // Encode one FP64 block (bit patterns v) into dst[0 .. words) at a fixed
-// rate: words = 2R, a budget of 64R bits.
+// rate: words = 2R, a budget of 64R bits.  Called by whole warps.
 __device__ __forceinline__ void encode_block64(const uint64_t (&v)[64], int words, uint32_t *dst, uint32_t *pm)
 {
     uint64_t mx = 0;
 #pragma unroll
     for (int i = 0; i < 64; ++i)
         mx = umax64(mx, v[i] & 0x7FFFFFFFFFFFFFFFull);
-    if (mx == 0ull) {
+    if (!__any_sync(0xffffffffu, mx != 0ull)) {
         dst[0] = 0u;
         clear_tail(dst, 0, words);
         return;
@@ -1043,7 +1055,7 @@ __device__ __forceinline__ void encode_block64(const uint64_t (&v)[64], int word
     dst[0] = 1u | ((uint32_t)(emax + 1023) << 1);
     dst[1] = 0u;
     CodePos c{0, 12 + skip};
-    int p = 63 - skip;
+    int p = mx != 0ull ? 63 - skip : -1;  // a block of zeros has no planes
     // planes base + 15 .. base, whose masks are in a[at ..] and a[at + 32 ..]
     auto code_part = [&](auto base_c, const uint32_t (&a)[64], auto at_c) {
         constexpr int base = decltype(base_c)::value;
@@ -1065,6 +1077,10 @@ __device__ __forceinline__ void encode_block64(const uint64_t (&v)[64], int word
         to_planes32<32>(lo);
         code_part(std::integral_constant<int, 16>{}, lo, std::integral_constant<int, 16>{});
         code_part(std::integral_constant<int, 0>{}, lo, std::integral_constant<int, 0>{});
+    }
+    if (mx == 0ull) {
+        dst[0] = 0u;
+        c.off = 0;
     }
     clear_tail(dst, c.off, words);
 }
@@ -1157,12 +1173,12 @@ __global__ void __launch_bounds__(kThreads64, 6) fr4d_encode_kernel(DConstRing i
     if (first >= nblk)
         return;
     uint32_t *mine = smem + threadIdx.x * stride;
+    uint64_t v[64] = {};
     if (b < nblk) {
         const int64_t nbx = nx >> 2, nby = ny >> 2;
         const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
         const int64_t slot = ring_slot(z0 + 4 * bz, in.zbase, in.nslot);
         const double *p = in.base + (slot * ny + 4 * by) * nx + 4 * bx;
-        uint64_t v[64];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -1174,8 +1190,8 @@ __global__ void __launch_bounds__(kThreads64, 6) fr4d_encode_kernel(DConstRing i
                 v[16 * k + 4 * j + 2] = (uint64_t)__double_as_longlong(c.x);
                 v[16 * k + 4 * j + 3] = (uint64_t)__double_as_longlong(c.y);
             }
-        encode_block64(v, words, mine, smem + kThreads64 * stride + threadIdx.x * kHalfStride);
     }
+    encode_block64(v, words, mine, smem + kThreads64 * stride + threadIdx.x * kHalfStride);
     store_blocks(out + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
                  mine - (threadIdx.x & 31) * stride);
 }
@@ -1310,14 +1326,13 @@ __global__ void __launch_bounds__(kThreads, 6)
     const int64_t first = b - (threadIdx.x & 31);
     if (first >= nblk)
         return;
+    const int64_t own = min(b, nblk - 1);  // lanes past the end code the last block too
     uint32_t *mine = smem + threadIdx.x * stride;
-    if (b < nblk) {
-        const int64_t nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
-        const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
-        uint32_t v[64];
-        gather_clamped<VEC>(in, nx, ny, nz, bx, by, bz, v);
-        encode_block<VEC>(v, words, OOC_FR4_RATE, 0, mine);
-    }
+    uint32_t v[64];
+    const int64_t nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
+    const int64_t bx = own % nbx, t2 = own / nbx, by = t2 % nby, bz = t2 / nby;
+    gather_clamped<VEC>(in, nx, ny, nz, bx, by, bz, v);
+    encode_block<VEC>(v, words, OOC_FR4_RATE, 0, mine);
     store_blocks(out + first * words, (int)min(nblk - first, (int64_t)32), words, stride,
                  mine - (threadIdx.x & 31) * stride);
 }
@@ -1448,16 +1463,14 @@ __global__ void __launch_bounds__(kThreads, 6)
     const int64_t tile = s_tile;
     const int stride = encode_stride<true>(cap);
     const int64_t b = tile * kThreads + threadIdx.x;
+    const int64_t own = min(b, nblk - 1);  // lanes past the end code the last block too
     uint32_t *mine = smem + threadIdx.x * stride;
-    uint64_t nw = 0;
-    if (b < nblk) {
-        const int64_t nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
-        const int64_t bx = b % nbx, t2 = b / nbx, by = t2 % nby, bz = t2 / nby;
-        uint32_t v[64];
-        gather_clamped<VEC>(in, nx, ny, nz, bx, by, bz, v);
-        const int bits = encode_block<true>(v, cap, mode, mparam, mine);
-        nw = (uint64_t)((bits + 31) >> 5);
-    }
+    uint32_t v[64];
+    const int64_t nbx = (nx + 3) >> 2, nby = (ny + 3) >> 2;
+    const int64_t bx = own % nbx, t2 = own / nbx, by = t2 % nby, bz = t2 / nby;
+    gather_clamped<VEC>(in, nx, ny, nz, bx, by, bz, v);
+    const int bits = encode_block<true>(v, cap, mode, mparam, mine);
+    const uint64_t nw = b < nblk ? (uint64_t)((bits + 31) >> 5) : 0;
     // exclusive scan of the word counts over the CTA
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint64_t incl = nw;
