@@ -91,14 +91,19 @@ __global__ void bf16_unpack_flat(const uint16_t *in, float *out, int64_t n)
 // nsteps heat7 steps in place on d_u.  Pairs of steps in one launch where one
 // pair takes less time than two steps, that is on all grids but small ones
 // (us per pair and per two steps: 512^3 218 and 340, 256^3 39 and 53; at
-// 192^3 and below single steps are faster, 28 and 19).  The launches alternate
-// between the two fields, so their number is made even by running up to three
-// steps singly (10 steps of 512^3: 4 pairs and 2 steps, no copy back).
+// 192^3 and below single steps are faster, 28 and 19) and those of 4 rows,
+// where 14-row tiles are mostly padding (4 x 2048 planes, 64 Mi points: 306 and
+// 202; 8 rows 162 and 189).  The launches alternate between the two fields, so
+// their number is made even by running up to three steps singly (10 steps of
+// 512^3: 4 pairs and 2 steps, no copy back).  Many rows of up to a quarter of
+// a tile take the copy instead, which costs them less (two steps, two launches
+// and a pair with the copy: 4096 x 1024 x 4 983 and 764, 64 x 8192 x 32 153 and
+// 130; 16384 x 32 x 32, where a pair gains less, 222 and 253).
 ooc_status heat7_run(float *d_u, float *d_tmp, int64_t nx, int64_t ny, int64_t nz, float r, int64_t nsteps,
                      cudaStream_t st)
 {
-    int64_t pairs = heat7_small(nx, ny, nz) ? 0 : nsteps / 2;
-    if (pairs > 0 && ((nsteps - pairs) & 1))
+    int64_t pairs = heat7_small(nx, ny, nz) || ny <= 4 ? 0 : nsteps / 2;
+    if (pairs > 0 && ((nsteps - pairs) & 1) && (nx > 32 || ny < 64))
         --pairs;
     float *a = d_u, *b = d_tmp;
     for (int64_t s = 0, j = 0; s < nsteps; ++j) {

@@ -85,6 +85,19 @@ def test_plan_pairs(ooc, shape, kind):
     assert np.array_equal(got.view(np.uint32), ref.view(np.uint32))
 
 
+@pytest.mark.parametrize("shape", [(2048, 4, 2048), (2048, 8, 1024), (4096, 1024, 4), (8192, 60, 32), (8192, 64, 32),
+                                   (640, 512, 36)])
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 6])
+def test_few_rows_or_columns(ooc, shape, n):
+    # 4 rows run single steps; many rows of at most 32 points an odd number
+    # of launches and a copy
+    assert np.prod(shape) > SMALL
+    u = torch.from_numpy(values("normal", shape)).cuda()
+    v = u.clone()
+    ooc.ooc_heat7_steps(v, torch.empty_like(v), n)
+    assert same(v, singly(ooc, u, n))
+
+
 def test_incore_pairs_match_fp64(ooc):
     shape = (16, 768, 1024)
     assert np.prod(shape) > SMALL
