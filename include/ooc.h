@@ -241,7 +241,15 @@ ooc_status ooc_bf16_unpack(const uint16_t *d_in, float *d_out, int64_t n, void *
  * wave25: from (d_p, d_pprev) = (p^t, p^{t-1}) to (p^{t+n}, p^{t+n-1}),
  * adding h_w[t + s] (host array, may be NULL) at (sx, sy, sz) in step s
  * (0-based); pass sx < 0 for no source.  Device buffers 16-byte aligned and
- * distinct; OOC_E_INVALID otherwise. */
+ * distinct; OOC_E_INVALID otherwise.
+ * ooc_heat7_steps runs one step per kernel launch, or, where that is faster
+ * (most grids of more than 11 Mi points), two: temporal blocking inside the
+ * kernel (Section III), the intermediate level in shared memory and registers,
+ * so that HBM carries one read and one write of the field per two steps.
+ * Results do not depend on the choice.  The two-step kernel waits for its
+ * copies with a limit: such a call can return OOC_OK and still leave planes
+ * unwritten, which ooc_take_device_fault reports (read it after synchronising
+ * the stream). */
 ooc_status ooc_heat7_steps(float *d_u, float *d_tmp, int64_t nx, int64_t ny, int64_t nz, double r,
                            int64_t nsteps, void *stream);
 ooc_status ooc_wave25_steps(float *d_p, float *d_pprev, const float *d_kappa, int64_t nx, int64_t ny,
@@ -272,12 +280,8 @@ ooc_status ooc_wave25_steps_f64(double *d_p, double *d_pprev, const double *d_ka
                                 int64_t nz, int64_t sx, int64_t sy, int64_t sz, const double *h_w, int64_t t,
                                 int64_t nsteps, void *stream);
 
-/* The nsteps heat7 steps of ooc_heat7_steps with each pair of steps in one
- * kernel launch (temporal blocking inside the kernel, Section III: the
- * intermediate level stays in shared memory and registers, so HBM carries
- * one read and one write of the field per two steps).  An odd last step
- * runs alone.  Same arguments and errors as ooc_heat7_steps; results are
- * bit-identical to it. */
+/* The same call as ooc_heat7_steps, which pairs steps itself; kept for
+ * programs that ask for pairs by name. */
 ooc_status ooc_heat7_steps_fused(float *d_u, float *d_tmp, int64_t nx, int64_t ny, int64_t nz, double r,
                                  int64_t nsteps, void *stream);
 
@@ -289,7 +293,7 @@ ooc_status ooc_heat7_steps_fused(float *d_u, float *d_tmp, int64_t nx, int64_t n
  * rest of its output; 2 if ooc_gather or ooc_scatter_add met an
  * index outside its field and skipped it.  ooc_step checks the first
  * itself and returns OOC_E_TIMEOUT; callers of the in-core entry points
- * read it after synchronising their stream.  Kernels never trap, spin
+ * (ooc_heat7_steps among them) read it after synchronising their stream.  Kernels never trap, spin
  * without bound or access memory through an unchecked index. */
 ooc_status ooc_take_device_fault(int *fault);
 

@@ -368,6 +368,8 @@ def ooc_bf16_unpack(d_in, d_out=None, stream=None):
 
 
 def ooc_heat7_steps(d_u, d_tmp, nsteps, r=1.0 / 6.0, stream=None):
+    """heat7 in place on d_u; on large grids two steps per launch, whose
+    bounded waits ooc_take_device_fault reports after a synchronise."""
     nz, ny, nx = d_u.shape
     _check(lib().ooc_heat7_steps(_dev(d_u, _f32(), "d_u", ndim=3), _dev(d_tmp, _f32(), "d_tmp", numel=d_u.numel()),
                                  nx, ny, nz, float(r), int(nsteps), _stream(stream)), "ooc_heat7_steps")
@@ -384,7 +386,7 @@ def ooc_heat7_steps_f64(d_u, d_tmp, nsteps, r=1.0 / 6.0, stream=None):
 
 
 def ooc_heat7_steps_fused(d_u, d_tmp, nsteps, r=1.0 / 6.0, stream=None):
-    """ooc_heat7_steps with each pair of steps in one launch (bit-identical)."""
+    """The same call as ooc_heat7_steps, which pairs steps itself."""
     nz, ny, nx = d_u.shape
     _check(lib().ooc_heat7_steps_fused(_dev(d_u, _f32(), "d_u", ndim=3),
                                        _dev(d_tmp, _f32(), "d_tmp", numel=d_u.numel()), nx, ny, nz, float(r),
