@@ -145,10 +145,6 @@ cudaError_t launch_wave25_f64(DConstRing p, DRing pprev_out, DConstRing kappa, i
 cudaError_t launch_wave25(ConstRing p, Ring pprev_out, ConstRing kappa, int64_t nx, int64_t ny, int64_t nz,
                           int64_t z0, int64_t z1, int64_t sx, int64_t sy, int64_t sz, float w, cudaStream_t st,
                           WaveSrcTable tab = WaveSrcTable{}, bool pdl = false);
-// Same step with p_prev read from `pprev` and p' written to `pnew` (may alias).
-cudaError_t launch_wave25_to(ConstRing p, ConstRing pprev, Ring pnew, ConstRing kappa, int64_t nx, int64_t ny,
-                             int64_t nz, int64_t z0, int64_t z1, int64_t sx, int64_t sy, int64_t sz, float w,
-                             cudaStream_t st, WaveSrcTable tab = WaveSrcTable{}, bool pdl = false);
 // Reads and clears the device word that a stencil kernel sets when one of
 // its bounded waits gives up (nonzero: that launch left planes unwritten).
 cudaError_t take_stencil_fault(unsigned *fault);

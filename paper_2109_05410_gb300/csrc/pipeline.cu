@@ -37,7 +37,7 @@ using namespace ooc;
 
 namespace {
 
-constexpr int kEv = 4;  // event ring depth (waits look back at most 2 slabs)
+constexpr int kEv = 4;  // event ring depth (waits look back at most 3 slabs)
 constexpr int64_t kSrcTable = 16384;  // source amplitudes kept on the device (graph replay)
 constexpr size_t kGuard = 256;        // guard bytes after each arena region (debug_checks)
 constexpr int kMaxGuards = 32;

@@ -901,17 +901,6 @@ cudaError_t run_wave25(bool pdl, const float *p, const float *pprev, float *pout
 }
 }  // namespace
 
-cudaError_t launch_wave25_to(ConstRing p, ConstRing pprev, Ring pnew, ConstRing kappa, int64_t nx, int64_t ny,
-                             int64_t nz, int64_t z0, int64_t z1, int64_t sx, int64_t sy, int64_t sz, float w,
-                             cudaStream_t st, WaveSrcTable tab, bool pdl)
-{
-    if (p.nslot != pnew.nslot || p.zbase != pnew.zbase || p.nslot != kappa.nslot || p.zbase != kappa.zbase ||
-        p.nslot != pprev.nslot || p.zbase != pprev.zbase)
-        return cudaErrorInvalidValue;
-    return run_wave25<0>(pdl, p.base, pprev.base, pnew.base, kappa.base, p.nslot, p.zbase, nx, ny, nz, z0, z1, sx, sy,
-                         sz, w, nullptr, tab, nullptr, nullptr, nullptr, false, st);
-}
-
 cudaError_t launch_wave25_grad(const float *p, const float *mu, double *g, int64_t nx, int64_t ny, int64_t nz,
                                cudaStream_t st)
 {
@@ -939,8 +928,10 @@ cudaError_t launch_wave25(ConstRing p, Ring pprev_out, ConstRing kappa, int64_t 
                           int64_t z0, int64_t z1, int64_t sx, int64_t sy, int64_t sz, float w, cudaStream_t st,
                           WaveSrcTable tab, bool pdl)
 {
-    return launch_wave25_to(p, ConstRing{pprev_out.base, pprev_out.nslot, pprev_out.zbase}, pprev_out, kappa, nx, ny,
-                            nz, z0, z1, sx, sy, sz, w, st, tab, pdl);
+    if (p.nslot != pprev_out.nslot || p.zbase != pprev_out.zbase || p.nslot != kappa.nslot || p.zbase != kappa.zbase)
+        return cudaErrorInvalidValue;
+    return run_wave25<0>(pdl, p.base, pprev_out.base, pprev_out.base, kappa.base, p.nslot, p.zbase, nx, ny, nz, z0, z1,
+                         sx, sy, sz, w, nullptr, tab, nullptr, nullptr, nullptr, false, st);
 }
 
 cudaError_t launch_add_time(int64_t *t, int64_t n, cudaStream_t st)
