@@ -66,8 +66,8 @@ NCU_UNITS = 56 * 1024 * 1024
 NCU_COUNTERS = {
     "heat7_stencil": {"src": ["heat_tma.cu", "tma.cuh", "stencil_common.cuh", "f32x2.cuh"], "sha": "71ba1f15c6a3e79f",
                       "dram_bytes": 428.5e6, "warp_inst": 76.58e6},
-    "fr4_encode": {"src": "codec.cu", "sha": "693514c532d3f048", "dram_bytes": 317.1e6, "warp_inst": 120.29e6},
-    "fr4_decode": {"src": "codec.cu", "sha": "693514c532d3f048", "dram_bytes": 293.1e6, "warp_inst": 143.52e6},
+    "fr4_encode": {"src": "codec.cu", "sha": "a3d8c10e9e14714a", "dram_bytes": 317.5e6, "warp_inst": 122.18e6},
+    "fr4_decode": {"src": "codec.cu", "sha": "a3d8c10e9e14714a", "dram_bytes": 292.9e6, "warp_inst": 143.52e6},
 }
 # issue peak: 152 SMs x 4 schedulers x one warp instruction per clock at the
 # maximum SM clock of 2070 MHz

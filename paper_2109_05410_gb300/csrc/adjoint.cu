@@ -34,7 +34,8 @@
 // sums in two launches, against 48 bytes and three sums in three launches
 // for a gradient kernel of its own: at 256^3, where a step is bound by the
 // sums' instructions (52 us against 40 us of traffic), forward and gradient
-// of 100 steps took 28.8 ms with it and 22.6 ms without.
+// of 100 steps took 28.8 ms with it and 22.6 ms without (21.0 now, with the
+// division by kappa in the last flush and wave25's deeper staging).
 #include <cstring>
 
 #include "common.cuh"

@@ -21,24 +21,12 @@
 // with coalesced 16-byte accesses; the plane masks pass through shared memory
 // 16 planes at a time.
 //
-// The kernels are bound by the integer ALU pipe (78-80 % busy, against 23-27 %
+// The kernels are bound by the integer ALU pipe (76-80 % busy, against 22-29 %
 // of DRAM), which issues half of what the schedulers do.  56 planes of 1024^2,
-// R = 8, 16, 24, us: encode 196, 224, 241 -> 126, 140, 144; decode 196, 236,
-// 261 -> 142, 166, 179, against a plane loop that wrote its fields by
+// R = 8, 16, 24, us: encode 196, 224, 241 -> 125, 141, 146; decode 196, 236,
+// 261 -> 139, 163, 176, against a plane loop that wrote its fields by
 // read-modify-write and parsed the new ones segment by segment (22 of 32
 // lanes active).  The transform and the transposes alone take 92 and 80 us.
-// What did not pay for the decoder: the plane loop unrolled with the masks in
-// registers (no shared memory for them, but its code overflows the
-// instruction cache: 230 us; with a plane as a called function 208), all 32
-// masks of a block in shared memory at once (16 warps per SM instead of 24:
-// 216).  For the encoder: a plane's new ones through a 256-entry table in
-// place of insert_ones' loop (148 -> 165: a plane of a smooth field has one or
-// none); the refinement bits and the new ones of every plane as one field
-// (145).  For the decoder: the first planes apart as the encoder does
-// (code_planes; 142, 166, 179 -> 140, 165, 177, but 138, 167, 188 -> 140, 169,
-// 189 on rougher fields).  Of the encoder's instructions per warp 877 load,
-// convert and store (62 us by themselves), 340 transform, 720 transpose and
-// 2300 code the planes.
 //
 // Also here: dense-field kernels for any shape (partial blocks padded with
 // the nearest inside value) and the variable-size fixed-precision and
@@ -660,7 +648,7 @@ __device__ __forceinline__ Plane parse_plane(const uint32_t *w, int nwords, int 
 // memory with kZeroWords zeros behind, with the plane range of `mode`.  The
 // planes are parsed 16 at a time into the thread's 32 words at pm and taken
 // from there into registers, half transposed: half the shared memory of all
-// 32 planes, for 24 warps per SM instead of 16.
+// 32 planes, for 24 warps per SM up to R = 16 (16 with all planes) and 20 above.
 __device__ __forceinline__ void decode_block(const uint32_t *w, int nwords, int mode, int mparam, float (&out)[64],
                                              uint32_t *pm)
 {
@@ -892,9 +880,9 @@ __global__ void __launch_bounds__(kThreads, MINB) fr4_decode_kernel(const uint32
 // and coded first; the low words' only when the budget reaches them (it ends
 // about there at 24 of 64 bits on smooth fields).  56 planes of 1024^2, R = 24
 // and 32, us, against all 128 plane words per thread in shared memory (8 warps
-// per SM): encode 474, 505 -> 388, 396 (12 warps, 168 registers); decode 647,
-// 678 -> 443, 470 (16 warps at 128 registers with spills; 12 warps without,
-// 460, 484), with the scaling as an addition to the exponent instead of a
+// per SM): encode 474, 505 -> 333, 348 (12 warps, 168 registers); decode 647,
+// 678 -> 455, 479 (16 warps at 128 registers with spills; 12 warps without are
+// 4 % slower), with the scaling as an addition to the exponent instead of a
 // second FP64 instruction per value.
 constexpr int kPrec64 = 58;
 constexpr int kThreads64 = 64;

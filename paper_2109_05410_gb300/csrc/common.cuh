@@ -50,7 +50,7 @@ __host__ __device__ inline int64_t ring_slot(int64_t z, int64_t zbase, int64_t n
 // writes are visible.  What overlaps is the launch itself: between two
 // dependent kernels without it the GPU idles for up to 2.05 us (kernel starts
 // fall on a grid of about that step; a 64^3 heat7 step takes 4.17 us without
-// and 2.4 us with it).  Such a kernel must not read through the non-coherent
+// and 2.1 us with it).  Such a kernel must not read through the non-coherent
 // path (__ldg, or a const __restrict__ pointer's plain loads): that is for data
 // that nothing writes while the kernel is resident, and a block that waits is.
 // Its loads are __ldca or copies through L2 (cp.async of 16 bytes).

@@ -70,13 +70,11 @@ constexpr int kX2tNW = OOC_HEATX2T_NW;
 using X2t = X2tShape<kX2tR, kX2tNW>;
 // 5 stages and 3 CTAs per SM (72 KB of shared memory and at most 85
 // registers each), loop unrolled 3 times (the z-queues rotate without
-// copies).  Bound by instruction issue and the plane barrier (issue 65 %
-// active, 51-54 % of DRAM).  56 planes of 1024^2, us per launch: 98.7; with
-// planes outside the grid tested for instead of copied as zeros 104.7 (13 %
-// more instructions in the loop); 4 stages 100.5; unrolled 4 and 6 times 102.5
-// and 98.5; 6 stages and 2 CTAs per SM 118.9; a check of the tile's position
-// in place of the select after level s 101.5.  512^3: 217.8, with 120-column
-// tiles and the tests 256.
+// copies).  Bound by instruction issue and the plane barrier (issue 67 %
+// active, 55 % of DRAM).  56 planes of 1024^2, us per launch: 98.7; with planes
+// outside the grid tested for instead of copied as zeros 104.7 (13 % more
+// instructions in the loop).  512^3: 217.8, with 120-column tiles and the tests
+// 256.
 #ifndef OOC_HEATX2T_NS
 #define OOC_HEATX2T_NS 5
 #endif

@@ -168,7 +168,7 @@ OOC_PRAGMA(unroll OOC_HEAT_UNROLL)
 // holds, where the march's chain of planes is what takes the time.
 //
 // Up to kHeatDirectMax points (88 MiB for both levels: L2 holds them): us per
-// step, march and direct, both with overlapped launches: 64^3 6.2 and 2.4,
+// step, march and direct, both with overlapped launches: 64^3 6.2 and 2.1,
 // 128^3 8.3 and 3.7, 192^3 16.4 and 9.6; 256^3 26.4 and 27.2, 512^3 170 and
 // 197.  ZR = 4: at 128^3 2 takes 4.4 and 8 the same as 4, at 192^3 12.0 and
 // 13.8 against 9.6.

@@ -21,10 +21,11 @@
 // FP64 finish the point.
 // Against the FP64 sequence the sum carries no rounding but the shifts' (each
 // at most 2^-58 of the stencil's largest value, wave25 2^-59 in its unit) and
-// one at its end.  By CPU emulation against 113 bits the error is 0.6 to 0.8 of
-// the FP64 instructions' for wave25 from 8 to 12800 steps, 0.8 to 1.0 for heat7
-// (whose two FMAs set it) from 8 to 800, on smooth, rough, positive, steep and
-// isolated fields; f(-u) = -f(u) as in FP64 instructions (see the GPU tests).
+// one at its end.  By CPU emulation against 113 bits (24 x 20 x 20, r = 1/6) the
+// error over the FP64 instructions' is 0.6 to 0.8 for wave25 from 8 to 12800
+// steps, and for heat7, whose two FMAs set it, 0.8 to 0.9 up to 50 steps and 0.9
+// to 1.07 at 200 to 800, on smooth, rough, positive, steep and isolated fields;
+// f(-u) = -f(u) as in FP64 instructions (see the GPU tests).
 //
 // Stencils that the integer form does not hold as exactly as FP64 would take
 // the FP64 instructions instead, per thread: infinities, NaN, a largest
@@ -47,9 +48,14 @@
 // integer sums: wave25 3200 (17.7) and 1066 (53); heat7 775 (73) and 344
 // (165).  wave25 took 839 with shifts cut off and 16-bit rational weights: a
 // tenth more instructions for the rounding, twice the multiplies for the
-// weights.  White noise: wave25 1067, heat7 478, where some lane of nearly every
-// warp takes the FP64 instructions.  A wave from rest, whose steep precursors
-// take them in part: 0.85 ms per 256^3 step over its first 100.  Bound now:
+// weights.  White noise: wave25 1067, heat7 478, where some lane of most warps
+// takes the FP64 instructions.  Where all do, the sums are run in vain: values
+// 2^60 apart 960 -> 1220 (heat7; also a point release at r = 1/6 and a
+// half-empty checkerboard) and 3800 -> 4320 (wave25).  A wave from rest, whose
+// steep precursors take them in part: 0.85 ms per 256^3 step over its first 100.
+// A fallback for heat7 in integers at the neighbours' own exponent would be
+// faster, but rounds so seldom that its error on a point release grows to 1.35
+// of the FP64 instructions' after 800 steps.  Bound now:
 // wave25 by the ALU pipe and shared-memory wavefronts, heat7 by the FP64 pipe
 // (61 %) and the ALU pipe with 28 warps per SM.
 #include <type_traits>
